@@ -97,7 +97,12 @@ AIR_API air_status air_plan_destroy(air_plan *plan);
  * air_plan_tune overrides the choice (AIR_ERR_INVALID_ARG outside the
  * allowed values: bwd_view_parts in 1..*bwd_view_parts_max); results agree
  * to rounding whatever the configuration (the summation order over views
- * depends on the split).  Either pointer of air_plan_config may be NULL. */
+ * depends on the split).  Either pointer of air_plan_config may be NULL.
+ * Full scans whose views are taken into one another by at least four of the
+ * eight symmetries of the pixel grid (n_views even and beta0 a multiple of
+ * half the view pitch, or n_views a multiple of 4; n >= 64) run the projector
+ * pair over orbits of symmetric rays: their projector has one tile shape, and
+ * bwd_view_parts counts images, eight for each split of the backprojector. */
 AIR_API air_status air_plan_tune(air_plan *plan, int fwd_views_per_block, int bwd_view_parts);
 AIR_API air_status air_plan_config(const air_plan *plan, int *fwd_views_per_block, int *bwd_view_parts,
                                    int *bwd_view_parts_max);
@@ -192,7 +197,10 @@ AIR_API air_status air_shrink(const air_plan *plan, const float *X, float *b, fl
  * Y: n_views*n_bins (input), X: n*n (output only).  resid: device, n_outer
  * doubles, may be NULL: ||W X - d||_2 after each outer step.  lambda >= 0,
  * mu > 0, n_outer >= 0, n_cg >= 0.  CG dot products and the residual norms
- * are accumulated in FP64 on the device; no host synchronisation inside. */
+ * are accumulated in FP64 on the device; no host synchronisation inside.
+ * With resid the solve runs the general projector pair whatever the scan's
+ * symmetries (see air_plan_tune), so that the history keeps one summation
+ * order; X then differs from a call without resid by rounding. */
 AIR_API air_status air_solve(const air_plan *plan, const float *Y, float lambda, float mu,
                      int n_outer, int n_cg, float *X, double *resid, air_stream stream);
 

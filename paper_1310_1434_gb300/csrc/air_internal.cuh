@@ -40,6 +40,10 @@ enum Op : int {
     OP_PROX,       // x = W^T S_tau(W q)        (framelet proximal step)
     OP_FBP,        // ext_out = fan-beam FBP weighted backprojection of zc
     OP_RESTART,    // CG restart of an outer step: r = rhs0 (arg -1) or r += mu (g_new - g_old); p = r; rho
+    OP_ORB_PACK,   // frames of src for the orbit projector   (in place of OP_TRANSPOSE; arg = FwdSrc)
+    OP_ORB_FWD,    // z = A src by orbits                      (in place of OP_FWD; arg = FwdSrc)
+    OP_ORB_ZPACK,  // samples of the orbits' rays side by side  (before OP_ORB_BWD; arg = BwdMode)
+    OP_ORB_BWD,    // per-frame parts of A^T zc by orbits      (in place of OP_BWD; OP_BWD_FIN sums them)
     OP_COUNT
 };
 
@@ -105,6 +109,30 @@ __host__ __device__ inline unsigned vt_pack(int j0, int j1, int o, bool neg, boo
            (mixed ? VT_MIXED : 0u);
 }
 
+// A symmetry of the square as a code: exchange x and y (ORB_T), then turn the
+// x axis (ORB_FX) and the y axis (ORB_FY).
+enum OrbCode : int { ORB_T = 1, ORB_FX = 2, ORB_FY = 4 };
+// One segment of the orbit tables (orbit.h): neighbouring rays of one view
+// that share a frame, as canonical rays by ascending angle.
+struct __align__(16) OrbSeg {
+    float sx, sy;        // canonical source position, pixels from the image corner
+    float cx, cy;        // canonical direction of the view's central ray
+    float ioff;          // ray index of the central direction, less OrbitTables::eps
+    int ray0, cnt;       // canonical rays [ray0, ray0 + cnt)
+    int cls;             // class of its frames
+    int down;            // bit f: frame f's sinogram index falls along the segment
+    int zoff[8];         // sinogram index of ray 0 in frame f of the class, -1: none
+    int pad0;            // its place in the padded arrays, ORB_CAND empty rays after it
+    int pad[2];
+};
+constexpr int BWD_T = 32;         // side of a backprojector pixel tile
+constexpr int ORB_MIN_N = 64;     // smallest image side the orbit kernels take
+constexpr int ORB_VIEWS = 8;      // base views whose projector warps follow one another
+constexpr int ORB_RAYS = 96;      // most rays of a segment in a backprojector tile
+constexpr int ORB_CAND = 8;       // most rays of a segment that can meet two pixels of a column
+constexpr int ORB_PAD = 2;        // zero rows below and above a stack column
+__host__ __device__ inline int orb_ld(int n) { return n + 2 * ORB_PAD; }
+
 // Everything a tile function needs to know about one slice.  Plain data:
 // copied by value into kernel parameters or into a device task table.
 struct SliceDesc {
@@ -136,6 +164,22 @@ struct SliceDesc {
     float *bwd_part;                   // bwd_parts * n*n: the backprojector's per-view-part sums
     int bwd_parts;                     // S: views split over S blocks per pixel tile (tuned)
     int fwd_vpb;                       // projector tile: views per block (1, 2, 4, 8; tuned)
+    // orbit tables (orbit.h; orb = frames per orbit, 0: the scan has too few symmetries)
+    int orb;
+    int orb_splits;                    // segments split over this many blocks per pixel tile; 8 parts each (tuned)
+    int orb_ks;                        // projector: columns split over this many warps per ray (1, 2, 4, 8)
+    int orb_ntask;                     // projector warps
+    int orb_frame[8];                  // symmetry codes, plane-major
+    const OrbSeg *orb_seg;
+    const RayFx *orb_ray;
+    const uint2 *orb_info;             // per ray {walk word, segment}
+    const unsigned *orb_task;
+    const int *orb_tile0;              // [2][tiles + 1]
+    int orb_nseg, orb_npad;            // segments; rays of the padded arrays
+    const uint2 *orb_ent;              // {segment | rays << 17 | candidates << 24, first ray in the padded arrays}
+    const uint4 *orb_bray;             // padded rays {L0, |M|, 0}
+    float4 *orb_z;                     // [planes of a ray][padded rays]: c times the samples of a ray's orbit
+    float4 *orb_stack;                 // [2 planes][n][n + 4]: the projector's input in four frames a plane
     float *b, *b2;                     // 9*n*n each (Bregman variable, double-buffered)
     float *z, *zc;                     // V*nb
     const float *y;                    // V*nb measured sinogram
@@ -166,11 +210,26 @@ __host__ __device__ inline int tiles_fwd(const SliceDesc &s) {
 }
 __host__ __device__ inline int tiles_ramp(const SliceDesc &s) { return s.V; }
 // backprojector tile: 32 x 32 pixels x one of bwd_parts view parts
-constexpr int BWD_T = 32;
 __host__ __device__ inline int tiles_bwd_xy(const SliceDesc &s) {
     return ((s.n + BWD_T - 1) / BWD_T) * ((s.n + BWD_T - 1) / BWD_T);
 }
 __host__ __device__ inline int tiles_bwd(const SliceDesc &s) { return tiles_bwd_xy(s) * s.bwd_parts; }
+// orbit projector: warps of rays x column parts.  Planes a ray reads: both
+// with 8 frames, the plane of its class with 4.
+__host__ __device__ inline int orb_planes(const SliceDesc &s) { return s.orb == 8 ? 2 : 1; }
+__host__ __device__ inline int tiles_orb_fwd(const SliceDesc &s) {
+    const int w = AIR_THREADS / 32 / s.orb_ks;
+    return (s.orb_ntask + w - 1) / w;
+}
+// sample packing: ORB_ZPACK rays of a segment
+constexpr int ORB_ZPACK = AIR_THREADS;
+__host__ __device__ inline int orb_zchunks(const SliceDesc &s) { return (s.nb + ORB_CAND + ORB_ZPACK - 1) / ORB_ZPACK; }
+// orbit backprojector: classes x splits x pixel tiles
+__host__ __device__ inline int tiles_orb_bwd(const SliceDesc &s) {
+    return tiles_bwd_xy(s) * s.orb_splits * (s.orb == 8 ? 1 : 2);
+}
+// images OP_BWD_FIN sums: the view parts, or eight frames for each split
+__host__ __device__ inline int bwd_images(const SliceDesc &s) { return s.orb ? 8 * s.orb_splits : s.bwd_parts; }
 constexpr int VEC_PER_TILE = AIR_THREADS * 4;   // elementwise ops: 4 per thread
 __host__ __device__ inline int tiles_vec(const SliceDesc &s) {
     return (s.n * s.n + VEC_PER_TILE - 1) / VEC_PER_TILE;
@@ -190,6 +249,10 @@ __host__ __device__ inline int tiles_of(const SliceDesc &s, int op) {
     case OP_BWD: return tiles_bwd(s);
     case OP_CG_A: case OP_CG_B: case OP_ZERO: case OP_BWD_FIN: case OP_AXPY: case OP_RESTART: return tiles_vec(s);
     case OP_TRANSPOSE: return tiles_tr(s);
+    case OP_ORB_PACK: return 2 * tiles_tr(s);
+    case OP_ORB_FWD: return tiles_orb_fwd(s);
+    case OP_ORB_ZPACK: return s.orb_nseg * orb_zchunks(s);
+    case OP_ORB_BWD: return tiles_orb_bwd(s);
     case OP_SHRINK: case OP_FRAMELET: case OP_FRAMELET_T: case OP_PROX: case OP_FBP:
         return tiles_shr(s);
     default: return 0;

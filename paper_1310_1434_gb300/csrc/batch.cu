@@ -117,7 +117,7 @@ air_status prepare(int n, air_plan *const *plans, const float *const *Y, const f
         if (tc && !allow_tc)
             return fail(AIR_ERR_INVALID_ARG, "the persistent batch runs the FP32 filter; use FP32 plans");
         B->slices[i] = solve_desc(plans[i], Y[i], lambda[i], mu[i], X[i], nullptr);
-        B->progs[i] = solve_program(n_outer[i], n_cg[i], tc);
+        B->progs[i] = solve_program(n_outer[i], n_cg[i], tc, plans[i]->desc.orb != 0);
         B->nphases = std::max(B->nphases, B->progs[i].size());
     }
     int dev = 0;
@@ -423,8 +423,11 @@ extern "C" air_status air_solve_batch_persistent(int n, air_plan *const *plans, 
     air_status s = prepare(n, plans, Y, lambda, mu, n_outer, n_cg, X, st, false, &B);
     if (s != AIR_OK) return s;
     size_t smem = 0;
-    for (int i = 0; i < n; ++i)
-        for (int op : {OP_RAMP, OP_SHRINK, OP_TRANSPOSE, OP_BWD}) smem = std::max(smem, tile_smem(B.slices[i], op));
+    bool orb = false;
+    for (int i = 0; i < n; ++i) {
+        for (const Phase &ph : B.progs[i]) smem = std::max(smem, tile_smem(B.slices[i], ph.op));
+        orb |= B.slices[i].orb != 0;
+    }
     std::vector<Phase> prog(n * B.nphases, Phase{OP_NOP, 0});
     for (int i = 0; i < n; ++i)
         std::memcpy(&prog[i * B.nphases], B.progs[i].data(), B.progs[i].size() * sizeof(Phase));
@@ -432,7 +435,7 @@ extern "C" air_status air_solve_batch_persistent(int n, air_plan *const *plans, 
     BatchGraph &G = g_persistent;
     if (G.key != B.key || !G.exec) {
         release(G);
-        const int grid = persistent_grid(smem);
+        const int grid = persistent_grid(smem, orb);
         if (grid <= 0) return fail(AIR_ERR_CUDA, "batch set-up: no co-resident grid for the persistent kernel");
         // per phase: prefix sums of the slices' tile counts, and the phase's
         // first ticket (earlier phases' tiles plus one closing ticket per block)
@@ -481,7 +484,7 @@ extern "C" air_status air_solve_batch_persistent(int n, air_plan *const *plans, 
         }
         cudaError_t le = cudaMemsetAsync(G.ctl, 0, sizeof(BatchCtl), G.cap);
         if (le == cudaSuccess)
-            le = launch_persistent(d_slices, n, d_prog, (int)B.nphases, d_tb, d_pb, G.ctl, grid, smem, G.cap);
+            le = launch_persistent(d_slices, n, d_prog, (int)B.nphases, d_tb, d_pb, G.ctl, grid, smem, orb, G.cap);
         if ((s = end_capture(G, G.cap, le)) != AIR_OK) return s;
         G.key = B.key;
     }

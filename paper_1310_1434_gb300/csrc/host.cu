@@ -11,6 +11,7 @@
 
 #include "host_common.h"
 #include "launch.h"
+#include "orbit.h"
 #include "ramp_tc.h"
 
 using namespace air;
@@ -83,17 +84,47 @@ namespace air {
 // Backprojector view parts of a slice: enough (pixel tile, part) blocks for
 // about 12 per SM (2.4 waves at 5 resident blocks), at most one part per
 // view.  The autotuner starts from this and tries up to twice as many.
+static int sm_count();
 int choose_bwd_parts(const SliceDesc &s) {
-    int sms = 148, dev = 0;
-    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaGetLastError();
+    const int sms = sm_count();
     const int txy = tiles_bwd_xy(s), target = 2 * 6 * sms;
     const int S = (target + txy - 1) / txy;
     return S < 1 ? 1 : (S > s.V ? s.V : S);
 }
 
+cudaError_t launch_backprojection(const SliceDesc &s, int mode, cudaStream_t st) {
+    cudaError_t e = s.orb ? launch_op(OP_ORB_ZPACK, s, mode, st) : cudaSuccess;
+    if (e == cudaSuccess) e = launch_op(s.orb ? OP_ORB_BWD : OP_BWD, s, mode, st);
+    if (e == cudaSuccess && (mode != BWD_PLAIN || bwd_images(s) > 1)) e = launch_op(OP_BWD_FIN, s, mode, st);
+    return e;
+}
+
+// Most splits of the orbit backprojector's segments: about four waves of
+// three blocks per SM, at most 16 (each split adds eight images to the sum).
+static int orb_splits_max(int n, int nf, int sms) {
+    const int tiles = ((n + BWD_T - 1) / BWD_T) * ((n + BWD_T - 1) / BWD_T) * (nf == 8 ? 1 : 2);
+    const int S = (4 * 3 * sms + tiles - 1) / tiles;
+    return S < 1 ? 1 : (S > 16 ? 16 : S);
+}
+
+// Column parts of the orbit projector: as few as give the device about 24
+// warps per SM (each part pays for the warp's set-up and the sum).
+static int choose_orb_ks(int warps, int sms) {
+    int ks = 1;
+    while (ks < 8 && (long long)warps * ks < 2400ll * sms) ks *= 2;
+    return ks;
+}
+
+static int sm_count() {
+    int sms = 148, dev = 0;
+    if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaGetLastError();
+    return sms;
+}
+
 // Device bytes a plan of this geometry will hold (the pieces of plan_build
-// and, for BF16X3, the tensor-core filter buffers), to within alignment.
+// and, for BF16X3, the tensor-core filter buffers), to within alignment and,
+// for scans with orbit tables, the number of their segments.
 size_t plan_bytes_estimate(const air_geometry &g) {
     SliceDesc s{};
     s.n = g.n;
@@ -101,8 +132,14 @@ size_t plan_bytes_estimate(const air_geometry &g) {
     s.nb = g.n_bins;
     const size_t nn = (size_t)g.n * g.n, rays = (size_t)g.n_views * g.n_bins;
     // the part buffer holds the autotuner's largest split, as plan_build sizes it
-    const size_t parts = (size_t)std::min(g.n_views, 2 * choose_bwd_parts(s));
-    size_t b = rays * (sizeof(RayFx) + 4) + (size_t)g.n_views * tiles_bwd_xy(s) * 4 + (size_t)g.n_bins * 4;
+    size_t parts = (size_t)std::min(g.n_views, 2 * choose_bwd_parts(s)), orbit = 0;
+    if (const int nf = orbit_frames(g); nf) {
+        parts = std::max(parts, (size_t)8 * orb_splits_max(g.n, nf, sm_count()));
+        const size_t segs = 2 * ((size_t)g.n_views / nf + 2);
+        orbit = nn * 32 + (size_t)g.n * 128 + (rays / nf + segs * ORB_CAND) * (sizeof(RayFx) + 8 + 1 + 16 + 4 * nf) + segs * sizeof(OrbSeg) +
+                (size_t)tiles_bwd_xy(s) * (segs * 6 + 8);
+    }
+    size_t b = orbit + rays * (sizeof(RayFx) + 4) + (size_t)g.n_views * tiles_bwd_xy(s) * 4 + (size_t)g.n_bins * 4;
     b += nn * 4 * (7 + parts + 18 + 1);          // x r p q rhs0 g g', parts, b b2, xbuf
     b += (size_t)g.n * (g.n + 1) * 8 * 2;        // xp xt (pairs)
     b += (size_t)g.n_views * 8 + (size_t)g.n_bins * 8;   // FBP tables
@@ -187,8 +224,11 @@ struct TuneKey {
         return std::memcmp(this, &o, sizeof(TuneKey)) < 0;
     }
 };
+struct Tuned {
+    int vpb, parts, splits;   // general projector and backprojector; orbit backprojector
+};
 std::mutex g_tune_mu;
-std::map<TuneKey, std::pair<int, int>> g_tune_cache;
+std::map<TuneKey, Tuned> g_tune_cache;
 }  // namespace
 
 namespace air {
@@ -208,8 +248,9 @@ air_status autotune(air_plan *P) {
         std::lock_guard<std::mutex> lock(g_tune_mu);
         auto it = g_tune_cache.find(key);
         if (it != g_tune_cache.end()) {
-            s.fwd_vpb = it->second.first;
-            s.bwd_parts = std::min(it->second.second, P->bwd_parts_max);
+            s.fwd_vpb = it->second.vpb;
+            s.bwd_parts = std::min(it->second.parts, P->bwd_parts_max);
+            s.orb_splits = std::min(it->second.splits, std::max(1, P->bwd_parts_max / 8));
             return AIR_OK;
         }
     }
@@ -235,6 +276,7 @@ air_status autotune(air_plan *P) {
     // kept only if it is 2 % faster (within that, grouped batches run the
     // taller tiles a little faster)
     SliceDesc t = s;
+    t.orb = 0;
     t.ext_in = s.x;
     t.ext_out = s.z;
     int best_vpb = 1;
@@ -255,21 +297,34 @@ air_status autotune(air_plan *P) {
     // solver runs them (the parts, then their sum, OP_BWD_FIN, which the CG
     // epilogue needs at any split); the heuristic's choice is tried first
     // and kept unless another is 2 % faster
-    t = s;
     if (e == cudaSuccess) e = cudaMemsetAsync(s.zc, 0, (size_t)s.V * s.nb * 4, st);
-    const int S0 = s.bwd_parts;
+    const int S0 = s.bwd_parts, most = std::min(s.V, 2 * S0);
     int best_S = S0;
     best = 1e30f;
     for (int S : {S0, 1, 2, 3, 4, 6, 8, 12, 16}) {
-        if (S > P->bwd_parts_max || (S == S0 && best < 1e30f)) continue;
+        if (S > most || (S == S0 && best < 1e30f)) continue;
         t.bwd_parts = S;
         const float ms = timed([&] {
-            if (e == cudaSuccess) e = launch_op(OP_BWD, t, BWD_RHS0, st);
-            if (e == cudaSuccess) e = launch_op(OP_BWD_FIN, t, BWD_RHS0, st);
+            if (e == cudaSuccess) e = launch_backprojection(t, BWD_RHS0, st);
         });
         if (ms < best * 0.98f) {
             best = ms;
             best_S = S;
+        }
+    }
+    // orbit backprojector: splits of its segments, the fewest first
+    int best_split = 1;
+    best = 1e30f;
+    t.orb = s.orb;
+    for (int S : {1, 2, 3, 4, 6, 8, 12, 16}) {
+        if (!s.orb || 8 * S > P->bwd_parts_max) continue;
+        t.orb_splits = S;
+        const float ms = timed([&] {
+            if (e == cudaSuccess) e = launch_backprojection(t, BWD_RHS0, st);
+        });
+        if (ms < best * 0.98f) {
+            best = ms;
+            best_split = S;
         }
     }
     if (e0) cudaEventDestroy(e0);
@@ -278,8 +333,9 @@ air_status autotune(air_plan *P) {
     if (e != cudaSuccess) return fail(AIR_ERR_CUDA, std::string("autotuning: ") + cudaGetErrorString(e));
     s.fwd_vpb = best_vpb;
     s.bwd_parts = best_S;
+    s.orb_splits = best_split;
     std::lock_guard<std::mutex> lock(g_tune_mu);
-    g_tune_cache[key] = {best_vpb, best_S};
+    g_tune_cache[key] = {best_vpb, best_S, best_split};
     return AIR_OK;
 }
 }  // namespace air
@@ -296,6 +352,7 @@ struct HostTables {
     std::vector<float> taps, fbw, fbt;
     std::vector<float2> fview;
     float ramp_diag = 0.f, fbp_diag = 0.f;
+    OrbitTables orb;
 };
 
 air_status build_tables(const air_geometry &g, double dg, int ntxy, HostTables &T) {
@@ -417,6 +474,7 @@ air_status build_tables(const air_geometry &g, double dg, int ntxy, HostTables &
         hfbw[k] = (float)std::cos(((double)k - 0.5 * (nb - 1)) * dg);
     }
     T.fbp_diag = (float)fdiag;
+    build_orbits(g, dg, T.orb);
     return AIR_OK;
 }
 
@@ -474,8 +532,23 @@ air_status plan_build(const air_geometry *geom, air_plan *P) {
 
     s.fwd_vpb = 1;
     s.bwd_parts = choose_bwd_parts(s);
-    // the autotuner may pick up to twice the heuristic's view split
-    const int parts_max = std::min(V, 2 * s.bwd_parts);
+    const int ntxy = tiles_bwd_xy(s);
+    std::shared_ptr<const HostTables> T;
+    if (air_status st = geometry_tables(g, dg, ntxy, &T); st != AIR_OK) return st;
+    const OrbitTables &O = T->orb;
+    const int sms = sm_count();
+    // the autotuner may pick up to twice the heuristic's view split; the
+    // orbit backprojector's splits write eight images each
+    int parts_max = std::min(V, 2 * s.bwd_parts);
+    const int splits_max = O.nf ? orb_splits_max(n, O.nf, sms) : 0;
+    parts_max = std::max(parts_max, 8 * splits_max);
+    s.orb = O.nf;
+    s.orb_splits = 1;
+    s.orb_ntask = (int)O.task.size();
+    s.orb_nseg = (int)O.seg.size();
+    s.orb_npad = (int)O.bray.size();
+    s.orb_ks = choose_orb_ks(s.orb_ntask, sms);
+    for (int p = 0; p < 8; ++p) s.orb_frame[p] = O.frame[p];
     // carve one allocation
     struct Piece { void **dst; size_t bytes; };
     float *x, *r, *p, *q, *rhs0, *gg, *gg2, *b, *b2, *z, *zc, *ybuf, *xbuf, *xp, *xt, *bpart;
@@ -485,7 +558,16 @@ air_status plan_build(const air_geometry *geom, air_plan *P) {
     unsigned *vt;
     float2 *fview;
     float *fbw, *fbt;
-    const int ntxy = tiles_bwd_xy(s);
+    OrbSeg *oseg;
+    RayFx *oray;
+    uint2 *oinfo, *oent;
+    uint4 *obray;
+    float4 *oz;
+    unsigned *otask;
+    int *otile0;
+    float4 *ostack;
+    const size_t nstack = O.nf ? (size_t)2 * n * orb_ld(n) : 0;
+    const size_t nz = O.bray.size() * orb_planes(s);
     float *taps;
     CgState *cg;
     double *partial;
@@ -499,6 +581,11 @@ air_status plan_build(const air_geometry *geom, air_plan *P) {
         {(void **)&x, nn * 4}, {(void **)&r, nn * 4}, {(void **)&p, nn * 4}, {(void **)&q, nn * 4},
         {(void **)&rhs0, nn * 4}, {(void **)&gg, nn * 4}, {(void **)&gg2, nn * 4}, {(void **)&b, 9 * nn * 4}, {(void **)&b2, 9 * nn * 4},
         {(void **)&z, rays * 4}, {(void **)&zc, rays * 4}, {(void **)&ybuf, rays * 4}, {(void **)&xbuf, nn * 4},
+        {(void **)&oseg, O.seg.size() * sizeof(OrbSeg)}, {(void **)&oray, O.ray.size() * sizeof(RayFx)},
+        {(void **)&oinfo, O.info.size() * sizeof(uint2)}, {(void **)&oent, O.ent.size() * sizeof(uint2)},
+        {(void **)&otask, O.task.size() * sizeof(unsigned)}, {(void **)&otile0, O.tile0.size() * sizeof(int)},
+        {(void **)&ostack, nstack * sizeof(float4)}, {(void **)&obray, O.bray.size() * sizeof(uint4)},
+        {(void **)&oz, nz * sizeof(float4)},
         {(void **)&cg, sizeof(CgState)}, {(void **)&partial, npart * sizeof(double)}};
     size_t total = 0;
     for (auto &pc : pieces) total = align_up(total, 256) + pc.bytes;
@@ -515,11 +602,6 @@ air_status plan_build(const air_geometry *geom, air_plan *P) {
         off += pc.bytes;
     }
 
-    std::shared_ptr<const HostTables> T;
-    if (air_status st = geometry_tables(g, dg, ntxy, &T); st != AIR_OK) {
-        cudaFree(mem);
-        return st;
-    }
     const std::vector<RayFx> &hray = T->ray;
     const std::vector<unsigned> &hwalk = T->walk;
     const std::vector<unsigned> &hvt = T->vt;
@@ -539,6 +621,17 @@ air_status plan_build(const air_geometry *geom, air_plan *P) {
     if (e == cudaSuccess) e = cudaMemcpy(fview, hfview.data(), V * sizeof(float2), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(fbw, hfbw.data(), nb * sizeof(float), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(fbt, hfbt.data(), nb * sizeof(float), cudaMemcpyHostToDevice);
+    auto upload = [&](void *dst, const void *src, size_t bytes) {
+        if (e == cudaSuccess && bytes) e = cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice);
+    };
+    upload(oseg, O.seg.data(), O.seg.size() * sizeof(OrbSeg));
+    upload(oray, O.ray.data(), O.ray.size() * sizeof(RayFx));
+    upload(oinfo, O.info.data(), O.info.size() * sizeof(uint2));
+    upload(oent, O.ent.data(), O.ent.size() * sizeof(uint2));
+    upload(otask, O.task.data(), O.task.size() * sizeof(unsigned));
+    upload(otile0, O.tile0.data(), O.tile0.size() * sizeof(int));
+    upload(obray, O.bray.data(), O.bray.size() * sizeof(uint4));
+    if (e == cudaSuccess && nstack) e = cudaMemset(ostack, 0, nstack * sizeof(float4));   // the pad rows stay zero
     if (e == cudaSuccess) e = cudaMemset(cg, 0, sizeof(CgState));
     if (e == cudaSuccess) e = cudaMemset(xp, 0, npad * 4);   // the pads stay zero
     if (e == cudaSuccess) e = cudaMemset(xt, 0, npad * 4);
@@ -553,6 +646,15 @@ air_status plan_build(const air_geometry *geom, air_plan *P) {
     s.fbp_w = fbw;
     s.fbp_taps = fbt;
     s.taps = taps;
+    s.orb_seg = oseg;
+    s.orb_ray = oray;
+    s.orb_info = oinfo;
+    s.orb_ent = oent;
+    s.orb_bray = obray;
+    s.orb_z = oz;
+    s.orb_task = otask;
+    s.orb_tile0 = otile0;
+    s.orb_stack = ostack;
     s.x = x; s.r = r; s.p = p; s.q = q; s.rhs0 = rhs0; s.g = gg; s.g2 = gg2; s.b = b; s.b2 = b2; s.xp = xp; s.xt = xt;
     s.bwd_part = bpart;
     s.z = z; s.zc = zc; s.y = ybuf;
@@ -621,6 +723,7 @@ extern "C" air_status air_plan_tune(air_plan *P, int fwd_views_per_block, int bw
         return fail(AIR_ERR_INVALID_ARG, "bwd_view_parts must be in 1.." + std::to_string(P->bwd_parts_max));
     P->desc.fwd_vpb = v;
     P->desc.bwd_parts = bwd_view_parts;
+    P->desc.orb_splits = std::max(1, bwd_view_parts / 8);
     return AIR_OK;
 }
 
@@ -628,7 +731,7 @@ extern "C" air_status air_plan_config(const air_plan *P, int *fwd_views_per_bloc
                                       int *bwd_view_parts_max) {
     if (!P) return fail(AIR_ERR_INVALID_ARG, "plan is NULL");
     if (fwd_views_per_block) *fwd_views_per_block = P->desc.fwd_vpb;
-    if (bwd_view_parts) *bwd_view_parts = P->desc.bwd_parts;
+    if (bwd_view_parts) *bwd_view_parts = bwd_images(P->desc);
     if (bwd_view_parts_max) *bwd_view_parts_max = P->bwd_parts_max;
     return AIR_OK;
 }
@@ -689,8 +792,8 @@ extern "C" air_status air_project(const air_plan *P, const float *X, float *Y, a
     SliceDesc s = P->desc;
     s.ext_in = X;
     s.ext_out = Y;
-    CUDA_TRY(launch_op(OP_TRANSPOSE, s, SRC_EXT, (cudaStream_t)stream));
-    CUDA_TRY(launch_op(OP_FWD, s, SRC_EXT, (cudaStream_t)stream));
+    CUDA_TRY(launch_op(s.orb ? OP_ORB_PACK : OP_TRANSPOSE, s, SRC_EXT, (cudaStream_t)stream));
+    CUDA_TRY(launch_op(s.orb ? OP_ORB_FWD : OP_FWD, s, SRC_EXT, (cudaStream_t)stream));
     return AIR_OK;
 }
 
@@ -710,8 +813,7 @@ extern "C" air_status air_backproject(const air_plan *P, const float *Y, float *
     SliceDesc s = P->desc;
     s.ext_in = Y;
     s.ext_out = X;
-    CUDA_TRY(launch_op(OP_BWD, s, BWD_PLAIN, (cudaStream_t)stream));
-    if (s.bwd_parts > 1) CUDA_TRY(launch_op(OP_BWD_FIN, s, BWD_PLAIN, (cudaStream_t)stream));
+    CUDA_TRY(launch_backprojection(s, BWD_PLAIN, (cudaStream_t)stream));
     return AIR_OK;
 }
 
@@ -726,8 +828,7 @@ extern "C" air_status air_filtered_backproject(const air_plan *P, const float *Y
     SliceDesc s = P->desc;
     s.ext_in = P->desc.zc;
     s.ext_out = X;
-    CUDA_TRY(launch_op(OP_BWD, s, BWD_PLAIN, st));
-    if (s.bwd_parts > 1) CUDA_TRY(launch_op(OP_BWD_FIN, s, BWD_PLAIN, st));
+    CUDA_TRY(launch_backprojection(s, BWD_PLAIN, st));
     return AIR_OK;
 }
 
@@ -778,20 +879,25 @@ namespace air {
 // Each outer step's CG restarts from the residual the previous CG left,
 // corrected for the change of the right-hand side (OP_RESTART): CG keeps
 // r = b - M X, and b changes between outer steps only by mu (g_new - g_old).
-std::vector<Phase> solve_program(int n_outer, int n_cg, bool tc_ramp) {
+std::vector<Phase> solve_program(int n_outer, int n_cg, bool tc_ramp, bool orb) {
     std::vector<Phase> prog;
     const int ramp = tc_ramp ? OP_RAMP_TC : OP_RAMP;
+    const int copies = orb ? OP_ORB_PACK : OP_TRANSPOSE, fwd = orb ? OP_ORB_FWD : OP_FWD;
+    auto push_bwd = [&](int mode) {
+        if (orb) prog.push_back({OP_ORB_ZPACK, mode});
+        prog.push_back({orb ? OP_ORB_BWD : OP_BWD, mode});
+    };
     prog.push_back({ramp, RSRC_Y});        // zc = C y
-    prog.push_back({OP_BWD, BWD_RHS0});   // rhs0 = A^T zc
+    push_bwd(BWD_RHS0);   // rhs0 = A^T zc
     prog.push_back({OP_BWD_FIN, BWD_RHS0});
     prog.push_back({OP_ZERO, 0});         // X = 0, b = 0, g = g' = 0
     prog.push_back({OP_RESTART, -1});     // r = p = rhs0 (X = 0, g = 0)
     for (int k = 0; k < n_outer; ++k) {
         for (int i = 0; i < n_cg; ++i) {
-            prog.push_back({OP_TRANSPOSE, SRC_P});    // q = M p
-            prog.push_back({OP_FWD, SRC_P});
+            prog.push_back({copies, SRC_P});    // q = M p
+            prog.push_back({fwd, SRC_P});
             prog.push_back({ramp, RSRC_Z});
-            prog.push_back({OP_BWD, BWD_Q});
+            push_bwd(BWD_Q);
             prog.push_back({OP_BWD_FIN, BWD_Q});
             prog.push_back({OP_CG_A, 0});
             prog.push_back({OP_CG_B, 0});
@@ -805,8 +911,8 @@ std::vector<Phase> solve_program(int n_outer, int n_cg, bool tc_ramp) {
 // L2-regularised AIR, Eq. (5): (A'^T A + lambda I) X = A'^T Y by n_cg CG steps
 // from X = 0 (the first L2 step of the split-Bregman program with g = 0 and
 // mu = lambda, without the shrink).
-std::vector<Phase> l2_program(int n_cg, bool tc_ramp) {
-    std::vector<Phase> prog = solve_program(1, n_cg, tc_ramp);
+std::vector<Phase> l2_program(int n_cg, bool tc_ramp, bool orb) {
+    std::vector<Phase> prog = solve_program(1, n_cg, tc_ramp, orb);
     prog.pop_back();   // the SHRINK of the outer step
     return prog;
 }
@@ -814,18 +920,23 @@ std::vector<Phase> l2_program(int n_cg, bool tc_ramp) {
 // Forward-backward splitting AIR: per iteration the forward step of Eq. (6),
 // X + step A'^T (Y - A X) (the residual epilogue at mu = 0 gives
 // r = A'^T Y - A'^T A X), then the framelet proximal step.
-std::vector<Phase> fbs_program(int n_iter, bool tc_ramp) {
+std::vector<Phase> fbs_program(int n_iter, bool tc_ramp, bool orb) {
     std::vector<Phase> prog;
     const int ramp = tc_ramp ? OP_RAMP_TC : OP_RAMP;
+    const int copies = orb ? OP_ORB_PACK : OP_TRANSPOSE, fwd = orb ? OP_ORB_FWD : OP_FWD;
+    auto push_bwd = [&](int mode) {
+        if (orb) prog.push_back({OP_ORB_ZPACK, mode});
+        prog.push_back({orb ? OP_ORB_BWD : OP_BWD, mode});
+    };
     prog.push_back({ramp, RSRC_Y});
-    prog.push_back({OP_BWD, BWD_RHS0});
+    push_bwd(BWD_RHS0);
     prog.push_back({OP_BWD_FIN, BWD_RHS0});
     prog.push_back({OP_ZERO, 0});
     for (int k = 0; k < n_iter; ++k) {
-        prog.push_back({OP_TRANSPOSE, SRC_X});
-        prog.push_back({OP_FWD, SRC_X});
+        prog.push_back({copies, SRC_X});
+        prog.push_back({fwd, SRC_X});
         prog.push_back({ramp, RSRC_Z});
-        prog.push_back({OP_BWD, BWD_RESID});
+        push_bwd(BWD_RESID);
         prog.push_back({OP_BWD_FIN, BWD_RESID});
         prog.push_back({OP_AXPY, 0});
         prog.push_back({OP_PROX, 0});
@@ -865,6 +976,10 @@ SliceDesc solve_desc(const air_plan *P, const float *Y, float lambda, float mu, 
     s.mu = mu;
     s.tau = lambda / mu;
     s.resid_out = resid;
+    // A caller that takes the residual history compares it between runs and
+    // versions; its FP64 values show another summation order at 1e-8.  Such a
+    // solve keeps the general projector pair and the order it has always had.
+    if (resid) s.orb = 0;
     return s;
 }
 
@@ -878,7 +993,7 @@ extern "C" air_status air_solve(const air_plan *P, const float *Y, float lambda,
     if (resid) TRY(check_dev_ptr(resid, "resid"));
     const bool tc = P->geom.precision == AIR_PREC_BF16X3 && P->geom.filter == AIR_FILTER_RAMLAK;
     SliceDesc s = solve_desc(P, Y, lambda, mu, X, resid);
-    return run_program_single(P, s, solve_program(n_outer, n_cg, tc), (cudaStream_t)stream);
+    return run_program_single(P, s, solve_program(n_outer, n_cg, tc, s.orb != 0), (cudaStream_t)stream);
 }
 
 extern "C" air_status air_solve_l2(const air_plan *P, const float *Y, float lambda, int n_cg, float *X,
@@ -889,7 +1004,7 @@ extern "C" air_status air_solve_l2(const air_plan *P, const float *Y, float lamb
     TRY(check_dev_ptr(X, "X"));
     const bool tc = P->geom.precision == AIR_PREC_BF16X3 && P->geom.filter == AIR_FILTER_RAMLAK;
     SliceDesc s = solve_desc(P, Y, 0.f, lambda, X, nullptr);
-    return run_program_single(P, s, l2_program(n_cg, tc), (cudaStream_t)stream);
+    return run_program_single(P, s, l2_program(n_cg, tc, P->desc.orb != 0), (cudaStream_t)stream);
 }
 
 extern "C" air_status air_solve_fbs(const air_plan *P, const float *Y, float lambda, float step, int n_iter,
@@ -903,7 +1018,7 @@ extern "C" air_status air_solve_fbs(const air_plan *P, const float *Y, float lam
     s.mu = 0.f;                 // the residual epilogue then gives A'^T (Y - A X)
     s.tau = step * lambda;      // the proximal threshold
     s.step = step;
-    return run_program_single(P, s, fbs_program(n_iter, tc), (cudaStream_t)stream);
+    return run_program_single(P, s, fbs_program(n_iter, tc, P->desc.orb != 0), (cudaStream_t)stream);
 }
 
 extern "C" air_status air_fbp(const air_plan *P, const float *Y, float *X, air_stream stream) {
@@ -936,7 +1051,7 @@ extern "C" air_status air_solve_host(const air_plan *P, const float *Y_host, flo
     CUDA_TRY(cudaMemcpyAsync(P->ybuf, Y_host, sino_bytes(P), cudaMemcpyHostToDevice, st));
     const bool tc = P->geom.precision == AIR_PREC_BF16X3 && P->geom.filter == AIR_FILTER_RAMLAK;
     SliceDesc s = solve_desc(P, P->ybuf, lambda, mu, P->xbuf, nullptr);
-    TRY(run_program_single(P, s, solve_program(n_outer, n_cg, tc), st));
+    TRY(run_program_single(P, s, solve_program(n_outer, n_cg, tc, P->desc.orb != 0), st));
     CUDA_TRY(cudaMemcpyAsync(X_host, P->xbuf, img_bytes(P), cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
     return tc ? air_plan_status(P) : AIR_OK;

@@ -18,7 +18,7 @@ struct air_plan {
     float *xbuf = nullptr;
     void *tc = nullptr;        // tensor-core filter resources (AIR_PREC_BF16X3)
     size_t tc_bytes = 0;
-    int bwd_parts_max = 1;     // view parts the backprojector's part buffer holds
+    int bwd_parts_max = 1;     // images the backprojector's part buffer holds
 };
 
 namespace air {
@@ -28,9 +28,9 @@ air_status check_dev_ptr(const void *p, const char *what);
 bool overlap(const void *a, size_t na, const void *b, size_t nb);
 size_t align_up(size_t v, size_t a);
 double fan_pitch(const air_geometry &g);
-std::vector<Phase> solve_program(int n_outer, int n_cg, bool tc_ramp);
-std::vector<Phase> l2_program(int n_cg, bool tc_ramp);
-std::vector<Phase> fbs_program(int n_iter, bool tc_ramp);
+std::vector<Phase> solve_program(int n_outer, int n_cg, bool tc_ramp, bool orb);
+std::vector<Phase> l2_program(int n_cg, bool tc_ramp, bool orb);
+std::vector<Phase> fbs_program(int n_iter, bool tc_ramp, bool orb);
 air_status check_solve_args(const air_plan *P, const float *Y, float lambda, float mu, int n_outer,
                             int n_cg, const float *X);
 SliceDesc solve_desc(const air_plan *P, const float *Y, float lambda, float mu, float *X, double *resid);
@@ -38,6 +38,9 @@ air_status run_program_single(const air_plan *P, const SliceDesc &s, const std::
                               cudaStream_t st);
 RayFx make_ray_fx(double px, double py, double ux, double uy, int n, unsigned *walk);
 int choose_bwd_parts(const SliceDesc &s);
+// A^T of ext_in (BWD_PLAIN) or zc on the plan's path: the parts and, where
+// there is more than one, their sum with the mode's epilogue.
+cudaError_t launch_backprojection(const SliceDesc &s, int mode, cudaStream_t st);
 air_status autotune(air_plan *P);
 size_t plan_bytes_estimate(const air_geometry &g);
 air_status apply_filter(const air_plan *P, const SliceDesc &base, const float *src, float *dst,

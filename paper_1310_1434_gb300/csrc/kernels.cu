@@ -26,8 +26,13 @@ static cudaError_t opt_in_smem(Kernel kernel, std::atomic<unsigned long long> &d
 // ------------------------------------------------------------------------
 // per-op kernels: one block per tile of one slice
 // ------------------------------------------------------------------------
+// The orbit backprojector is held to three blocks per SM by its shared memory
+// (60 KB at eight frames); its registers must allow as many.
 template <int OP>
-__global__ void __launch_bounds__(AIR_THREADS) k_op(const SliceDesc s, int arg) {
+constexpr int min_blocks = OP == OP_ORB_BWD ? 3 : 0;
+
+template <int OP>
+__global__ void __launch_bounds__(AIR_THREADS, min_blocks<OP>) k_op(const SliceDesc s, int arg) {
     extern __shared__ __align__(16) float sm[];
     const int tile = blockIdx.x;
     if constexpr (OP == OP_FWD) {
@@ -63,6 +68,14 @@ __global__ void __launch_bounds__(AIR_THREADS) k_op(const SliceDesc s, int arg) 
         tile_framelet(s, arg, tile, sm);
     } else if constexpr (OP == OP_TRANSPOSE) {
         tile_transpose(s, arg, tile, sm);
+    } else if constexpr (OP == OP_ORB_PACK) {
+        tile_orb_pack(s, arg, tile, sm);
+    } else if constexpr (OP == OP_ORB_FWD) {
+        tile_orb_fwd(s, arg, tile, sm);
+    } else if constexpr (OP == OP_ORB_ZPACK) {
+        tile_orb_zpack(s, arg, tile);
+    } else if constexpr (OP == OP_ORB_BWD) {
+        tile_orb_bwd(s, arg, tile, sm);
     }
 }
 
@@ -94,6 +107,10 @@ cudaError_t launch_op(int op, const SliceDesc &s, int arg, cudaStream_t st) {
     case OP_PROX: return launch_one<OP_PROX>(s, arg, st);
     case OP_FBP: return launch_one<OP_FBP>(s, arg, st);
     case OP_RESTART: return launch_one<OP_RESTART>(s, arg, st);
+    case OP_ORB_PACK: return launch_one<OP_ORB_PACK>(s, arg, st);
+    case OP_ORB_FWD: return launch_one<OP_ORB_FWD>(s, arg, st);
+    case OP_ORB_ZPACK: return launch_one<OP_ORB_ZPACK>(s, arg, st);
+    case OP_ORB_BWD: return launch_one<OP_ORB_BWD>(s, arg, st);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -121,7 +138,7 @@ __device__ __forceinline__ const SliceDesc &stage_desc(const SliceDesc *__restri
 // Grouped form of one op: the tiles of many slices in one launch, the
 // kernel specialised for the op (its own register budget).
 template <int OP>
-__global__ void __launch_bounds__(AIR_THREADS)
+__global__ void __launch_bounds__(AIR_THREADS, min_blocks<OP>)
 k_group(const SliceDesc *__restrict__ slices, const Task *__restrict__ tasks, int ntasks) {
     extern __shared__ __align__(16) float sm[];
     __shared__ __align__(16) SliceDesc sd;
@@ -148,6 +165,10 @@ k_group(const SliceDesc *__restrict__ slices, const Task *__restrict__ tasks, in
     else if constexpr (OP == OP_TRANSPOSE) tile_transpose(s, t.arg, tile, sm);
     else if constexpr (OP == OP_SHRINK) run_shrink(s, t.arg, tile, sm);
     else if constexpr (OP == OP_RESTART) tile_restart(s, t.arg, tile);
+    else if constexpr (OP == OP_ORB_PACK) tile_orb_pack(s, t.arg, tile, sm);
+    else if constexpr (OP == OP_ORB_FWD) tile_orb_fwd(s, t.arg, tile, sm);
+    else if constexpr (OP == OP_ORB_ZPACK) tile_orb_zpack(s, t.arg, tile);
+    else if constexpr (OP == OP_ORB_BWD) tile_orb_bwd(s, t.arg, tile, sm);
 }
 
 template <int OP>
@@ -188,6 +209,10 @@ cudaError_t launch_group(int op, const SliceDesc *d_slices, const Task *d_tasks,
     case OP_AXPY: return launch_group_op<OP_AXPY>(d_slices, d_tasks, ntasks, total_tiles, smem, st);
     case OP_PROX: return launch_group_op<OP_PROX>(d_slices, d_tasks, ntasks, total_tiles, smem, st);
     case OP_RESTART: return launch_group_op<OP_RESTART>(d_slices, d_tasks, ntasks, total_tiles, smem, st);
+    case OP_ORB_PACK: return launch_group_op<OP_ORB_PACK>(d_slices, d_tasks, ntasks, total_tiles, smem, st);
+    case OP_ORB_FWD: return launch_group_op<OP_ORB_FWD>(d_slices, d_tasks, ntasks, total_tiles, smem, st);
+    case OP_ORB_ZPACK: return launch_group_op<OP_ORB_ZPACK>(d_slices, d_tasks, ntasks, total_tiles, smem, st);
+    case OP_ORB_BWD: return launch_group_op<OP_ORB_BWD>(d_slices, d_tasks, ntasks, total_tiles, smem, st);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -244,7 +269,8 @@ __device__ bool grid_barrier(BatchCtl *ctl) {
 // its first ticket past the phase's last tile; the phase's first ticket
 // (phase_base) counts those closing tickets, one per block, of every earlier
 // phase, and the grid barrier keeps the phases' tickets apart.
-__global__ void __launch_bounds__(AIR_THREADS, 5)
+template <bool ORB>
+__global__ void __launch_bounds__(AIR_THREADS, ORB ? 3 : 5)
 k_persistent(const SliceDesc *__restrict__ slices, int nslices, const Phase *__restrict__ prog,
              int nphases, const int *__restrict__ tile_base, const unsigned long long *__restrict__ phase_base,
              BatchCtl *ctl) {
@@ -264,7 +290,7 @@ k_persistent(const SliceDesc *__restrict__ slices, int nslices, const Phase *__r
             if (t >= ntiles) break;
             while (t >= tb[si + 1]) ++si;       // a block's tickets increase
             const Phase P = prog[(size_t)si * nphases + ph];
-            run_tile(stage_desc(slices, si, &sd, &staged), P.op, P.arg, (int)(t - tb[si]), sm);
+            run_tile<ORB>(stage_desc(slices, si, &sd, &staged), P.op, P.arg, (int)(t - tb[si]), sm);
         }
         if (!grid_barrier(ctl)) return;
     }
@@ -279,15 +305,17 @@ k_persistent(const SliceDesc *__restrict__ slices, int nslices, const Phase *__r
 // parallelism than the L1 gains).
 constexpr int PERSISTENT_BLOCKS = 4;
 
-int persistent_grid(size_t smem) {
+namespace {
+template <bool ORB>
+int grid_of(size_t smem) {
     int dev = 0, sms = 0, per = 0, max_smem = 0;
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
     if (cudaDeviceGetAttribute(&max_smem, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) != cudaSuccess)
         return 0;
     static std::atomic<unsigned long long> attr_done{0};
-    if (opt_in_smem(k_persistent, attr_done) != cudaSuccess) return 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_persistent, AIR_THREADS, smem) != cudaSuccess)
+    if (opt_in_smem(k_persistent<ORB>, attr_done) != cudaSuccess) return 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k_persistent<ORB>, AIR_THREADS, smem) != cudaSuccess)
         return 0;
     const int blocks = per < PERSISTENT_BLOCKS ? per : PERSISTENT_BLOCKS;
     if (blocks < 1 || max_smem <= 0) return 0;
@@ -297,14 +325,17 @@ int persistent_grid(size_t smem) {
     const double need = (double)blocks * ((double)smem + 2048.0);
     int pct = (int)(100.0 * need / max_smem) + 2;
     if (pct > 100) pct = 100;
-    if (cudaFuncSetAttribute(k_persistent, cudaFuncAttributePreferredSharedMemoryCarveout, pct) != cudaSuccess)
+    if (cudaFuncSetAttribute(k_persistent<ORB>, cudaFuncAttributePreferredSharedMemoryCarveout, pct) != cudaSuccess)
         return 0;
     return sms * blocks;
 }
+}  // namespace
+
+int persistent_grid(size_t smem, bool orb) { return orb ? grid_of<true>(smem) : grid_of<false>(smem); }
 
 cudaError_t launch_persistent(const SliceDesc *d_slices, int nslices, const Phase *d_prog,
                               int nphases, const int *d_tile_base, const unsigned long long *d_phase_base,
-                              BatchCtl *d_ctl, int grid, size_t smem, cudaStream_t st) {
+                              BatchCtl *d_ctl, int grid, size_t smem, bool orb, cudaStream_t st) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(AIR_THREADS);
@@ -315,7 +346,7 @@ cudaError_t launch_persistent(const SliceDesc *d_slices, int nslices, const Phas
     attr[0].val.cooperative = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_persistent, d_slices, nslices, d_prog, nphases, d_tile_base, d_phase_base,
+    return cudaLaunchKernelEx(&cfg, orb ? k_persistent<true> : k_persistent<false>, d_slices, nslices, d_prog, nphases, d_tile_base, d_phase_base,
                               d_ctl);
 }
 

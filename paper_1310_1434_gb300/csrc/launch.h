@@ -35,9 +35,10 @@ struct BatchCtl {
 // earlier phases of their tiles plus one closing ticket per block.
 cudaError_t launch_persistent(const SliceDesc *d_slices, int nslices, const Phase *d_prog,
                               int nphases, const int *d_tile_base, const unsigned long long *d_phase_base,
-                              BatchCtl *d_ctl, int grid, size_t smem, cudaStream_t st);
-// Largest co-resident grid of the persistent kernel for the given smem.
-int persistent_grid(size_t smem);
+                              BatchCtl *d_ctl, int grid, size_t smem, bool orb, cudaStream_t st);
+// Largest co-resident grid of the persistent kernel for the given smem (orb:
+// the form that also runs the orbit ops).
+int persistent_grid(size_t smem, bool orb);
 // Poll budget of the persistent kernel's grid-barrier wait on the current
 // device (negative: the default).  Synchronous.
 cudaError_t set_barrier_budget(long long polls);

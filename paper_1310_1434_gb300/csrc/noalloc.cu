@@ -5,6 +5,7 @@
 // allocate.  Its only scratch -- the filtered sinogram C Y and the
 // backprojector's per-view-part images -- lives in the file-scope device
 // array below instead of in plan or caller memory.
+#include <algorithm>
 #include <mutex>
 #include <string>
 
@@ -106,15 +107,22 @@ extern "C" air_status air_filtered_backproject_noalloc(const air_plan *P, const 
     if (e == cudaSuccess) {
         // X = A^T (C Y) over S view parts that fit beside C Y (one part is
         // written straight to X), their sum by the finish op
-        const size_t nn = (size_t)P->geom.n * P->geom.n, off = align_up(samples, 64);
-        int parts = P->desc.bwd_parts;
-        while (parts > 1 && off + (size_t)parts * nn > NOALLOC_FLOATS) --parts;
+        const size_t nn = (size_t)P->geom.n * P->geom.n;
+        size_t off = align_up(samples, 64);
+        const size_t nz = d.orb ? align_up((size_t)d.orb_npad * orb_planes(d) * 4, 64) : 0;
+        if (d.orb && off + nz + 8 * nn <= NOALLOC_FLOATS) {          // the orbit path's packed samples, eight images
+            d.orb_z = reinterpret_cast<float4 *>(scratch + off);
+            off += nz;
+            d.orb_splits = std::min(d.orb_splits, (int)((NOALLOC_FLOATS - off) / (8 * nn)));
+        } else {
+            d.orb = 0;
+        }
+        const size_t room = (NOALLOC_FLOATS - off) / nn;             // images beside them
         d.ext_in = scratch;
         d.ext_out = X;
-        d.bwd_parts = parts;
-        d.bwd_part = parts > 1 ? scratch + off : nullptr;
-        e = launch_op(OP_BWD, d, BWD_PLAIN, s);
-        if (e == cudaSuccess && parts > 1) e = launch_op(OP_BWD_FIN, d, BWD_PLAIN, s);
+        d.bwd_parts = std::max(1, (int)std::min<size_t>(P->desc.bwd_parts, room));
+        d.bwd_part = bwd_images(d) > 1 ? scratch + off : nullptr;
+        e = launch_backprojection(d, BWD_PLAIN, s);
     }
     if (e != cudaSuccess) return fail(AIR_ERR_CUDA, std::string("filtered backprojection: ") + cudaGetErrorString(e));
     return AIR_OK;

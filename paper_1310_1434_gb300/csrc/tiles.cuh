@@ -4,6 +4,7 @@
 #pragma once
 
 #include "air_internal.cuh"
+#include "tiles_orbit.cuh"
 
 namespace air {
 
@@ -343,36 +344,70 @@ __device__ __forceinline__ void tile_bwd(const SliceDesc &s, int mode, int tile,
 }
 
 
-// Sums the S view parts of the backprojection in a fixed order and applies
-// the mode's epilogue (the CG and residual updates of the Eq. 5 system).
+// Sums the parts of the backprojection (bwd_images of them) in a fixed order
+// and applies the mode's epilogue (the CG and residual updates of the Eq. 5
+// system).  A thread takes N neighbouring pixels: four with 16-byte accesses
+// for the orbit path's eight images and more, where the image's size keeps
+// them aligned (24 images at 512^2: 19 -> 9 us); one for the general path,
+// whose tuned split, and with it the order of its sums, follows this sum's
+// time.
+template <int N>
+__device__ __forceinline__ double bwd_fin(const SliceDesc &s, int mode, int i) {
+    struct __align__(4 * N) Vec { float v[N]; };
+    auto get = [&](const float *a) { return *reinterpret_cast<const Vec *>(a + i); };
+    auto put = [&](float *a, const Vec &x) { *reinterpret_cast<Vec *>(a + i) = x; };
+    const int S = bwd_images(s);
+    const size_t nn = (size_t)s.n * s.n;
+    Vec a{};
+#pragma unroll (N == 4 ? 8 : 4)
+    for (int p = 0; p < S; ++p) {
+        const Vec x = get(s.bwd_part + p * nn);
+#pragma unroll
+        for (int q = 0; q < N; ++q) a.v[q] += x.v[q];
+    }
+#pragma unroll
+    for (int q = 0; q < N; ++q) a.v[q] *= s.dx;
+    double part = 0.0;
+    if (mode == BWD_PLAIN) {
+        put(s.ext_out, a);
+    } else if (mode == BWD_RHS0) {
+        put(s.rhs0, a);
+    } else if (mode == BWD_RESID) {
+        const Vec x = get(s.x), g = get(s.g), b = get(s.rhs0);
+        Vec r;
+#pragma unroll
+        for (int q = 0; q < N; ++q) {
+            r.v[q] = fmaf(s.mu, g.v[q], b.v[q]) - fmaf(s.mu, x.v[q], a.v[q]);
+            part += (double)r.v[q] * (double)r.v[q];
+        }
+        put(s.r, r);
+        put(s.p, r);
+    } else {  // BWD_Q
+        const Vec p = get(s.p);
+        Vec o;
+#pragma unroll
+        for (int q = 0; q < N; ++q) {
+            o.v[q] = fmaf(s.mu, p.v[q], a.v[q]);
+            part += (double)p.v[q] * (double)o.v[q];
+        }
+        put(s.q, o);
+    }
+    return part;
+}
+
 __device__ __forceinline__ void tile_bwd_fin(const SliceDesc &s, int mode, int tile) {
     __shared__ double sh[AIR_THREADS / 32];
     if (mode == BWD_Q && s.cg->stop) return;
-    const int nn = s.n * s.n, S = s.bwd_parts;
-    const int base = tile * VEC_PER_TILE;
+    const int nn = s.n * s.n, base = tile * VEC_PER_TILE;
     double part = 0.0;
+    if (s.orb && nn % 4 == 0) {
+        const int i = base + 4 * (int)threadIdx.x;
+        if (i < nn) part = bwd_fin<4>(s, mode, i);
+    } else {
 #pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int i = base + k * AIR_THREADS + threadIdx.x;
-        if (i >= nn) continue;
-        float a = 0.f;
-        for (int p = 0; p < S; ++p) a += __ldcg(s.bwd_part + (size_t)p * nn + i);
-        const float acc = s.dx * a;
-        if (mode == BWD_PLAIN) {
-            s.ext_out[i] = acc;
-        } else if (mode == BWD_RHS0) {
-            s.rhs0[i] = acc;
-        } else if (mode == BWD_RESID) {
-            const float mx = fmaf(s.mu, s.x[i], acc);
-            const float rv = fmaf(s.mu, s.g[i], s.rhs0[i]) - mx;
-            s.r[i] = rv;
-            s.p[i] = rv;
-            part += (double)rv * (double)rv;
-        } else {  // BWD_Q
-            const float pv = s.p[i];
-            const float qv = fmaf(s.mu, pv, acc);
-            s.q[i] = qv;
-            part += (double)pv * (double)qv;
+        for (int k = 0; k < 4; ++k) {
+            const int i = base + k * AIR_THREADS + (int)threadIdx.x;
+            if (i < nn) part += bwd_fin<1>(s, mode, i);
         }
     }
     if (mode == BWD_PLAIN || mode == BWD_RHS0) return;
@@ -892,6 +927,9 @@ __host__ inline size_t tile_smem(const SliceDesc &s, int op) {
     case OP_FRAMELET: case OP_FRAMELET_T: return sizeof(float) * 9 * SHR_H * SHR_H;
     case OP_TRANSPOSE: return sizeof(float) * 32 * 33;
     case OP_BWD: return sizeof(float) * BWD_SMEM_FLOATS;
+    case OP_ORB_PACK: return sizeof(float) * ORB_PACK_FLOATS;
+    case OP_ORB_FWD: return s.orb_ks > 1 ? sizeof(float4) * AIR_THREADS * orb_planes(s) : 0;
+    case OP_ORB_BWD: return orb_bwd_smem(s.orb);
     default: return 0;
     }
 }
@@ -904,7 +942,8 @@ __device__ __forceinline__ void run_shrink(const SliceDesc &s, int arg, int tile
     tile_shrink(s, a, tile, true, nullptr, sm);
 }
 
-// One tile of any op (used by the persistent kernel).
+// One tile of any op (used by the persistent kernel; ORB: also the orbit ops).
+template <bool ORB>
 __device__ __forceinline__ void run_tile(const SliceDesc &s, int op, int arg, int tile, float *sm) {
     switch (op) {
     case OP_FWD: tile_fwd(s, arg, tile); break;
@@ -920,7 +959,14 @@ __device__ __forceinline__ void run_tile(const SliceDesc &s, int op, int arg, in
     case OP_FBP: tile_fbp(s, tile); break;
     case OP_SHRINK: run_shrink(s, arg, tile, sm); break;
     case OP_RESTART: tile_restart(s, arg, tile); break;
-    default: break;
+    default:
+        if constexpr (ORB) {
+            if (op == OP_ORB_PACK) tile_orb_pack(s, arg, tile, sm);
+            else if (op == OP_ORB_FWD) tile_orb_fwd(s, arg, tile, sm);
+            else if (op == OP_ORB_ZPACK) tile_orb_zpack(s, arg, tile);
+            else if (op == OP_ORB_BWD) tile_orb_bwd(s, arg, tile, sm);
+        }
+        break;
     }
 }
 
