@@ -234,7 +234,15 @@ constexpr int VEC_PER_TILE = AIR_THREADS * 4;   // elementwise ops: 4 per thread
 __host__ __device__ inline int tiles_vec(const SliceDesc &s) {
     return (s.n * s.n + VEC_PER_TILE - 1) / VEC_PER_TILE;
 }
-constexpr int SHR_T = 16;                      // shrink/framelet output tile
+// fused framelet passes: a block takes fs_down tiles of 30 x 6 pixels
+// downwards, one where the image gives the device few blocks (12 us instead
+// of 17 at 64^2), four from 768^2 on, where their joint reduction pays (57
+// instead of 69 us at 1024^2; 27 against 28 at 512^2)
+__host__ __device__ inline int fs_down(int n) { return n >= 768 ? 4 : 1; }
+__host__ __device__ inline int tiles_fs(const SliceDesc &s) {
+    return ((s.n + 29) / 30) * ((s.n + 6 * fs_down(s.n) - 1) / (6 * fs_down(s.n)));
+}
+constexpr int SHR_T = 16;                      // framelet (API call) and FBP output tile
 __host__ __device__ inline int tiles_shr(const SliceDesc &s) {
     return ((s.n + SHR_T - 1) / SHR_T) * ((s.n + SHR_T - 1) / SHR_T);
 }
@@ -253,14 +261,14 @@ __host__ __device__ inline int tiles_of(const SliceDesc &s, int op) {
     case OP_ORB_FWD: return tiles_orb_fwd(s);
     case OP_ORB_ZPACK: return s.orb_nseg * orb_zchunks(s);
     case OP_ORB_BWD: return tiles_orb_bwd(s);
-    case OP_SHRINK: case OP_FRAMELET: case OP_FRAMELET_T: case OP_PROX: case OP_FBP:
-        return tiles_shr(s);
+    case OP_SHRINK: case OP_PROX: return tiles_fs(s);
+    case OP_FRAMELET: case OP_FRAMELET_T: case OP_FBP: return tiles_shr(s);
     default: return 0;
     }
 }
 // largest number of tiles of any reducing op: sizes SliceDesc::partial
 __host__ inline int max_reduce_tiles(const SliceDesc &s) {
-    const int b = tiles_vec(s), c = tiles_shr(s);
+    const int b = tiles_vec(s), c = tiles_fs(s);
     return b > c ? b : c;
 }
 

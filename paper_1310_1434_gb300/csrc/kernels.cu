@@ -62,7 +62,7 @@ __global__ void __launch_bounds__(AIR_THREADS, min_blocks<OP>) k_op(const SliceD
             run_shrink(s, arg, tile, sm);
         } else {  // stand-alone call: X, b (read), scratch b', g from the ext operands
             ShrinkArgs a{s.ext_in, s.ext_out, s.b2, s.ext_out2, s.tau};
-            tile_shrink(s, a, tile, true, s.ext_scalar, sm);
+            tile_shrink(s, a, tile, s.ext_scalar, sm);
         }
     } else if constexpr (OP == OP_FRAMELET) {
         tile_framelet(s, arg, tile, sm);

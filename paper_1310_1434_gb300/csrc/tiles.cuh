@@ -689,6 +689,8 @@ __device__ __forceinline__ float ftap(int a, int p) {
 }
 
 __device__ __forceinline__ int wrapi(int v, int n) {
+    const int w = v < 0 ? v + n : (v >= n ? v - n : v);
+    if ((unsigned)w < (unsigned)n) return w;       // no division within one period of the image
     v %= n;
     return v < 0 ? v + n : v;
 }
@@ -735,81 +737,169 @@ struct ShrinkArgs {
     float tau;
 };
 
-constexpr int SHR_H = SHR_T + 2;   // coefficient tile incl. halo 1
-constexpr int SHR_X = SHR_T + 4;   // image tile incl. halo 2
+// A sum of squares kept in two floats (hi + lo, 48 significant bits): the
+// squares of differences x - y enter with their rounding errors (Knuth's
+// two-sum, an FMA for the product's error).
+struct SumSq {
+    float hi, lo, top;             // top: the largest |x - y|
+    __device__ __forceinline__ void add_diff(float x, float y) {
+        const float e = __fsub_rn(x, y), yy = __fsub_rn(e, x);
+        top = fmaxf(top, fabsf(e));
+        const float de = __fsub_rn(__fsub_rn(x, __fsub_rn(e, yy)), __fadd_rn(y, yy));   // x - y = e + de
+        const float p = __fmul_rn(e, e), dp = fmaf(2.f * e, de, fmaf(e, e, -p));
+        add(p, dp);
+    }
+    __device__ __forceinline__ void add(float p, float dp) {
+        const float h = __fadd_rn(hi, p), t = __fsub_rn(h, hi);
+        lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(__fsub_rn(hi, __fsub_rn(h, t)), __fsub_rn(p, t)), dp));
+        hi = h;
+    }
+    // the squares neither overflowed nor lost what the sum needs of them
+    __device__ __forceinline__ bool fits() const { return top == 0.f || (top > 0x1p-40f && top < 0x1p50f); }
+};
 
-// Shared-memory layout of the shrink tile (floats): X tile, then E[9][SHR_H^2]
-constexpr int SHR_SMEM_FLOATS = SHR_X * SHR_X + 9 * SHR_H * SHR_H;
+// The fused framelet passes W, soft threshold, W^T of one FS_W x FS_H output
+// tile: the image in shared memory with a halo of 2, the nine bands'
+// coefficients with a halo of 1 (both periodic), a warp to a row, so that
+// the row pass of W^T takes its neighbours by shuffles and shared memory
+// hands only its results to the column pass.  SHRINK: t = W X + b; d =
+// soft(t); b_out = t - d; the output is W^T(d - b_out), and thread 0 gets the
+// tile's sum of ||W X - d||^2.  Otherwise (the proximal step of
+// forward-backward splitting for R = ||W X||_1 with the tight frame W):
+// W^T soft(W X).  The high-pass bands are shrunk, the low-pass band kept.
+// The residual's squares are summed per warp in two floats (SumSq) and from
+// there in FP64: GB300 issues one FP64 instruction for 64 FP32 ones, and four
+// for each of the nine coefficients bound the form that did (FP64 pipe 67 %
+// active).  The coefficient tile is 32 x 8, one row for each warp.
+// At 512^2 the kernel takes 20 us, 36 with FP64 squares and 16 x 16 tiles
+// (49 % of the issue slots; the chain of loads, barriers and the reduction of
+// each short block bounds it).  Walking each warp down a strip of 8 rows with
+// all passes in registers took 27 us: too few warps for that chain.
+constexpr int FS_W = 30, FS_H = 6;                 // output tile, as tiles_fs counts them
+constexpr int FS_CW = FS_W + 2, FS_CH = FS_H + 2;  // coefficient tile
+constexpr int FS_XW = FS_W + 4, FS_XH = FS_H + 4;  // image tile
+constexpr int FS_SMEM_FLOATS = FS_XW * FS_XH + 9 * FS_CW * FS_CH;
+static_assert(FS_CW == 32 && FS_CH == AIR_THREADS / 32, "one coefficient per thread, a row for each warp");
 
-__device__ __forceinline__ void tile_shrink(const SliceDesc &s, const ShrinkArgs &A, int tile,
-                                            bool reduce, double *resid_dst, float *sm) {
+// WIDE: only the residual, every square in FP64 (values whose squares leave
+// FP32's range).
+template <bool SHRINK, bool WIDE>
+__device__ __forceinline__ void fs_coefficients(const ShrinkArgs &A, int n, int x0, int y0, const float *bo,
+                                                const float *Xs, float *R, SumSq &sq, double &wide) {
+    const size_t nn = (size_t)n * n;
+    const float c1 = 0.35355339059327373f;
+    const int k = threadIdx.x, cy = k / FS_CW, cx = k % FS_CW;
+    const bool keep = cy >= 1 && cy <= FS_H && cx >= 1 && cx <= FS_W && y0 - 1 + cy < n && x0 - 1 + cx < n;
+    float *out = A.b_out + (size_t)(y0 - 1 + cy) * n + (x0 - 1 + cx);              // used where keep
+    float f[3][3];                 // row filters of the rows above, at and below; f[.][1] without its factor c1
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+        const float *row = Xs + (cy + p) * FS_XW + cx;
+        f[p][0] = fmaf(0.25f, __fadd_rn(row[0], row[2]), 0.5f * row[1]);
+        f[p][1] = __fsub_rn(row[0], row[2]);
+        f[p][2] = fmaf(-0.25f, __fadd_rn(row[0], row[2]), 0.5f * row[1]);
+    }
+#pragma unroll
+    for (int band = 0; band < 9; ++band) {
+        const int a = band / 3, b = band % 3;
+        // the column filter; the antisymmetric row filter's factor goes into
+        // it by an FMA, as framelet9 is compiled (same rounding)
+        const float mid = b == 1 ? __fmul_rn(c1, f[1][1]) : f[1][b], low = b == 1 ? __fmul_rn(c1, f[2][1]) : f[2][b];
+        const float sum = b == 1 ? fmaf(c1, f[0][1], low) : __fadd_rn(f[0][b], low);
+        const float dif = b == 1 ? fmaf(c1, f[0][1], -low) : __fsub_rn(f[0][b], low);
+        const float wx = a == 0 ? fmaf(0.25f, sum, 0.5f * mid) : (a == 1 ? __fmul_rn(c1, dif) : fmaf(-0.25f, sum, 0.5f * mid));
+        const float t = SHRINK ? __fadd_rn(wx, bo[band]) : wx;
+        float d = t;
+        if (band > 0) {
+            const float m = fabsf(t) - A.tau;
+            d = m > 0.f ? copysignf(m, t) : 0.f;
+        }
+        if (WIDE) {
+            const double dd = (double)wx - (double)d;
+            if (keep) wide += dd * dd;
+            continue;
+        }
+        float e = d;
+        if (SHRINK) {
+            const float bn = __fsub_rn(t, d);
+            e = __fsub_rn(d, bn);
+            if (keep) {
+                out[band * nn] = bn;
+                sq.add_diff(wx, d);
+            }
+        }
+        // the row pass of W^T: neighbours are lanes (halo lanes get no output)
+        const float el = __shfl_up_sync(0xffffffffu, e, 1), eh = __shfl_down_sync(0xffffffffu, e, 1);
+        R[band * (FS_CW * FS_CH) + k] = fmaf(ftap(b, 1), el, fmaf(ftap(b, 0), e, fmaf(ftap(b, -1), eh, 0.f)));
+    }
+}
+
+template <bool SHRINK>
+__device__ __forceinline__ double fs_tile(const ShrinkArgs &A, int n, int tile, float *sm) {
     __shared__ double sh[AIR_THREADS / 32];
-    const int n = s.n, nn = n * n;
-    const int tpr = (n + SHR_T - 1) / SHR_T;
-    const int x0 = (tile % tpr) * SHR_T, y0 = (tile / tpr) * SHR_T;
-    float *Xs = sm;                      // [SHR_X][SHR_X], origin (y0-2, x0-2)
-    float *E = sm + SHR_X * SHR_X;       // [9][SHR_H][SHR_H], origin (y0-1, x0-1)
-    for (int k = threadIdx.x; k < SHR_X * SHR_X; k += AIR_THREADS) {
-        const int ly = k / SHR_X, lx = k % SHR_X;
-        Xs[k] = A.X[wrapi(y0 - 2 + ly, n) * n + wrapi(x0 - 2 + lx, n)];
-    }
-    __syncthreads();
-    double part = 0.0;
-    for (int k = threadIdx.x; k < SHR_H * SHR_H; k += AIR_THREADS) {
-        const int cy = k / SHR_H, cx = k % SHR_H;
-        const int gy = wrapi(y0 - 1 + cy, n), gx = wrapi(x0 - 1 + cx, n);
-        const bool interior = cy >= 1 && cy <= SHR_T && cx >= 1 && cx <= SHR_T &&
-                              y0 - 1 + cy < n && x0 - 1 + cx < n;
-        float nb3[3][3];
+    const int tpr = (n + FS_W - 1) / FS_W, ty = tile / tpr;
+    const int x0 = (tile - ty * tpr) * FS_W, rows = fs_down(n) * FS_H;
+    const int ly = threadIdx.x / FS_CW, lx = threadIdx.x % FS_CW;
+    const size_t nn = (size_t)n * n;
+    float *R = sm + FS_XW * FS_XH;
+    SumSq sq{0.f, 0.f, 0.f};
+    double total = 0.0;
+#pragma unroll 1
+    for (int y0 = ty * rows; y0 < min(n, (ty + 1) * rows); y0 += FS_H) {
+        // b and the image tile (origin x0 - 2, y0 - 2) in one memory latency
+        float bo[9];
+        if (SHRINK) {
+            const float *p = A.b_in + (size_t)wrapi(y0 - 1 + ly, n) * n + wrapi(x0 - 1 + lx, n);
 #pragma unroll
-        for (int p = 0; p < 3; ++p)
-#pragma unroll
-            for (int q = 0; q < 3; ++q) nb3[p][q] = Xs[(cy + p) * SHR_X + cx + q];
-        float wx[9];
-        framelet9(nb3, wx);
-        const size_t gi = (size_t)gy * n + gx;
-#pragma unroll
-        for (int band = 0; band < 9; ++band) {
-            const float bo = A.b_in[(size_t)band * nn + gi];
-            const float t = wx[band] + bo;
-            float d = t;
-            if (band > 0) {
-                const float m = fabsf(t) - A.tau;
-                d = m > 0.f ? copysignf(m, t) : 0.f;
-            }
-            const float bn = t - d;
-            E[band * SHR_H * SHR_H + k] = d - bn;
-            if (interior) {
-                A.b_out[(size_t)band * nn + gi] = bn;
-                const double e = (double)wx[band] - (double)d;
-                part += e * e;
-            }
+            for (int band = 0; band < 9; ++band) bo[band] = __ldg(p + band * nn);
         }
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < SHR_T * SHR_T; k += AIR_THREADS) {
-        const int ly = k / SHR_T, lx = k % SHR_T;
-        if (y0 + ly >= n || x0 + lx >= n) continue;
-        float acc = 0.f;
-#pragma unroll
-        for (int band = 0; band < 9; ++band) {
-            float e3[3][3];
-            const float *Eb = E + band * SHR_H * SHR_H;
-#pragma unroll
-            for (int p = 0; p < 3; ++p)
-#pragma unroll
-                for (int q = 0; q < 3; ++q) e3[p][q] = Eb[(ly + p) * SHR_H + lx + q];
-            acc += framelet_t1(band / 3, band % 3, e3);
+        for (int k = threadIdx.x; k < FS_XW * FS_XH; k += AIR_THREADS) {
+            const int iy = k / FS_XW, ix = k - iy * FS_XW;
+            sm[k] = __ldg(A.X + (size_t)wrapi(y0 - 2 + iy, n) * n + wrapi(x0 - 2 + ix, n));
         }
-        A.g[(size_t)(y0 + ly) * n + x0 + lx] = acc;
-    }
-    if (!reduce) {
         __syncthreads();
-        return;
+        SumSq one{0.f, 0.f, 0.f};
+        double wide = 0.0;
+        fs_coefficients<SHRINK, false>(A, n, x0, y0, bo, sm, R, one, wide);
+        const int out_of_range = __syncthreads_or(!one.fits());
+        if (SHRINK && out_of_range) {
+            fs_coefficients<SHRINK, SHRINK>(A, n, x0, y0, bo, sm, R, one, wide);
+            total += block_sum(wide, sh);
+        } else if (SHRINK) {
+            sq.add(one.hi, one.lo);
+        }
+        if (ly < FS_H && lx < FS_W && y0 + ly < n && x0 + lx < n) {
+            float acc = 0.f;       // the column pass, in framelet_t1's order
+#pragma unroll
+            for (int band = 0; band < 9; ++band) {
+                const float *r = R + band * (FS_CW * FS_CH) + ly * FS_CW + lx + 1;
+                const int a = band / 3;
+                acc += fmaf(ftap(a, 1), r[0], fmaf(ftap(a, 0), r[FS_CW], fmaf(ftap(a, -1), r[2 * FS_CW], 0.f)));
+            }
+            A.g[(size_t)(y0 + ly) * n + x0 + lx] = acc;
+        }
+        __syncthreads();           // the next tile's
     }
-    part = block_sum(part, sh);
+    if (SHRINK) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            const float hi = __shfl_xor_sync(0xffffffffu, sq.hi, o), lo = __shfl_xor_sync(0xffffffffu, sq.lo, o);
+            sq.add(hi, lo);
+        }
+        if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = (double)sq.hi + (double)sq.lo;
+        __syncthreads();
+        if (threadIdx.x == 0)
+            for (int w = 0; w < AIR_THREADS / 32; ++w) total += sh[w];
+    }
+    return total;
+}
+
+__device__ __forceinline__ void tile_shrink(const SliceDesc &s, const ShrinkArgs &A, int tile, double *resid_dst,
+                                            float *sm) {
+    __shared__ double sh[AIR_THREADS / 32];
+    const double part = fs_tile<true>(A, s.n, tile, sm);
     double tot;
-    if (reduce_tiles(s, tile, tiles_shr(s), part, sh, &tot) && threadIdx.x == 0) {
+    if (reduce_tiles(s, tile, tiles_fs(s), part, sh, &tot) && threadIdx.x == 0) {
         const double rn = sqrt(tot);
         CgState *c = s.cg;
         c->resid = rn;
@@ -820,60 +910,13 @@ __device__ __forceinline__ void tile_shrink(const SliceDesc &s, const ShrinkArgs
     __syncthreads();
 }
 
-// The proximal step of forward-backward splitting for R = ||W X||_1 with the
-// tight frame W (W^T W = I): x = W^T S_tau(W q), the high-pass bands
-// soft-thresholded by tau = step * lambda and the low-pass band kept.  Reads q
-// (with a 2-pixel periodic halo) and writes x, so tiles never read what
-// another tile writes.
+// Reads q (with a 2-pixel periodic halo) and writes x, so tiles never read
+// what another tile writes.
 __device__ __forceinline__ void tile_prox(const SliceDesc &s, int tile, float *sm) {
-    const int n = s.n;
-    const int tpr = (n + SHR_T - 1) / SHR_T;
-    const int x0 = (tile % tpr) * SHR_T, y0 = (tile / tpr) * SHR_T;
-    float *Xs = sm;                      // [SHR_X][SHR_X], origin (y0-2, x0-2)
-    float *E = sm + SHR_X * SHR_X;       // [9][SHR_H][SHR_H], origin (y0-1, x0-1)
-    for (int k = threadIdx.x; k < SHR_X * SHR_X; k += AIR_THREADS) {
-        const int ly = k / SHR_X, lx = k % SHR_X;
-        Xs[k] = s.q[wrapi(y0 - 2 + ly, n) * n + wrapi(x0 - 2 + lx, n)];
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < SHR_H * SHR_H; k += AIR_THREADS) {
-        const int cy = k / SHR_H, cx = k % SHR_H;
-        float nb3[3][3];
-#pragma unroll
-        for (int p = 0; p < 3; ++p)
-#pragma unroll
-            for (int q = 0; q < 3; ++q) nb3[p][q] = Xs[(cy + p) * SHR_X + cx + q];
-        float wx[9];
-        framelet9(nb3, wx);
-#pragma unroll
-        for (int band = 0; band < 9; ++band) {
-            float d = wx[band];
-            if (band > 0) {
-                const float m = fabsf(d) - s.tau;
-                d = m > 0.f ? copysignf(m, d) : 0.f;
-            }
-            E[band * SHR_H * SHR_H + k] = d;
-        }
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < SHR_T * SHR_T; k += AIR_THREADS) {
-        const int ly = k / SHR_T, lx = k % SHR_T;
-        if (y0 + ly >= n || x0 + lx >= n) continue;
-        float acc = 0.f;
-#pragma unroll
-        for (int band = 0; band < 9; ++band) {
-            float e3[3][3];
-            const float *Eb = E + band * SHR_H * SHR_H;
-#pragma unroll
-            for (int p = 0; p < 3; ++p)
-#pragma unroll
-                for (int q = 0; q < 3; ++q) e3[p][q] = Eb[(ly + p) * SHR_H + lx + q];
-            acc += framelet_t1(band / 3, band % 3, e3);
-        }
-        s.x[(size_t)(y0 + ly) * n + x0 + lx] = acc;
-    }
-    __syncthreads();
+    fs_tile<false>(ShrinkArgs{s.q, nullptr, nullptr, s.x, s.tau}, s.n, tile, sm);
 }
+
+constexpr int SHR_H = SHR_T + 2;   // framelet tile incl. halo 1
 
 // out = W in (adjoint = 0) or W^T in (adjoint = 1), for the API call.
 __device__ __forceinline__ void tile_framelet(const SliceDesc &s, int adjoint, int tile, float *sm) {
@@ -923,7 +966,7 @@ __device__ __forceinline__ void tile_framelet(const SliceDesc &s, int adjoint, i
 __host__ inline size_t tile_smem(const SliceDesc &s, int op) {
     switch (op) {
     case OP_RAMP: return sizeof(float) * (4 * (size_t)((3 * s.nb + 2 * RAMP_R + 4 + 3) / 4) + (size_t)s.nb);
-    case OP_SHRINK: case OP_PROX: return sizeof(float) * SHR_SMEM_FLOATS;
+    case OP_SHRINK: case OP_PROX: return sizeof(float) * FS_SMEM_FLOATS;
     case OP_FRAMELET: case OP_FRAMELET_T: return sizeof(float) * 9 * SHR_H * SHR_H;
     case OP_TRANSPOSE: return sizeof(float) * 32 * 33;
     case OP_BWD: return sizeof(float) * BWD_SMEM_FLOATS;
@@ -939,7 +982,7 @@ __host__ inline size_t tile_smem(const SliceDesc &s, int op) {
 // even steps and to g2 on odd ones (the restart needs the previous g).
 __device__ __forceinline__ void run_shrink(const SliceDesc &s, int arg, int tile, float *sm) {
     ShrinkArgs a{s.x, arg ? s.b2 : s.b, arg ? s.b : s.b2, arg ? s.g2 : s.g, s.tau};
-    tile_shrink(s, a, tile, true, nullptr, sm);
+    tile_shrink(s, a, tile, nullptr, sm);
 }
 
 // One tile of any op (used by the persistent kernel; ORB: also the orbit ops).
