@@ -246,21 +246,23 @@ AIR_API air_status air_solve_host(const air_plan *plan, const float *Y_host, flo
  * n_cg[i], X[i]).  The programs advance phase by phase, each phase one
  * grouped launch over the tiles of its slices (FP32 and BF16X3 plans may be
  * mixed); the launch sequence is captured into a CUDA graph once per batch
- * composition and replayed by later calls with the same arguments.  The
- * graph runs the slices as one chain of phases or as two independent chains
- * (slice i in chain i mod 2); the first call of a composition runs both
- * graphs once (twice each when they are within 3 %), keeps the faster and
- * returns the last run's result, so it takes two to four times as long
- * (batches too large for two chains to pay are run once).  plans must be distinct (each slice uses its plan's
- * workspace).  Arrays of length n are HOST arrays; Y[i], X[i] are device
+ * composition (plans, n_outer, n_cg) and replayed by later calls with their
+ * own Y, X, lambda and mu; the graphs of the last eight compositions are kept
+ * until one of their plans is destroyed.  The graph runs the slices as one
+ * chain of phases or as two independent chains (slice i in chain i mod 2);
+ * the first call of a batch of new shapes (geometries, n_outer, n_cg) runs
+ * both graphs once (twice each when they are within 3 %), keeps the faster
+ * and returns the last run's result, so it takes two to four times as long
+ * (batches too large for two chains to pay are run once).  plans must be
+ * distinct (each slice uses its plan's workspace).  Arrays of length n are HOST arrays; Y[i], X[i] are device
  * pointers.  Returns after the batch has finished (synchronises `stream`). */
 AIR_API air_status air_solve_batch(int n, air_plan *const *plans, const float *const *Y,
                            const float *lambda, const float *mu, const int *n_outer,
                            const int *n_cg, float *const *X, air_stream stream);
 
-/* Diagnostic description of the grouped batch graph in use (built by the
- * last air_solve_batch or air_solve_batch_host call that built one; the
- * paper has no counterpart): its number of chains (1 or 2) and the kernels
+/* Diagnostic description of the grouped batch graph in use (the one the last
+ * air_solve_batch or air_solve_batch_host call ran; the paper has no
+ * counterpart): its number of chains (1 or 2) and the kernels
  * one run of it launches (one per grouped phase launch, two per tensor-core
  * filter application).  Either pointer may be NULL, not both.
  * AIR_ERR_INVALID_ARG if no batch graph exists yet. */

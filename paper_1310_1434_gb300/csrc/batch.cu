@@ -15,6 +15,8 @@
 #include <cmath>
 #include <climits>
 #include <cstring>
+#include <iterator>
+#include <list>
 #include <map>
 #include <mutex>
 #include <vector>
@@ -36,50 +38,55 @@ constexpr int TC_SIDE = 8;
 // other's.  Whether that pays depends on the launches (chains of short
 // launches gain, chains of long ones slow each other down), so the first
 // call of a batch times the one-chain and the two-chain graph and keeps the
-// faster.  A batch whose backprojector phase takes more than CHAIN_WAVES
-// waves of the device is not tried in two chains.
+// faster; later batches of the same shapes take the same form.  A batch whose
+// backprojector phase takes more than CHAIN_WAVES waves of the device is not
+// tried in two chains.
 constexpr int CHAINS = 2;
 constexpr double CHAIN_WAVES = 64.0;
+// Graphs kept for the compositions used last, and chain choices for the
+// shapes seen last: a program that alternates between a few sets of plans
+// replays each one's graph (8 slices of 512^2, 30 x 8: building a graph and
+// trying both forms took two to four runs of the batch).  A graph goes with
+// the first of its plans that is destroyed.
+constexpr size_t GRAPHS_MAX = 8, CHOICES_MAX = 64;
 
-struct BatchGraph {
-    std::vector<uintptr_t> key;
-    cudaStream_t cap = nullptr;     // private stream the graph is captured on
+// Streams and events the graphs are captured on.
+struct Capture {
+    cudaStream_t cap = nullptr;        // private stream the graph is captured on
     cudaStream_t chain[CHAINS] = {};   // chain 0 is cap
     cudaEvent_t start = nullptr, done[CHAINS] = {};
     cudaStream_t side[TC_SIDE] = {};
     cudaEvent_t fork = nullptr, join[TC_SIDE] = {};
+};
+
+struct BatchGraph {
+    std::vector<uintptr_t> key;
+    std::vector<uintptr_t> plan_ids;
+    int device = 0;
     cudaGraphExec_t exec = nullptr;
     char *dmem = nullptr;
     BatchCtl *ctl = nullptr;
     std::vector<const air_plan *> tc_plans;   // plans whose status is checked after a run
-    int chains = 1;                 // of the grouped graph in use
+    int chains = 1;                 // of the grouped graph
     long long kernels = 0;          // kernels one run of it launches
 };
 
 std::mutex g_batch_mu;
-BatchGraph g_grouped, g_persistent;
+std::map<int, Capture> g_capture;             // by device
+std::list<BatchGraph> g_grouped;              // most recently used first
+std::map<std::vector<uintptr_t>, int> g_choice;   // chains of a batch's shapes
+BatchGraph g_persistent;
 
 void release(BatchGraph &b) {
     if (b.exec) cudaGraphExecDestroy(b.exec);
     if (b.dmem) cudaFree(b.dmem);
-    BatchGraph keep;   // the capture streams and events outlive a graph
-    keep.cap = b.cap;
-    keep.fork = b.fork;
-    keep.start = b.start;
-    for (int c = 0; c < CHAINS; ++c) {
-        keep.chain[c] = b.chain[c];
-        keep.done[c] = b.done[c];
-    }
-    for (int i = 0; i < TC_SIDE; ++i) {
-        keep.side[i] = b.side[i];
-        keep.join[i] = b.join[i];
-    }
-    b = keep;
+    b = BatchGraph();
 }
 
-cudaError_t make_side_streams(BatchGraph &b) {
+cudaError_t make_capture(Capture &b) {
     cudaError_t e = cudaSuccess;
-    if (!b.fork) e = cudaEventCreateWithFlags(&b.fork, cudaEventDisableTiming);
+    if (!b.cap) e = cudaStreamCreateWithFlags(&b.cap, cudaStreamNonBlocking);
+    if (e == cudaSuccess && !b.fork) e = cudaEventCreateWithFlags(&b.fork, cudaEventDisableTiming);
     if (e == cudaSuccess && !b.start) e = cudaEventCreateWithFlags(&b.start, cudaEventDisableTiming);
     for (int c = 1; c < CHAINS && e == cudaSuccess; ++c) {
         if (!b.chain[c]) e = cudaStreamCreateWithFlags(&b.chain[c], cudaStreamNonBlocking);
@@ -89,6 +96,7 @@ cudaError_t make_side_streams(BatchGraph &b) {
         if (!b.side[i]) e = cudaStreamCreateWithFlags(&b.side[i], cudaStreamNonBlocking);
         if (e == cudaSuccess && !b.join[i]) e = cudaEventCreateWithFlags(&b.join[i], cudaEventDisableTiming);
     }
+    b.chain[0] = b.cap;
     return e;
 }
 
@@ -96,11 +104,15 @@ struct Batch {
     std::vector<SliceDesc> slices;
     std::vector<std::vector<Phase>> progs;
     size_t nphases = 0;
-    std::vector<uintptr_t> key;
+    int device = 0;
+    std::vector<uintptr_t> key;     // plans, their configuration and programs
+    std::vector<uintptr_t> shape;   // the same with geometries in place of plans
+    std::vector<uintptr_t> data;    // sinograms, images and weights
+    std::vector<uintptr_t> ids;     // of the plans
 };
 
 air_status prepare(int n, air_plan *const *plans, const float *const *Y, const float *lambda, const float *mu,
-                   const int *n_outer, const int *n_cg, float *const *X, cudaStream_t st, bool allow_tc, Batch *B) {
+                   const int *n_outer, const int *n_cg, float *const *X, bool allow_tc, Batch *B) {
     if (n < 1 || n > 4096) return fail(AIR_ERR_INVALID_ARG, "n must be in 1..4096");
     if (!plans || !Y || !lambda || !mu || !n_outer || !n_cg || !X)
         return fail(AIR_ERR_INVALID_ARG, "NULL array argument");
@@ -120,16 +132,27 @@ air_status prepare(int n, air_plan *const *plans, const float *const *Y, const f
         B->progs[i] = solve_program(n_outer[i], n_cg[i], tc, plans[i]->desc.orb != 0);
         B->nphases = std::max(B->nphases, B->progs[i].size());
     }
-    int dev = 0;
-    cudaGetDevice(&dev);
-    B->key.push_back((uintptr_t)dev);
-    B->key.push_back((uintptr_t)st);
+    cudaGetDevice(&B->device);
+    B->key.push_back((uintptr_t)B->device);
+    B->shape.push_back((uintptr_t)B->device);
+    auto bits = [](double v) {
+        uint64_t u;
+        std::memcpy(&u, &v, 8);
+        return (uintptr_t)u;
+    };
     for (int i = 0; i < n; ++i) {
-        uint32_t lb, mb;
-        std::memcpy(&lb, &lambda[i], 4);
-        std::memcpy(&mb, &mu[i], 4);
-        B->key.insert(B->key.end(), {(uintptr_t)plans[i], (uintptr_t)Y[i], (uintptr_t)X[i], (uintptr_t)lb,
-                                     (uintptr_t)mb, (uintptr_t)n_outer[i], (uintptr_t)n_cg[i]});
+        const SliceDesc &d = B->slices[i];
+        const air_geometry &g = plans[i]->geom;
+        B->ids.push_back((uintptr_t)plans[i]->id);
+        B->key.push_back((uintptr_t)plans[i]->id);
+        B->shape.insert(B->shape.end(), {(uintptr_t)g.n, (uintptr_t)g.n_views, (uintptr_t)g.n_bins, bits(g.pixel_mm),
+                                         bits(g.dso_mm), bits(fan_pitch(g)), bits(g.beta0), bits(g.arc),
+                                         (uintptr_t)g.filter, (uintptr_t)g.precision});
+        const uintptr_t how[] = {(uintptr_t)n_outer[i], (uintptr_t)n_cg[i], (uintptr_t)d.fwd_vpb, (uintptr_t)d.bwd_parts,
+                                 (uintptr_t)d.orb_splits};
+        B->key.insert(B->key.end(), std::begin(how), std::end(how));
+        B->shape.insert(B->shape.end(), std::begin(how), std::end(how));
+        B->data.insert(B->data.end(), {(uintptr_t)Y[i], (uintptr_t)X[i], bits(lambda[i]), bits(mu[i])});
     }
     return AIR_OK;
 }
@@ -197,7 +220,7 @@ void plan_chains(const Batch &B, int n, int nch, std::vector<Task> &tasks, std::
 // Captures the chains' launch lists (each chain on a stream of its own with
 // its share of the filter side streams, all joined at the end) and
 // instantiates them into *exec.
-air_status capture_chains(BatchGraph &G, const Batch &B, air_plan *const *plans, int nch,
+air_status capture_chains(Capture &G, const Batch &B, air_plan *const *plans, int nch,
                           const std::vector<Launch> *launches, const SliceDesc *d_slices, const Task *d_tasks,
                           cudaGraphExec_t *exec, long long *kernels) {
     *exec = nullptr;
@@ -205,7 +228,6 @@ air_status capture_chains(BatchGraph &G, const Batch &B, air_plan *const *plans,
     cudaError_t e = cudaStreamBeginCapture(G.cap, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return fail(AIR_ERR_CUDA, std::string("batch set-up: ") + cudaGetErrorString(e));
     const cudaStream_t cs = G.cap;
-    G.chain[0] = cs;
     cudaError_t le = cudaEventRecord(G.start, cs);
     std::string tc_msg;
     for (int c = 0; c < nch && le == cudaSuccess && tc_msg.empty(); ++c) {
@@ -231,9 +253,9 @@ air_status capture_chains(BatchGraph &G, const Batch &B, air_plan *const *plans,
             for (size_t q = li; q < end && le == cudaSuccess && tc_msg.empty(); ++q) {
                 const Launch &T = ls[q];
                 const SliceDesc &sd = B.slices[T.slice];
-                const float *src = T.arg == RSRC_Y ? sd.y : sd.z;
-                if (ramp_tc_apply(plans[T.slice], src, sd.zc, sd.cg, T.arg == RSRC_Z,
-                                  G.side[s0 + (int)((q - li) % nside)]) != AIR_OK)
+                // the measured sinogram changes from call to call: through the descriptor
+                if (ramp_tc_apply(plans[T.slice], sd.z, T.arg == RSRC_Y ? d_slices + T.slice : nullptr, sd.zc, sd.cg,
+                                  T.arg == RSRC_Z, G.side[s0 + (int)((q - li) % nside)]) != AIR_OK)
                     tc_msg = air_last_error();
                 *kernels += 2;   // the split and the tensor-core product
             }
@@ -286,104 +308,126 @@ extern "C" air_status air_solve_batch(int n, air_plan *const *plans, const float
                                       air_stream stream) {
     const cudaStream_t st = (cudaStream_t)stream;
     Batch B;
-    air_status s = prepare(n, plans, Y, lambda, mu, n_outer, n_cg, X, st, true, &B);
+    air_status s = prepare(n, plans, Y, lambda, mu, n_outer, n_cg, X, true, &B);
     if (s != AIR_OK) return s;
     std::lock_guard<std::mutex> lock(g_batch_mu);
-    BatchGraph &G = g_grouped;
-    if (G.key != B.key || !G.exec) {
+    cudaError_t e = cudaSuccess;
+    const size_t b_slices = align_up(n * sizeof(SliceDesc), 256);
+    // this call's descriptors, ahead of the graph on the caller's stream
+    auto describe = [&](BatchGraph &G) {
+        return cudaMemcpyAsync(G.dmem, B.slices.data(), n * sizeof(SliceDesc), cudaMemcpyHostToDevice, st);
+    };
+    for (auto it = g_grouped.begin(); it != g_grouped.end(); ++it) {
+        if (it->key != B.key) continue;
+        g_grouped.splice(g_grouped.begin(), g_grouped, it);
+        BatchGraph &G = g_grouped.front();
+        e = describe(G);
+        if (e != cudaSuccess) return fail(AIR_ERR_CUDA, std::string("batch set-up: ") + cudaGetErrorString(e));
+        return run_cached(G, st);
+    }
+    // one chain, and two chains where the batch is small enough for them to
+    // pay (see CHAINS)
+    int nch = std::min(CHAINS, n);
+    {
+        double waves = 0.0;
+        for (int i = 0; i < n; ++i) {
+            const int op = B.slices[i].orb ? OP_ORB_BWD : OP_BWD;
+            const int cap = group_bwd_capacity(op, tile_smem(B.slices[i], op));
+            if (cap <= 0) nch = 1;
+            else waves += (double)tiles_of(B.slices[i], op) / cap;
+        }
+        if (waves > CHAIN_WAVES) nch = 1;
+    }
+    const auto known = g_choice.find(B.shape);
+    const int forms = known == g_choice.end() ? (nch > 1 ? 2 : 1) : 1;     // graphs to try
+    if (known != g_choice.end()) nch = known->second;
+    std::vector<Task> tasks;
+    std::vector<Launch> one[1], many[CHAINS];
+    if (forms > 1 || nch == 1) plan_chains(B, n, 1, tasks, one);
+    if (nch > 1) plan_chains(B, n, nch, tasks, many);
+    BatchGraph G;
+    G.device = B.device;
+    const size_t b_tasks = align_up(std::max<size_t>(tasks.size(), 1) * sizeof(Task), 256);
+    if (cudaMalloc(&G.dmem, b_slices + b_tasks) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(AIR_ERR_OOM, "batch table allocation failed");
+    }
+    SliceDesc *d_slices = (SliceDesc *)G.dmem;
+    Task *d_tasks = (Task *)(G.dmem + b_slices);
+    // captured on a private stream (the caller's may be the legacy default
+    // stream, which cannot be captured); launched on the caller's stream
+    Capture &C = g_capture[B.device];
+    e = make_capture(C);
+    if (e == cudaSuccess) e = describe(G);
+    if (e == cudaSuccess && !tasks.empty())
+        e = cudaMemcpy(d_tasks, tasks.data(), tasks.size() * sizeof(Task), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
         release(G);
-        // one chain, and two chains where the batch is small enough for them
-        // to pay (see CHAINS)
-        int nch = std::min(CHAINS, n);
-        {
-            long long bwd_tiles = 0;
-            size_t bwd_smem = 0;
-            for (int i = 0; i < n; ++i) {
-                bwd_tiles += tiles_of(B.slices[i], OP_BWD);
-                bwd_smem = std::max(bwd_smem, tile_smem(B.slices[i], OP_BWD));
-            }
-            const int cap = group_bwd_capacity(bwd_smem);
-            if (cap <= 0 || (double)bwd_tiles > CHAIN_WAVES * cap) nch = 1;
-        }
-        std::vector<Task> tasks;
-        std::vector<Launch> one[1], many[CHAINS];
-        plan_chains(B, n, 1, tasks, one);
-        if (nch > 1) plan_chains(B, n, nch, tasks, many);
-        const size_t b_slices = align_up(n * sizeof(SliceDesc), 256);
-        const size_t b_tasks = align_up(std::max<size_t>(tasks.size(), 1) * sizeof(Task), 256);
-        if (cudaMalloc(&G.dmem, b_slices + b_tasks) != cudaSuccess) {
-            cudaGetLastError();
-            G.dmem = nullptr;
-            return fail(AIR_ERR_OOM, "batch table allocation failed");
-        }
-        SliceDesc *d_slices = (SliceDesc *)G.dmem;
-        Task *d_tasks = (Task *)(G.dmem + b_slices);
-        cudaError_t e = cudaMemcpy(d_slices, B.slices.data(), n * sizeof(SliceDesc), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess && !tasks.empty())
-            e = cudaMemcpy(d_tasks, tasks.data(), tasks.size() * sizeof(Task), cudaMemcpyHostToDevice);
-        // captured on a private stream (the caller's may be the legacy default
-        // stream, which cannot be captured); launched on the caller's stream
-        if (e == cudaSuccess && !G.cap) e = cudaStreamCreateWithFlags(&G.cap, cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = make_side_streams(G);
-        if (e != cudaSuccess) {
-            release(G);
-            return fail(AIR_ERR_CUDA, std::string("batch set-up: ") + cudaGetErrorString(e));
-        }
-        cudaGraphExec_t x1 = nullptr, xn = nullptr;
-        long long k1 = 0, kn = 0;
-        s = capture_chains(G, B, plans, 1, one, d_slices, d_tasks, &x1, &k1);
-        if (s == AIR_OK && nch > 1) s = capture_chains(G, B, plans, nch, many, d_slices, d_tasks, &xn, &kn);
-        if (s != AIR_OK) {
-            if (x1) cudaGraphExecDestroy(x1);
-            release(G);
-            return s;
-        }
-        G.key = B.key;
-        for (int i = 0; i < n; ++i)
-            if (plans[i]->tc) G.tc_plans.push_back(plans[i]);
-        G.chains = 1;
-        G.kernels = k1;
-        if (!xn) {
-            G.exec = x1;
-        } else {
-            // timed runs of both forms on the caller's stream (both uploaded
-            // first, so neither run pays for it): one of each, and when they
-            // are within 3 % one more of each in the other order; the faster
-            // form is kept.  The forms compute the same results, so the last
-            // run's output is this call's.
-            cudaEvent_t ev[3] = {};
-            for (int k = 0; k < 3 && e == cudaSuccess; ++k) e = cudaEventCreate(&ev[k]);
-            if (e == cudaSuccess) e = cudaGraphUpload(x1, st);
-            if (e == cudaSuccess) e = cudaGraphUpload(xn, st);
-            float tn = 0.f, t1 = 0.f;
-            auto pair = [&](cudaGraphExec_t a, float *ta, cudaGraphExec_t b, float *tb) {
-                float da = 0.f, db = 0.f;
-                if (e == cudaSuccess) e = cudaEventRecord(ev[0], st);
-                if (e == cudaSuccess) e = cudaGraphLaunch(a, st);
-                if (e == cudaSuccess) e = cudaEventRecord(ev[1], st);
-                if (e == cudaSuccess) e = cudaGraphLaunch(b, st);
-                if (e == cudaSuccess) e = cudaEventRecord(ev[2], st);
-                if (e == cudaSuccess) e = cudaEventSynchronize(ev[2]);
-                if (e == cudaSuccess) e = cudaEventElapsedTime(&da, ev[0], ev[1]);
-                if (e == cudaSuccess) e = cudaEventElapsedTime(&db, ev[1], ev[2]);
-                *ta += da;
-                *tb += db;
-            };
-            pair(xn, &tn, x1, &t1);
-            if (e == cudaSuccess && std::fabs(tn - t1) < 0.03f * std::min(tn, t1)) pair(x1, &t1, xn, &tn);
-            for (int k = 0; k < 3; ++k)
-                if (ev[k]) cudaEventDestroy(ev[k]);
-            G.exec = (e == cudaSuccess && tn < t1) ? xn : x1;
-            cudaGraphExecDestroy(G.exec == xn ? x1 : xn);
-            if (G.exec == xn) {
-                G.chains = nch;
-                G.kernels = kn;
-            }
-            if (e != cudaSuccess) return fail(AIR_ERR_CUDA, std::string("batch solve: ") + cudaGetErrorString(e));
-            return finish_run(G, st);
+        return fail(AIR_ERR_CUDA, std::string("batch set-up: ") + cudaGetErrorString(e));
+    }
+    cudaGraphExec_t x1 = nullptr, xn = nullptr;
+    long long k1 = 0, kn = 0;
+    if (forms > 1 || nch == 1) s = capture_chains(C, B, plans, 1, one, d_slices, d_tasks, &x1, &k1);
+    if (s == AIR_OK && nch > 1) s = capture_chains(C, B, plans, nch, many, d_slices, d_tasks, &xn, &kn);
+    if (s != AIR_OK) {
+        if (x1) cudaGraphExecDestroy(x1);
+        release(G);
+        return s;
+    }
+    G.key = B.key;
+    G.plan_ids = B.ids;
+    for (int i = 0; i < n; ++i)
+        if (plans[i]->tc) G.tc_plans.push_back(plans[i]);
+    bool first = true;              // the run below was not made by the trial
+    G.exec = x1 ? x1 : xn;
+    if (x1 && xn) {
+        // timed runs of both forms on the caller's stream (both uploaded
+        // first, so neither run pays for it): one of each, and when they are
+        // within 3 % one more of each in the other order; the faster form is
+        // kept.  The forms compute the same results, so the last run's output
+        // is this call's.
+        cudaEvent_t ev[3] = {};
+        for (int k = 0; k < 3 && e == cudaSuccess; ++k) e = cudaEventCreate(&ev[k]);
+        if (e == cudaSuccess) e = cudaGraphUpload(x1, st);
+        if (e == cudaSuccess) e = cudaGraphUpload(xn, st);
+        float tn = 0.f, t1 = 0.f;
+        auto pair = [&](cudaGraphExec_t a, float *ta, cudaGraphExec_t b, float *tb) {
+            float da = 0.f, db = 0.f;
+            if (e == cudaSuccess) e = cudaEventRecord(ev[0], st);
+            if (e == cudaSuccess) e = cudaGraphLaunch(a, st);
+            if (e == cudaSuccess) e = cudaEventRecord(ev[1], st);
+            if (e == cudaSuccess) e = cudaGraphLaunch(b, st);
+            if (e == cudaSuccess) e = cudaEventRecord(ev[2], st);
+            if (e == cudaSuccess) e = cudaEventSynchronize(ev[2]);
+            if (e == cudaSuccess) e = cudaEventElapsedTime(&da, ev[0], ev[1]);
+            if (e == cudaSuccess) e = cudaEventElapsedTime(&db, ev[1], ev[2]);
+            *ta += da;
+            *tb += db;
+        };
+        pair(xn, &tn, x1, &t1);
+        if (e == cudaSuccess && std::fabs(tn - t1) < 0.03f * std::min(tn, t1)) pair(x1, &t1, xn, &tn);
+        for (int k = 0; k < 3; ++k)
+            if (ev[k]) cudaEventDestroy(ev[k]);
+        G.exec = (e == cudaSuccess && tn < t1) ? xn : x1;
+        cudaGraphExecDestroy(G.exec == xn ? x1 : xn);
+        first = false;
+        if (e == cudaSuccess) {
+            if (g_choice.size() >= CHOICES_MAX) g_choice.erase(g_choice.begin());
+            g_choice[B.shape] = G.exec == xn ? nch : 1;
         }
     }
-    return run_cached(G, st);
+    G.chains = G.exec == xn ? nch : 1;
+    G.kernels = G.exec == xn ? kn : k1;
+    if (e != cudaSuccess) {
+        release(G);
+        return fail(AIR_ERR_CUDA, std::string("batch solve: ") + cudaGetErrorString(e));
+    }
+    g_grouped.push_front(G);
+    while (g_grouped.size() > GRAPHS_MAX) {
+        release(g_grouped.back());          // not running: every call waits for its run
+        g_grouped.pop_back();
+    }
+    return first ? run_cached(g_grouped.front(), st) : finish_run(g_grouped.front(), st);
 }
 
 extern "C" air_status air_solve_batch_host(int n, air_plan *const *plans, const float *const *Y_host,
@@ -420,7 +464,7 @@ extern "C" air_status air_solve_batch_persistent(int n, air_plan *const *plans, 
                                                  const int *n_cg, float *const *X, air_stream stream) {
     const cudaStream_t st = (cudaStream_t)stream;
     Batch B;
-    air_status s = prepare(n, plans, Y, lambda, mu, n_outer, n_cg, X, st, false, &B);
+    air_status s = prepare(n, plans, Y, lambda, mu, n_outer, n_cg, X, false, &B);
     if (s != AIR_OK) return s;
     size_t smem = 0;
     bool orb = false;
@@ -433,7 +477,10 @@ extern "C" air_status air_solve_batch_persistent(int n, air_plan *const *plans, 
         std::memcpy(&prog[i * B.nphases], B.progs[i].data(), B.progs[i].size() * sizeof(Phase));
     std::lock_guard<std::mutex> lock(g_batch_mu);
     BatchGraph &G = g_persistent;
-    if (G.key != B.key || !G.exec) {
+    Capture &C = g_capture[B.device];
+    std::vector<uintptr_t> key = B.key;     // this form's descriptors are written with the graph
+    key.insert(key.end(), B.data.begin(), B.data.end());
+    if (G.key != key || !G.exec) {
         release(G);
         const int grid = persistent_grid(smem, orb);
         if (grid <= 0) return fail(AIR_ERR_CUDA, "batch set-up: no co-resident grid for the persistent kernel");
@@ -476,17 +523,19 @@ extern "C" air_status air_solve_batch_persistent(int n, air_plan *const *plans, 
         if (e == cudaSuccess)
             e = cudaMemcpy(d_pb, phase_base.data(), phase_base.size() * sizeof(unsigned long long),
                            cudaMemcpyHostToDevice);
-        if (e == cudaSuccess && !G.cap) e = cudaStreamCreateWithFlags(&G.cap, cudaStreamNonBlocking);
-        if (e == cudaSuccess) e = cudaStreamBeginCapture(G.cap, cudaStreamCaptureModeThreadLocal);
+        if (e == cudaSuccess) e = make_capture(C);
+        if (e == cudaSuccess) e = cudaStreamBeginCapture(C.cap, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) {
             release(G);
             return fail(AIR_ERR_CUDA, std::string("batch set-up: ") + cudaGetErrorString(e));
         }
-        cudaError_t le = cudaMemsetAsync(G.ctl, 0, sizeof(BatchCtl), G.cap);
+        cudaError_t le = cudaMemsetAsync(G.ctl, 0, sizeof(BatchCtl), C.cap);
         if (le == cudaSuccess)
-            le = launch_persistent(d_slices, n, d_prog, (int)B.nphases, d_tb, d_pb, G.ctl, grid, smem, orb, G.cap);
-        if ((s = end_capture(G, G.cap, le)) != AIR_OK) return s;
-        G.key = B.key;
+            le = launch_persistent(d_slices, n, d_prog, (int)B.nphases, d_tb, d_pb, G.ctl, grid, smem, orb, C.cap);
+        if ((s = end_capture(G, C.cap, le)) != AIR_OK) return s;
+        G.key = key;
+        G.plan_ids = B.ids;
+        G.device = B.device;
     }
     return run_cached(G, st);
 }
@@ -494,8 +543,25 @@ extern "C" air_status air_solve_batch_persistent(int n, air_plan *const *plans, 
 extern "C" air_status air_batch_graph_info(int *chains, int64_t *kernels) {
     if (!chains && !kernels) return fail(AIR_ERR_INVALID_ARG, "both outputs are NULL");
     std::lock_guard<std::mutex> lock(g_batch_mu);
-    if (!g_grouped.exec) return fail(AIR_ERR_INVALID_ARG, "no batch graph has been built");
-    if (chains) *chains = g_grouped.chains;
-    if (kernels) *kernels = (int64_t)g_grouped.kernels;
+    if (g_grouped.empty()) return fail(AIR_ERR_INVALID_ARG, "no batch graph has been built");
+    if (chains) *chains = g_grouped.front().chains;
+    if (kernels) *kernels = (int64_t)g_grouped.front().kernels;
     return AIR_OK;
+}
+
+// Drops the graphs that run a plan which is about to be destroyed.
+void air::batch_forget(uint64_t plan_id) {
+    std::lock_guard<std::mutex> lock(g_batch_mu);
+    auto has = [&](const BatchGraph &G) {
+        return std::find(G.plan_ids.begin(), G.plan_ids.end(), (uintptr_t)plan_id) != G.plan_ids.end();
+    };
+    for (auto it = g_grouped.begin(); it != g_grouped.end();) {
+        if (has(*it)) {
+            release(*it);
+            it = g_grouped.erase(it);
+        } else {
+            ++it;
+        }
+    }
+    if (has(g_persistent)) release(g_persistent);
 }

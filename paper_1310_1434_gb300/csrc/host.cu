@@ -2,6 +2,7 @@
 // checking, the stand-alone operator calls and the solver programs.
 #include <cmath>
 #include <algorithm>
+#include <atomic>
 #include <cstring>
 #include <map>
 #include <memory>
@@ -696,6 +697,8 @@ extern "C" air_status air_plan_create(const air_geometry *geom, air_plan **out) 
     if (st != AIR_OK) return st;
     air_plan *P = new (std::nothrow) air_plan();
     if (!P) return fail(AIR_ERR_OOM, "host allocation failed");
+    static std::atomic<uint64_t> ids{0};
+    P->id = ++ids;
     st = plan_build(geom, P);
     if (st != AIR_OK) {
         delete P;
@@ -707,6 +710,7 @@ extern "C" air_status air_plan_create(const air_geometry *geom, air_plan **out) 
 
 extern "C" air_status air_plan_destroy(air_plan *P) {
     if (!P) return AIR_OK;
+    batch_forget(P->id);
     ramp_tc_destroy(P);
     if (P->mem) cudaFree(P->mem);
     delete P;
@@ -775,7 +779,7 @@ namespace air {
 air_status apply_filter(const air_plan *P, const SliceDesc &base, const float *src, float *dst,
                         cudaStream_t st) {
     if (P->geom.precision == AIR_PREC_BF16X3 && P->geom.filter == AIR_FILTER_RAMLAK)
-        return ramp_tc_apply(P, src, dst, base.cg, 0, st);
+        return ramp_tc_apply(P, src, nullptr, dst, base.cg, 0, st);
     SliceDesc s = base;
     s.ext_in = src;
     s.ext_out = dst;
@@ -949,7 +953,7 @@ air_status run_program_single(const air_plan *P, const SliceDesc &s, const std::
     for (const Phase &ph : prog) {
         if (ph.op == OP_RAMP_TC) {
             const float *src = ph.arg == RSRC_Y ? s.y : s.z;
-            TRY(ramp_tc_apply(P, src, s.zc, s.cg, ph.arg == RSRC_Z, st));
+            TRY(ramp_tc_apply(P, src, nullptr, s.zc, s.cg, ph.arg == RSRC_Z, st));
         } else {
             CUDA_TRY(launch_op(ph.op, s, ph.arg, st));
         }

@@ -10,6 +10,7 @@
 // A plan: geometry tables + solver workspace of one slice geometry.
 struct air_plan {
     air_geometry geom{};
+    uint64_t id = 0;           // of this plan, never used again in the process
     int device = 0;
     air::SliceDesc desc{};     // tables and workspace pointers
     char *mem = nullptr;       // the one allocation desc points into
@@ -42,6 +43,7 @@ int choose_bwd_parts(const SliceDesc &s);
 // there is more than one, their sum with the mode's epilogue.
 cudaError_t launch_backprojection(const SliceDesc &s, int mode, cudaStream_t st);
 air_status autotune(air_plan *P);
+void batch_forget(uint64_t plan_id);
 size_t plan_bytes_estimate(const air_geometry &g);
 air_status apply_filter(const air_plan *P, const SliceDesc &base, const float *src, float *dst,
                         cudaStream_t st);

@@ -10,9 +10,9 @@ namespace air {
 // One op over all tiles of one slice.
 cudaError_t launch_op(int op, const SliceDesc &s, int arg, cudaStream_t st);
 
-// Blocks of the grouped backprojector resident on the current device at
-// once, for the given dynamic shared memory (0 on failure).
-int group_bwd_capacity(size_t smem);
+// Blocks of a grouped backprojector (OP_BWD or OP_ORB_BWD) resident on the
+// current device at once, for the given dynamic shared memory (0 on failure).
+int group_bwd_capacity(int op, size_t smem);
 
 // One op over the tiles of many slices in one launch (tasks all of that op).
 cudaError_t launch_group(int op, const SliceDesc *d_slices, const Task *d_tasks, int ntasks, int total_tiles,

@@ -159,14 +159,16 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *out) {
 // ------------------------------------------------------------ kernels
 // One view per block: split the row into three BF16 pieces (GEMM operand A)
 // and write the near-band part of Z.
-__global__ void __launch_bounds__(256) k_split_near(const float *__restrict__ Y, float *__restrict__ Z,
+// measured: a slice descriptor whose sinogram y takes Y's place, or nullptr.
+__global__ void __launch_bounds__(256) k_split_near(const float *__restrict__ Y, const SliceDesc *__restrict__ measured,
+                                                    float *__restrict__ Z,
                                                     __nv_bfloat16 *__restrict__ A, const float *__restrict__ taps,
                                                     float near_diag, int nb, int kp, const CgState *cg,
                                                     int respect_stop) {
     extern __shared__ __align__(16) float P[];    // [NEAR + nb + NEAR], zero padded
     if (respect_stop && cg->stop) return;
     const int v = blockIdx.x;
-    const float *y = Y + (size_t)v * nb;
+    const float *y = (measured ? measured->y : Y) + (size_t)v * nb;
     for (int k = threadIdx.x; k < nb + 2 * NEAR; k += blockDim.x) {
         const int i = k - NEAR;
         P[k] = (i >= 0 && i < nb) ? y[i] : 0.f;
@@ -475,12 +477,12 @@ void ramp_tc_destroy(air_plan *P) {
     P->tc_bytes = 0;
 }
 
-air_status ramp_tc_apply(const air_plan *P, const float *src, float *dst, const CgState *cg, int respect_stop,
+air_status ramp_tc_apply(const air_plan *P, const float *src, const SliceDesc *measured, float *dst, const CgState *cg, int respect_stop,
                          cudaStream_t st) {
     const TcRes *R = static_cast<const TcRes *>(P->tc);
     if (!R) return fail(AIR_ERR_INVALID_ARG, "plan has no tensor-core filter");
     const int V = P->geom.n_views, nb = P->geom.n_bins;
-    k_split_near<<<V, 256, (nb + 2 * NEAR) * sizeof(float), st>>>(src, dst, R->a, R->near_taps, R->near_diag, nb,
+    k_split_near<<<V, 256, (nb + 2 * NEAR) * sizeof(float), st>>>(src, measured, dst, R->a, R->near_taps, R->near_diag, nb,
                                                                    R->kp, cg, respect_stop);
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) {

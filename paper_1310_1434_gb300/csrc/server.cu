@@ -337,7 +337,7 @@ air_status enqueue_step(air_server *S) {
             Request *r = it->second[0];
             const SliceDesc &sd = S->h_slices[r->slot];
             const int arg = r->prog[r->pc].arg;
-            st1 = ramp_tc_apply(r->plan, arg == RSRC_Y ? sd.y : sd.z, sd.zc, sd.cg, arg == RSRC_Z, S->stream);
+            st1 = ramp_tc_apply(r->plan, arg == RSRC_Y ? sd.y : sd.z, nullptr, sd.zc, sd.cg, arg == RSRC_Z, S->stream);
         }
         if (st1 != AIR_OK) return st1;
         return finish_step(S, k);
@@ -359,7 +359,7 @@ air_status enqueue_step(air_server *S) {
         Request *r = it->second[i];
         const SliceDesc &sd = S->h_slices[r->slot];
         const int arg = r->prog[r->pc].arg;
-        st = ramp_tc_apply(r->plan, arg == RSRC_Y ? sd.y : sd.z, sd.zc, sd.cg, arg == RSRC_Z, S->side[q++ % nside]);
+        st = ramp_tc_apply(r->plan, arg == RSRC_Y ? sd.y : sd.z, nullptr, sd.zc, sd.cg, arg == RSRC_Z, S->side[q++ % nside]);
     }
     for (int k2 = 0; k2 < nside; ++k2) {       // join even after a failure: the stream stays ordered
         cudaEventRecord(S->join[k2], S->side[k2]);
