@@ -39,6 +39,8 @@ enum Op : int {
     OP_AXPY,       // q = x + step r            (forward step of Eq. 6, r = A'^T(Y - A x))
     OP_PROX,       // x = W^T S_tau(W q)        (framelet proximal step)
     OP_FBP,        // ext_out = fan-beam FBP weighted backprojection of zc
+    OP_FBP_PACK,   // the filtered views of an orbit side by side      (before OP_FBP_ORB)
+    OP_FBP_ORB,    // per-symmetry parts of the FBP backprojection     (OP_BWD_FIN sums them)
     OP_RESTART,    // CG restart of an outer step: r = rhs0 (arg -1) or r += mu (g_new - g_old); p = r; rho
     OP_ORB_PACK,   // frames of src for the orbit projector   (in place of OP_TRANSPOSE; arg = FwdSrc)
     OP_ORB_FWD,    // z = A src by orbits                      (in place of OP_FWD; arg = FwdSrc)
@@ -126,6 +128,7 @@ struct __align__(16) OrbSeg {
     int pad[2];
 };
 constexpr int BWD_T = 32;         // side of a backprojector pixel tile
+constexpr int FBP_NONE = 0x7fffffff;
 constexpr int ORB_MIN_N = 64;     // smallest image side the orbit kernels take
 constexpr int ORB_VIEWS = 8;      // base views whose projector warps follow one another
 constexpr int ORB_RAYS = 96;      // most rays of a segment in a backprojector tile
@@ -157,6 +160,12 @@ struct SliceDesc {
     float dso_px;        // source-isocentre distance, pixels
     float inv_dg, inv_dg_lo, jmid;   // 1 / fan pitch (high and low parts), (nb - 1) / 2
     float fbp_scale;     // dbeta / dx^2
+    // FBP over orbits of views (orbit.h; fbp_nf = symmetries of the scan, 0: too few)
+    int fbp_nf, fbp_nbase, fbp_splits;
+    int fbp_code[8];     // symmetry of slot f
+    const float2 *fbp_c; // [nbase] central-ray direction of each base view
+    const int *fbp_view; // [nbase][8] view of slot f, ~view with its bins reversed, FBP_NONE: a view already there
+    float4 *fbp_q;       // [nbase][nb + 4][fbp_nf / 4] packed views, two zero bins at each end
     // solver state (plan-owned workspace)
     float *x, *r, *p, *q, *rhs0, *g;   // n*n
     float *g2;                         // n*n: g of the previous outer step (g is double-buffered)
@@ -257,6 +266,8 @@ __host__ __device__ inline int tiles_of(const SliceDesc &s, int op) {
     case OP_BWD: return tiles_bwd(s);
     case OP_CG_A: case OP_CG_B: case OP_ZERO: case OP_BWD_FIN: case OP_AXPY: case OP_RESTART: return tiles_vec(s);
     case OP_TRANSPOSE: return tiles_tr(s);
+    case OP_FBP_PACK: return (int)(((size_t)s.fbp_nbase * (s.nb + 4) + AIR_THREADS - 1) / AIR_THREADS);
+    case OP_FBP_ORB: return tiles_shr(s) * s.fbp_splits;
     case OP_ORB_PACK: return 2 * tiles_tr(s);
     case OP_ORB_FWD: return tiles_orb_fwd(s);
     case OP_ORB_ZPACK: return s.orb_nseg * orb_zchunks(s);

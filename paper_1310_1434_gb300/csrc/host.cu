@@ -116,6 +116,27 @@ static int choose_orb_ks(int warps, int sms) {
     return ks;
 }
 
+// The FBP backprojection over orbits of views: split until the blocks fill
+// the device about three times (five of 256 threads per SM), within what the
+// part buffer holds of images and, behind them, the packed views; a multiple
+// of eight images for their sum.
+static void choose_fbp(SliceDesc &s, const FbpOrbits &F, float *bpart, int parts_max, int sms) {
+    s.fbp_nf = 0;
+    if (!F.nf) return;
+    const size_t nn = (size_t)s.n * s.n, packed = F.base.size() * (size_t)(s.nb + 4) * F.nf;
+    const int step = 8 / F.nf, most = std::min<int>(8, (int)F.base.size()) / step * step;
+    int splits = std::min(most, (3 * 5 * sms + tiles_shr(s) - 1) / tiles_shr(s) / step * step);
+    splits = std::max(splits, step);
+    while (splits > step && align_up((size_t)splits * F.nf * nn, 4) + packed > (size_t)parts_max * nn) splits -= step;
+    const size_t off = align_up((size_t)splits * F.nf * nn, 4);
+    if (off + packed > (size_t)parts_max * nn) return;
+    s.fbp_nf = F.nf;
+    s.fbp_nbase = (int)F.base.size();
+    s.fbp_splits = splits;
+    for (int f = 0; f < 8; ++f) s.fbp_code[f] = F.code[f];
+    s.fbp_q = reinterpret_cast<float4 *>(bpart + off);
+}
+
 static int sm_count() {
     int sms = 148, dev = 0;
     if (cudaGetDevice(&dev) == cudaSuccess) cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -354,6 +375,8 @@ struct HostTables {
     std::vector<float2> fview;
     float ramp_diag = 0.f, fbp_diag = 0.f;
     OrbitTables orb;
+    FbpOrbits fbp;
+    std::vector<float2> fbp_c;
 };
 
 air_status build_tables(const air_geometry &g, double dg, int ntxy, HostTables &T) {
@@ -476,6 +499,8 @@ air_status build_tables(const air_geometry &g, double dg, int ntxy, HostTables &
     }
     T.fbp_diag = (float)fdiag;
     build_orbits(g, dg, T.orb);
+    build_fbp_orbits(g, T.fbp);
+    for (int v : T.fbp.base) T.fbp_c.push_back(hfview[v]);
     return AIR_OK;
 }
 
@@ -537,6 +562,7 @@ air_status plan_build(const air_geometry *geom, air_plan *P) {
     std::shared_ptr<const HostTables> T;
     if (air_status st = geometry_tables(g, dg, ntxy, &T); st != AIR_OK) return st;
     const OrbitTables &O = T->orb;
+    const FbpOrbits &F = T->fbp;
     const int sms = sm_count();
     // the autotuner may pick up to twice the heuristic's view split; the
     // orbit backprojector's splits write eight images each
@@ -564,6 +590,8 @@ air_status plan_build(const air_geometry *geom, air_plan *P) {
     uint2 *oinfo, *oent;
     uint4 *obray;
     float4 *oz;
+    float2 *fbpc;
+    int *fbpview;
     unsigned *otask;
     int *otile0;
     float4 *ostack;
@@ -586,7 +614,8 @@ air_status plan_build(const air_geometry *geom, air_plan *P) {
         {(void **)&oinfo, O.info.size() * sizeof(uint2)}, {(void **)&oent, O.ent.size() * sizeof(uint2)},
         {(void **)&otask, O.task.size() * sizeof(unsigned)}, {(void **)&otile0, O.tile0.size() * sizeof(int)},
         {(void **)&ostack, nstack * sizeof(float4)}, {(void **)&obray, O.bray.size() * sizeof(uint4)},
-        {(void **)&oz, nz * sizeof(float4)},
+        {(void **)&oz, nz * sizeof(float4)}, {(void **)&fbpc, T->fbp_c.size() * sizeof(float2)},
+        {(void **)&fbpview, F.view.size() * sizeof(int)},
         {(void **)&cg, sizeof(CgState)}, {(void **)&partial, npart * sizeof(double)}};
     size_t total = 0;
     for (auto &pc : pieces) total = align_up(total, 256) + pc.bytes;
@@ -631,6 +660,8 @@ air_status plan_build(const air_geometry *geom, air_plan *P) {
     upload(oent, O.ent.data(), O.ent.size() * sizeof(uint2));
     upload(otask, O.task.data(), O.task.size() * sizeof(unsigned));
     upload(otile0, O.tile0.data(), O.tile0.size() * sizeof(int));
+    upload(fbpc, T->fbp_c.data(), T->fbp_c.size() * sizeof(float2));
+    upload(fbpview, F.view.data(), F.view.size() * sizeof(int));
     upload(obray, O.bray.data(), O.bray.size() * sizeof(uint4));
     if (e == cudaSuccess && nstack) e = cudaMemset(ostack, 0, nstack * sizeof(float4));   // the pad rows stay zero
     if (e == cudaSuccess) e = cudaMemset(cg, 0, sizeof(CgState));
@@ -652,6 +683,9 @@ air_status plan_build(const air_geometry *geom, air_plan *P) {
     s.orb_info = oinfo;
     s.orb_ent = oent;
     s.orb_bray = obray;
+    s.fbp_c = fbpc;
+    s.fbp_view = fbpview;
+    choose_fbp(s, F, bpart, parts_max, sms);
     s.orb_z = oz;
     s.orb_task = otask;
     s.orb_tile0 = otile0;
@@ -1043,7 +1077,16 @@ extern "C" air_status air_fbp(const air_plan *P, const float *Y, float *X, air_s
     CUDA_TRY(launch_op(OP_RAMP, f, RSRC_EXT, st));
     SliceDesc b = P->desc;
     b.ext_out = X;
-    CUDA_TRY(launch_op(OP_FBP, b, 0, st));
+    if (!b.fbp_nf) {
+        CUDA_TRY(launch_op(OP_FBP, b, 0, st));
+        return AIR_OK;
+    }
+    CUDA_TRY(launch_op(OP_FBP_PACK, b, 0, st));
+    CUDA_TRY(launch_op(OP_FBP_ORB, b, 0, st));
+    b.orb = 8;                    // the sum of the orbits' images, scaled
+    b.orb_splits = b.fbp_splits * b.fbp_nf / 8;
+    b.dx = b.fbp_scale;
+    CUDA_TRY(launch_op(OP_BWD_FIN, b, BWD_PLAIN, st));
     return AIR_OK;
 }
 

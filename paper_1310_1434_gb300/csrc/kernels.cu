@@ -55,6 +55,10 @@ __global__ void __launch_bounds__(AIR_THREADS, min_blocks<OP>) k_op(const SliceD
         tile_prox(s, tile, sm);
     } else if constexpr (OP == OP_FBP) {
         tile_fbp(s, tile);
+    } else if constexpr (OP == OP_FBP_PACK) {
+        tile_fbp_pack(s, tile);
+    } else if constexpr (OP == OP_FBP_ORB) {
+        tile_fbp_orb(s, tile);
     } else if constexpr (OP == OP_RESTART) {
         tile_restart(s, arg, tile);
     } else if constexpr (OP == OP_SHRINK) {
@@ -106,6 +110,8 @@ cudaError_t launch_op(int op, const SliceDesc &s, int arg, cudaStream_t st) {
     case OP_AXPY: return launch_one<OP_AXPY>(s, arg, st);
     case OP_PROX: return launch_one<OP_PROX>(s, arg, st);
     case OP_FBP: return launch_one<OP_FBP>(s, arg, st);
+    case OP_FBP_PACK: return launch_one<OP_FBP_PACK>(s, arg, st);
+    case OP_FBP_ORB: return launch_one<OP_FBP_ORB>(s, arg, st);
     case OP_RESTART: return launch_one<OP_RESTART>(s, arg, st);
     case OP_ORB_PACK: return launch_one<OP_ORB_PACK>(s, arg, st);
     case OP_ORB_FWD: return launch_one<OP_ORB_FWD>(s, arg, st);

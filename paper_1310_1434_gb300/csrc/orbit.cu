@@ -61,6 +61,25 @@ int map_view(const Elem &e, int v, int V) { return ((e.sign * v + e.shift) % V +
 
 }  // namespace
 
+void build_fbp_orbits(const air_geometry &g, FbpOrbits &T) {
+    T = FbpOrbits();
+    const std::vector<Elem> G = scan_group(g);
+    if (G.size() != 4 && G.size() != 8) return;
+    const int V = g.n_views;
+    T.nf = (int)G.size();
+    for (int f = 0; f < T.nf; ++f) T.code[f] = code_of(G[f].s);
+    std::vector<char> seen(V, 0);
+    for (int v = 0; v < V; ++v) {
+        if (seen[v]) continue;
+        T.base.push_back(v);
+        for (int f = 0; f < 8; ++f) {
+            const int w = f < T.nf ? map_view(G[f], v, V) : 0;
+            T.view.push_back(f >= T.nf || seen[w] ? FBP_NONE : (G[f].sign < 0 ? ~w : w));
+            if (f < T.nf) seen[w] = 1;
+        }
+    }
+}
+
 int orbit_frames(const air_geometry &g) {
     if (g.n < ORB_MIN_N) return 0;
     const size_t order = scan_group(g).size();

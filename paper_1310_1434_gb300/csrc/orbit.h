@@ -38,6 +38,19 @@ struct OrbitTables {
     std::vector<uint4> bray;          // padded rays: each segment's, then ORB_CAND empty ones
 };
 
+// The views of a full scan grouped by its symmetries, for the analytic
+// reconstruction: what a pixel p takes from base view v, the pixel g p takes
+// from view g v.  Slot f is symmetry code[f]; a mirrored view's bins are
+// reversed; a base view that a mirror takes to itself has each view twice,
+// of which one slot is left empty.
+struct FbpOrbits {
+    int nf = 0;                       // symmetries, 8 or 4 (0: fewer)
+    int code[8] = {};
+    std::vector<int> base;            // base views
+    std::vector<int> view;            // [base][8]: view, ~view (reversed) or FBP_NONE
+};
+void build_fbp_orbits(const air_geometry &g, FbpOrbits &T);
+
 // Frames per orbit of a scan with enough symmetries (8 or 4, else 0).
 int orbit_frames(const air_geometry &g);
 

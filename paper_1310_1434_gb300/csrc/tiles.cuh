@@ -553,20 +553,6 @@ __device__ __forceinline__ void tile_ramp(const SliceDesc &s, int arg, int tile,
 // L cos(gamma') = D + cx x + cy y, which stay accurate in FP32.
 // One thread per pixel, 16 x 16 pixels per block.
 // ======================================================================
-// arctan(u) for |u| <= 0.45 by its Maclaurin (Gregory) series through u^13;
-// the alternating-series remainder is below 0.45^15/15 = 4.2e-7 rad.
-__device__ __forceinline__ float atan_series(float u) {
-    const float w = u * u;
-    float p = 1.f / 13.f;
-    p = fmaf(p, w, -1.f / 11.f);
-    p = fmaf(p, w, 1.f / 9.f);
-    p = fmaf(p, w, -1.f / 7.f);
-    p = fmaf(p, w, 1.f / 5.f);
-    p = fmaf(p, w, -1.f / 3.f);
-    p = fmaf(p, w, 1.f);
-    return u * p;
-}
-
 __device__ __forceinline__ void tile_fbp(const SliceDesc &s, int tile) {
     const int n = s.n, nb = s.nb, tpr = (n + SHR_T - 1) / SHR_T;
     const int ix = (tile % tpr) * SHR_T + (int)threadIdx.x % SHR_T;

@@ -292,9 +292,9 @@ __device__ __forceinline__ void tile_orb_zpack(const SliceDesc &s, int mode, int
     }
 }
 
-// arctan(u) for |u| <= 0.45 (atan_series of the analytic reconstruction), else atanf.
-__device__ __forceinline__ float orb_atan(float u) {
-    if (fabsf(u) > 0.45f) return atanf(u);
+// arctan(u) for |u| <= 0.45 by its Maclaurin (Gregory) series through u^13;
+// the alternating-series remainder is below 0.45^15/15 = 4.2e-7 rad.
+__device__ __forceinline__ float atan_series(float u) {
     const float w = u * u;
     float p = 1.f / 13.f;
     p = fmaf(p, w, -1.f / 11.f);
@@ -305,6 +305,7 @@ __device__ __forceinline__ float orb_atan(float u) {
     p = fmaf(p, w, 1.f);
     return u * p;
 }
+__device__ __forceinline__ float orb_atan(float u) { return fabsf(u) <= 0.45f ? atan_series(u) : atanf(u); }
 
 template <int NF>
 __device__ __forceinline__ void tile_orb_bwd_nf(const SliceDesc &s, int tile, float *sm) {
@@ -443,6 +444,85 @@ __device__ __forceinline__ void tile_orb_bwd(const SliceDesc &s, int mode, int t
     if (mode == BWD_Q && s.cg->stop) return;
     if (s.orb == 8) tile_orb_bwd_nf<8>(s, tile, sm);
     else tile_orb_bwd_nf<4>(s, tile, sm);
+}
+
+// ======================================================================
+// Fan-beam FBP over orbits of views: the fan angle, bin position, weight and
+// distance of a (pixel, base view) pair serve the four or eight pixels and
+// views that the scan's symmetries take it to, whose samples lie side by side
+// (orbit.h, FbpOrbits).  One thread per pixel and split of the base views; its
+// sum for each symmetry goes to an image of its own.
+// ======================================================================
+__device__ __forceinline__ void tile_fbp_pack(const SliceDesc &s, int tile) {
+    const int ld = s.nb + 4;
+    const long long i = (long long)tile * AIR_THREADS + threadIdx.x;
+    if (i >= (long long)s.fbp_nbase * ld) return;
+    const int b = (int)(i / ld), j = (int)(i - (long long)b * ld) - 2;
+    const int *__restrict__ view = s.fbp_view + 8 * b;
+    const bool in = j >= 0 && j < s.nb;
+    for (int p = 0; p < s.fbp_nf / 4; ++p) {
+        float v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int w = __ldg(view + 4 * p + q);
+            v[q] = !in || w == FBP_NONE ? 0.f
+                                        : __ldg(s.zc + (w < 0 ? (size_t)~w * s.nb + (s.nb - 1 - j) : (size_t)w * s.nb + j));
+        }
+        s.fbp_q[(size_t)i * (s.fbp_nf / 4) + p] = make_float4(v[0], v[1], v[2], v[3]);
+    }
+}
+
+template <int NV>
+__device__ __forceinline__ void tile_fbp_orb_nv(const SliceDesc &s, int tile) {
+    const int n = s.n, nb = s.nb, tpr = (n + SHR_T - 1) / SHR_T, nt = tiles_shr(s);
+    const int split = tile / nt, t = tile - split * nt, S = s.fbp_splits;
+    // a warp takes 8 x 4 pixels
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int ix = (t % tpr) * SHR_T + (w & 1) * 8 + (lane & 7), iy = (t / tpr) * SHR_T + (w >> 1) * 4 + (lane >> 3);
+    const float x = (float)ix + 0.5f - s.half_n, y = (float)iy + 0.5f - s.half_n;
+    const unsigned long long minus = pair2(-1.f, -1.f);
+    unsigned long long acc[2 * NV];
+#pragma unroll
+    for (int f = 0; f < 2 * NV; ++f) acc[f] = 0ull;
+    const ulonglong2 *__restrict__ Q = reinterpret_cast<const ulonglong2 *>(s.fbp_q) + 2 * NV;   // bin 0 of view 0
+#pragma unroll 2
+    for (int v = split; v < s.fbp_nbase; v += S) {
+        const float2 c = __ldg(s.fbp_c + v);
+        const float cr = fmaf(c.x, y, -c.y * x);                 // L sin(gamma')
+        const float dt = fmaf(c.x, x, fmaf(c.y, y, s.dso_px));   // L cos(gamma') > 0
+        const float u = cr / dt;
+        const float gp = fabsf(u) <= 0.45f ? atan_series(u) : atan2f(cr, dt);
+        // bin position as in tile_fbp
+        const float tr = floorf(fmaf(gp, s.inv_dg, s.jmid));
+        float wt = fmaf(gp, s.inv_dg, s.jmid - tr);
+        wt = fmaf(gp, s.inv_dg_lo, wt);
+        const int j0 = (int)tr + (wt < 0.f ? -1 : (wt >= 1.f ? 1 : 0));
+        wt = wt < 0.f ? wt + 1.f : (wt >= 1.f ? wt - 1.f : wt);
+        const float r2 = __fdividef(1.f, fmaf(cr, cr, dt * dt));
+        const unsigned long long w2 = pair2(wt, wt), i2 = pair2(r2, r2);
+        // off the detector: onto the zero bins at the row's ends
+        const ulonglong2 *__restrict__ q = Q + ((size_t)v * (nb + 4) + min(max(j0, -2), nb)) * NV;
+#pragma unroll
+        for (int f = 0; f < NV; ++f) {
+            const ulonglong2 a = __ldg(q + f), b = __ldg(q + NV + f);
+            acc[2 * f] = fma2(i2, fma2(w2, fma2(a.x, minus, b.x), a.x), acc[2 * f]);
+            acc[2 * f + 1] = fma2(i2, fma2(w2, fma2(a.y, minus, b.y), a.y), acc[2 * f + 1]);
+        }
+    }
+    if (ix >= n || iy >= n) return;
+#pragma unroll
+    for (int f = 0; f < 4 * NV; ++f) {
+        const int code = s.fbp_code[f];
+        const int a = code & ORB_T ? iy : ix, b = code & ORB_T ? ix : iy;
+        const int px = code & ORB_FX ? n - 1 - a : a, py = code & ORB_FY ? n - 1 - b : b;
+        const float2 r = unpair2(acc[f / 2]);
+        s.bwd_part[(size_t)(split * 4 * NV + f) * n * n + (size_t)py * n + px] = f & 1 ? r.y : r.x;
+    }
+}
+
+__device__ __forceinline__ void tile_fbp_orb(const SliceDesc &s, int tile) {
+    if (s.fbp_nf == 8) tile_fbp_orb_nv<2>(s, tile);
+    else tile_fbp_orb_nv<1>(s, tile);
 }
 
 }  // namespace air

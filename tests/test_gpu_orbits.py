@@ -84,3 +84,21 @@ def test_orbit_solve_matches_oracle(prec):
     air.air_solve(plan, torch.as_tensor(Y, device=DEV), w.lam, w.mu, w.n_outer, w.n_cg, X)
     torch.cuda.synchronize()
     assert rel(X, ref.reshape(X.shape)) <= 1e-4
+
+
+FBP_GEOMS = GEOMS + [inputs.Geometry(33, 2.0, 30, 41), inputs.Geometry(40, 2.0, 26, 50, beta0=math.pi / 26),
+                     inputs.Geometry(17, 3.0, 4, 31), inputs.Geometry(50, 1.1, 24, 64, dso_mm=60.0)]
+
+
+@pytest.mark.parametrize("g", FBP_GEOMS, ids=[f"{g.n}_{g.n_views}_{g.n_bins}" for g in FBP_GEOMS])
+def test_orbit_fbp_matches_oracle(g):
+    # the analytic reconstruction over orbits of views, at the tolerance
+    # derived for the general one (FP32 sum over the views and 2e-5 bins of
+    # interpolation position): 5e-6
+    og = oracle.Geometry(**{k: getattr(g, k) for k in oracle.Geometry.__dataclass_fields__})
+    Y = inputs.ellipse_line_integrals(g, inputs.random_phantom(g, 3, 6, 3)).astype(np.float32)
+    plan = air.Plan(g)
+    X = torch.full((g.n, g.n), float("nan"), device=DEV)
+    air.air_fbp(plan, torch.as_tensor(Y, device=DEV), X)
+    torch.cuda.synchronize()
+    assert rel(X, oracle.fbp(og, Y.astype(np.float64)).reshape(X.shape)) <= 5e-6
