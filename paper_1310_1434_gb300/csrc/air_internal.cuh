@@ -283,6 +283,24 @@ __host__ inline int max_reduce_tiles(const SliceDesc &s) {
     return b > c ? b : c;
 }
 
+// ------------------------------------------------ launch overlap ---------
+// Waits until everything before this kernel on its stream is complete and
+// visible (returns at once where the launch did not ask for overlap).  First in
+// every kernel; only what no kernel writes may be read before it.  A kernel
+// lets the next one's blocks in as its own leave: asking for them earlier
+// (griddepcontrol.launch_dependents at the start) put waiting blocks beside
+// running ones and cost the general pair at 512^2 / 800 views 15 % and the
+// 128^2 solve 15 % of what the overlap gives.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Loads of what other kernels (or earlier phases) write are plain: ordered
+// after grid_wait(), above which the compiler may lift a read-only load
+// (__ldg), and coherent, as the read-only path need not be while this kernel
+// already runs.  __ldg is for the plan's tables.  (As volatile PTX they cost
+// the general projector pair 15 % at 512^2 / 800 views.)
+template <typename T>
+__device__ __forceinline__ T ld_data(const T *p) { return *p; }
+
 // ------------------------------------------------ block reductions -------
 __device__ __forceinline__ double warp_sum(double v) {
 #pragma unroll

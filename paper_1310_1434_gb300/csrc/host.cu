@@ -93,10 +93,10 @@ int choose_bwd_parts(const SliceDesc &s) {
     return S < 1 ? 1 : (S > s.V ? s.V : S);
 }
 
-cudaError_t launch_backprojection(const SliceDesc &s, int mode, cudaStream_t st) {
-    cudaError_t e = s.orb ? launch_op(OP_ORB_ZPACK, s, mode, st) : cudaSuccess;
-    if (e == cudaSuccess) e = launch_op(s.orb ? OP_ORB_BWD : OP_BWD, s, mode, st);
-    if (e == cudaSuccess && (mode != BWD_PLAIN || bwd_images(s) > 1)) e = launch_op(OP_BWD_FIN, s, mode, st);
+cudaError_t launch_backprojection(const SliceDesc &s, int mode, cudaStream_t st, bool overlap) {
+    cudaError_t e = s.orb ? launch_op(OP_ORB_ZPACK, s, mode, st, overlap) : cudaSuccess;
+    if (e == cudaSuccess) e = launch_op(s.orb ? OP_ORB_BWD : OP_BWD, s, mode, st, overlap);
+    if (e == cudaSuccess && (mode != BWD_PLAIN || bwd_images(s) > 1)) e = launch_op(OP_BWD_FIN, s, mode, st, overlap);
     return e;
 }
 
@@ -237,7 +237,7 @@ RayFx air::make_ray_fx(double px, double py, double ux, double uy, int n, unsign
 // split are timed on the plan's own workspace (the kernels' work does not
 // depend on the data) and the fastest kept; results are cached per geometry
 // for the life of the process, so every plan of a geometry uses the same
-// configuration.
+// configuration.  Timed without launch overlap, each kernel by itself.
 namespace {
 struct TuneKey {
     int n, V, nb;
@@ -307,8 +307,8 @@ air_status autotune(air_plan *P) {
         if (vpb > s.V) continue;
         t.fwd_vpb = vpb;
         const float ms = timed([&] {
-            if (e == cudaSuccess) e = launch_op(OP_TRANSPOSE, t, SRC_EXT, st);
-            if (e == cudaSuccess) e = launch_op(OP_FWD, t, SRC_EXT, st);
+            if (e == cudaSuccess) e = launch_op(OP_TRANSPOSE, t, SRC_EXT, st, false);
+            if (e == cudaSuccess) e = launch_op(OP_FWD, t, SRC_EXT, st, false);
         });
         if (ms < best * 0.98f) {
             best = ms;
@@ -327,7 +327,7 @@ air_status autotune(air_plan *P) {
         if (S > most || (S == S0 && best < 1e30f)) continue;
         t.bwd_parts = S;
         const float ms = timed([&] {
-            if (e == cudaSuccess) e = launch_backprojection(t, BWD_RHS0, st);
+            if (e == cudaSuccess) e = launch_backprojection(t, BWD_RHS0, st, false);
         });
         if (ms < best * 0.98f) {
             best = ms;
@@ -342,7 +342,7 @@ air_status autotune(air_plan *P) {
         if (!s.orb || 8 * S > P->bwd_parts_max) continue;
         t.orb_splits = S;
         const float ms = timed([&] {
-            if (e == cudaSuccess) e = launch_backprojection(t, BWD_RHS0, st);
+            if (e == cudaSuccess) e = launch_backprojection(t, BWD_RHS0, st, false);
         });
         if (ms < best * 0.98f) {
             best = ms;

@@ -41,7 +41,7 @@ RayFx make_ray_fx(double px, double py, double ux, double uy, int n, unsigned *w
 int choose_bwd_parts(const SliceDesc &s);
 // A^T of ext_in (BWD_PLAIN) or zc on the plan's path: the parts and, where
 // there is more than one, their sum with the mode's epilogue.
-cudaError_t launch_backprojection(const SliceDesc &s, int mode, cudaStream_t st);
+cudaError_t launch_backprojection(const SliceDesc &s, int mode, cudaStream_t st, bool overlap = true);
 air_status autotune(air_plan *P);
 void batch_forget(uint64_t plan_id);
 size_t plan_bytes_estimate(const air_geometry &g);

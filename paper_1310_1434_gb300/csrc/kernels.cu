@@ -35,6 +35,7 @@ template <int OP>
 __global__ void __launch_bounds__(AIR_THREADS, min_blocks<OP>) k_op(const SliceDesc s, int arg) {
     extern __shared__ __align__(16) float sm[];
     const int tile = blockIdx.x;
+    grid_wait();
     if constexpr (OP == OP_FWD) {
         tile_fwd(s, arg, tile);
     } else if constexpr (OP == OP_RAMP) {
@@ -84,39 +85,38 @@ __global__ void __launch_bounds__(AIR_THREADS, min_blocks<OP>) k_op(const SliceD
 }
 
 template <int OP>
-static cudaError_t launch_one(const SliceDesc &s, int arg, cudaStream_t st) {
+static cudaError_t launch_one(const SliceDesc &s, int arg, cudaStream_t st, bool overlap) {
     const int tiles = tiles_of(s, OP == OP_FRAMELET && arg ? OP_FRAMELET_T : OP);
     if (tiles <= 0) return cudaSuccess;
     const size_t smem = tile_smem(s, OP);
     static std::atomic<unsigned long long> attr_done{0};
     if (cudaError_t e = opt_in_smem(k_op<OP>, attr_done); e != cudaSuccess) return e;
-    k_op<OP><<<tiles, AIR_THREADS, smem, st>>>(s, arg);
-    return cudaGetLastError();
+    return launch_overlapped(k_op<OP>, dim3(tiles), dim3(AIR_THREADS), smem, overlap, st, s, arg);
 }
 
-cudaError_t launch_op(int op, const SliceDesc &s, int arg, cudaStream_t st) {
+cudaError_t launch_op(int op, const SliceDesc &s, int arg, cudaStream_t st, bool overlap) {
     switch (op) {
-    case OP_FWD: return launch_one<OP_FWD>(s, arg, st);
-    case OP_RAMP: return launch_one<OP_RAMP>(s, arg, st);
-    case OP_BWD: return launch_one<OP_BWD>(s, arg, st);
-    case OP_CG_A: return launch_one<OP_CG_A>(s, arg, st);
-    case OP_CG_B: return launch_one<OP_CG_B>(s, arg, st);
-    case OP_ZERO: return launch_one<OP_ZERO>(s, arg, st);
-    case OP_SHRINK: return launch_one<OP_SHRINK>(s, arg, st);
-    case OP_FRAMELET: return launch_one<OP_FRAMELET>(s, 0, st);
-    case OP_FRAMELET_T: return launch_one<OP_FRAMELET>(s, 1, st);
-    case OP_TRANSPOSE: return launch_one<OP_TRANSPOSE>(s, arg, st);
-    case OP_BWD_FIN: return launch_one<OP_BWD_FIN>(s, arg, st);
-    case OP_AXPY: return launch_one<OP_AXPY>(s, arg, st);
-    case OP_PROX: return launch_one<OP_PROX>(s, arg, st);
-    case OP_FBP: return launch_one<OP_FBP>(s, arg, st);
-    case OP_FBP_PACK: return launch_one<OP_FBP_PACK>(s, arg, st);
-    case OP_FBP_ORB: return launch_one<OP_FBP_ORB>(s, arg, st);
-    case OP_RESTART: return launch_one<OP_RESTART>(s, arg, st);
-    case OP_ORB_PACK: return launch_one<OP_ORB_PACK>(s, arg, st);
-    case OP_ORB_FWD: return launch_one<OP_ORB_FWD>(s, arg, st);
-    case OP_ORB_ZPACK: return launch_one<OP_ORB_ZPACK>(s, arg, st);
-    case OP_ORB_BWD: return launch_one<OP_ORB_BWD>(s, arg, st);
+    case OP_FWD: return launch_one<OP_FWD>(s, arg, st, overlap);
+    case OP_RAMP: return launch_one<OP_RAMP>(s, arg, st, overlap);
+    case OP_BWD: return launch_one<OP_BWD>(s, arg, st, overlap);
+    case OP_CG_A: return launch_one<OP_CG_A>(s, arg, st, overlap);
+    case OP_CG_B: return launch_one<OP_CG_B>(s, arg, st, overlap);
+    case OP_ZERO: return launch_one<OP_ZERO>(s, arg, st, overlap);
+    case OP_SHRINK: return launch_one<OP_SHRINK>(s, arg, st, overlap);
+    case OP_FRAMELET: return launch_one<OP_FRAMELET>(s, 0, st, overlap);
+    case OP_FRAMELET_T: return launch_one<OP_FRAMELET>(s, 1, st, overlap);
+    case OP_TRANSPOSE: return launch_one<OP_TRANSPOSE>(s, arg, st, overlap);
+    case OP_BWD_FIN: return launch_one<OP_BWD_FIN>(s, arg, st, overlap);
+    case OP_AXPY: return launch_one<OP_AXPY>(s, arg, st, overlap);
+    case OP_PROX: return launch_one<OP_PROX>(s, arg, st, overlap);
+    case OP_FBP: return launch_one<OP_FBP>(s, arg, st, overlap);
+    case OP_FBP_PACK: return launch_one<OP_FBP_PACK>(s, arg, st, overlap);
+    case OP_FBP_ORB: return launch_one<OP_FBP_ORB>(s, arg, st, overlap);
+    case OP_RESTART: return launch_one<OP_RESTART>(s, arg, st, overlap);
+    case OP_ORB_PACK: return launch_one<OP_ORB_PACK>(s, arg, st, overlap);
+    case OP_ORB_FWD: return launch_one<OP_ORB_FWD>(s, arg, st, overlap);
+    case OP_ORB_ZPACK: return launch_one<OP_ORB_ZPACK>(s, arg, st, overlap);
+    case OP_ORB_BWD: return launch_one<OP_ORB_BWD>(s, arg, st, overlap);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -159,6 +159,7 @@ k_group(const SliceDesc *__restrict__ slices, const Task *__restrict__ tasks, in
     int staged = -1;
     const SliceDesc &s = stage_desc(slices, t.slice, &sd, &staged);
     const int tile = b - t.tile0;
+    grid_wait();     // the tables above are written by copies, which no kernel overlaps
     if constexpr (OP == OP_FWD) tile_fwd(s, t.arg, tile);
     else if constexpr (OP == OP_RAMP) tile_ramp(s, t.arg, tile, sm);
     else if constexpr (OP == OP_BWD) tile_bwd(s, t.arg, tile, sm);
@@ -182,8 +183,7 @@ static cudaError_t launch_group_op(const SliceDesc *d_slices, const Task *d_task
                                    size_t smem, cudaStream_t st) {
     static std::atomic<unsigned long long> attr_done{0};
     if (cudaError_t e = opt_in_smem(k_group<OP>, attr_done); e != cudaSuccess) return e;
-    k_group<OP><<<total_tiles, AIR_THREADS, smem, st>>>(d_slices, d_tasks, ntasks);
-    return cudaGetLastError();
+    return launch_overlapped(k_group<OP>, dim3(total_tiles), dim3(AIR_THREADS), smem, true, st, d_slices, d_tasks, ntasks);
 }
 
 // Blocks of the grouped backprojector that the device holds at once (SMs x

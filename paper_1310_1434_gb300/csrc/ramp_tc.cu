@@ -160,18 +160,18 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *out) {
 // One view per block: split the row into three BF16 pieces (GEMM operand A)
 // and write the near-band part of Z.
 // measured: a slice descriptor whose sinogram y takes Y's place, or nullptr.
-__global__ void __launch_bounds__(256) k_split_near(const float *__restrict__ Y, const SliceDesc *__restrict__ measured,
-                                                    float *__restrict__ Z,
+__global__ void __launch_bounds__(256) k_split_near(const float *Y, const SliceDesc *measured, float *Z,
                                                     __nv_bfloat16 *__restrict__ A, const float *__restrict__ taps,
                                                     float near_diag, int nb, int kp, const CgState *cg,
                                                     int respect_stop) {
     extern __shared__ __align__(16) float P[];    // [NEAR + nb + NEAR], zero padded
+    grid_wait();
     if (respect_stop && cg->stop) return;
     const int v = blockIdx.x;
     const float *y = (measured ? measured->y : Y) + (size_t)v * nb;
     for (int k = threadIdx.x; k < nb + 2 * NEAR; k += blockDim.x) {
         const int i = k - NEAR;
-        P[k] = (i >= 0 && i < nb) ? y[i] : 0.f;
+        P[k] = (i >= 0 && i < nb) ? ld_data(y + i) : 0.f;
     }
     __syncthreads();
     __nv_bfloat16 *a = A + (size_t)v * 3 * kp;
@@ -204,10 +204,9 @@ __global__ void __launch_bounds__(256) k_split_near(const float *__restrict__ Y,
 
 __global__ void __launch_bounds__(128, 1)
 k_ramp_gemm(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ CUtensorMap map_b,
-            float *__restrict__ Z, int V, int nb, int kp, int np, const CgState *cg, int respect_stop,
+            float *Z, int V, int nb, int kp, int np, const CgState *cg, int respect_stop,
             int *err) {
     extern __shared__ __align__(16) uint8_t raw[];
-    if (respect_stop && cg->stop) return;
     // 1024-byte aligned stage ring, then the barriers and the TMEM address
     uint8_t *base = (uint8_t *)(((uintptr_t)raw + 1023) & ~(uintptr_t)1023);
     uint64_t *full = reinterpret_cast<uint64_t *>(base + STAGES * STAGE_BYTES);
@@ -245,11 +244,13 @@ k_ramp_gemm(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
+    grid_wait();                          // the barriers and TMEM are set up ahead of the split's end
+    const bool idle = respect_stop && cg->stop;
 
     auto stage_a = [&](int s, int piece) { return base + s * STAGE_BYTES + piece * A_TILE; };
     auto stage_b = [&](int s, int piece) { return base + s * STAGE_BYTES + 3 * A_TILE + piece * B_TILE; };
 
-    if (threadIdx.x == 0) {
+    if (threadIdx.x == 0 && !idle) {
         // producer + MMA issuer
         const long long first_polls = g_tc_wait_budget < 0 ? WAIT_POLLS : g_tc_wait_budget;
         bool ok = true;
@@ -311,7 +312,9 @@ k_ramp_gemm(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     __syncthreads();
     const int have = __syncthreads_and(mma_any ? (mbar_wait(done, 0) ? 1 : 0) : 1);
     tc_fence_after();
-    if (have && !abort_flag) {
+    if (idle) {
+        // nothing to add
+    } else if (have && !abort_flag) {
         // lane l of warp w holds row 32 w + l of the tile: it sums the four
         // accumulators into a padded [row][TN + 1] table in the (now idle)
         // stage ring, and the warp then adds its 32 rows to Z with lanes along
@@ -482,15 +485,12 @@ air_status ramp_tc_apply(const air_plan *P, const float *src, const SliceDesc *m
     const TcRes *R = static_cast<const TcRes *>(P->tc);
     if (!R) return fail(AIR_ERR_INVALID_ARG, "plan has no tensor-core filter");
     const int V = P->geom.n_views, nb = P->geom.n_bins;
-    k_split_near<<<V, 256, (nb + 2 * NEAR) * sizeof(float), st>>>(src, measured, dst, R->a, R->near_taps, R->near_diag, nb,
-                                                                   R->kp, cg, respect_stop);
-    cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) {
-        dim3 grid((V + TM - 1) / TM, R->np / TN);   // both parities: 2 x (np / 2) / TN
-        k_ramp_gemm<<<grid, 128, GEMM_SMEM, st>>>(R->map_a, R->map_b, dst, V, nb, R->kp, R->np, cg, respect_stop,
-                                                  R->err);
-        e = cudaGetLastError();
-    }
+    cudaError_t e = launch_overlapped(k_split_near, dim3(V), dim3(256), (nb + 2 * NEAR) * sizeof(float), true, st, src,
+                                      measured, dst, R->a, R->near_taps, R->near_diag, nb, R->kp, cg, respect_stop);
+    const dim3 grid((V + TM - 1) / TM, R->np / TN);   // both parities: 2 x (np / 2) / TN
+    if (e == cudaSuccess)
+        e = launch_overlapped(k_ramp_gemm, grid, dim3(128), GEMM_SMEM, true, st, R->map_a, R->map_b, dst, V, nb, R->kp,
+                              R->np, cg, respect_stop, R->err);
     if (e != cudaSuccess) return fail(AIR_ERR_CUDA, std::string("tensor-core filter launch: ") + cudaGetErrorString(e));
     return AIR_OK;
 }

@@ -36,13 +36,13 @@ __host__ __device__ inline int pair_ld(int n) { return n + 1; }   // pairs per r
 // into one subtraction.  The same integers as the wrap test of the
 // backprojector, with fewer integer instructions on the walk's bound pipe;
 // the image row is a 32-bit element offset into the copy.
-__device__ __forceinline__ void fx_step(long long &nlo, const float2 *__restrict__ copy, unsigned &off, long long M,
+__device__ __forceinline__ void fx_step(long long &nlo, const float2 *copy, unsigned &off, long long M,
                                         unsigned Ma1, unsigned Ma, int ld, float &a0, float &a1) {
     const unsigned nf = (unsigned)nlo;                    // ~(lo mod 2^32)
     const unsigned nr = (unsigned)(nlo >> 32);            // ~r0
     const unsigned ov0 = min(Ma1, nf) + 1u;
     const unsigned ov1 = Ma - ov0;
-    const float2 xx = __ldg(copy + (off - nr));           // pair r0 + 1 of row k
+    const float2 xx = ld_data(copy + (off - nr));          // pair r0 + 1 of row k
     a0 = fmaf(__uint2float_rn(ov0), xx.x, a0);
     a1 = fmaf(__uint2float_rn(ov1), xx.y, a1);
     nlo -= M;
@@ -54,11 +54,11 @@ __device__ __forceinline__ void fx_step(long long &nlo, const float2 *__restrict
 // accumulators of about a quarter of the terms each (two independent FMA
 // chains), which keeps the ray sum's rounding error within the
 // single-application bound for images up to 1024^2.
-__device__ __forceinline__ float fx_ray(const float2 *__restrict__ XP, const float2 *__restrict__ XTP, int n,
+__device__ __forceinline__ float fx_ray(const float2 *XP, const float2 *XTP, int n,
                                         const RayFx &r, unsigned walk) {
     const int k0 = walk_k0(walk), k1 = walk_k1(walk);
     const int ld = pair_ld(n);
-    const float2 *__restrict__ copy = walk_cols(walk) ? XTP : XP;
+    const float2 *copy = walk_cols(walk) ? XTP : XP;
     unsigned off = (unsigned)k0 * (unsigned)ld;           // row k0 of the copy, pair {X[-1], X[0]}
     const long long M = ray_M(r);
     const unsigned Ma = ray_Ma(r);
@@ -225,7 +225,7 @@ __device__ __forceinline__ void tile_bwd(const SliceDesc &s, int mode, int tile,
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const bool colw = warp < BWD_GROUP;             // this warp takes the rays that walk columns
     const unsigned myo = colw ? 1u : 0u;
-    const float *__restrict__ Z = mode == BWD_PLAIN ? s.ext_in : s.zc;
+    const float *Z = mode == BWD_PLAIN ? s.ext_in : s.zc;
     float *wsm = sm + warp * BWD_WARP_FLOATS;
     float *a = wsm + lane;                          // this lane's strip: row r at a + 32 r
     float4 *stA = reinterpret_cast<float4 *>(wsm + BWD_ACC);
@@ -245,7 +245,7 @@ __device__ __forceinline__ void tile_bwd(const SliceDesc &s, int mode, int tile,
         if (j < (int)((e >> 14) & 0x3fffu)) {
             const size_t ri = (size_t)v * nb + j;
             rq = __ldg(reinterpret_cast<const float4 *>(s.ray + ri));
-            rz = __ldg(Z + ri);
+            rz = ld_data(Z + ri);
             if (e & VT_MIXED) ro = walk_cols(__ldg(s.walk + ri));
         }
     };
@@ -559,7 +559,7 @@ __device__ __forceinline__ void tile_fbp(const SliceDesc &s, int tile) {
     const int iy = (tile / tpr) * SHR_T + (int)threadIdx.x / SHR_T;
     if (ix >= n || iy >= n) return;
     const float x = (float)ix + 0.5f - s.half_n, y = (float)iy + 0.5f - s.half_n;
-    const float *__restrict__ Q = s.zc;
+    const float *Q = s.zc;
     float acc = 0.f;
 #pragma unroll 2
     for (int v = 0; v < s.V; ++v, Q += nb) {
@@ -577,8 +577,8 @@ __device__ __forceinline__ void tile_fbp(const SliceDesc &s, int tile) {
         w = fmaf(gp, s.inv_dg_lo, w);
         const int j0 = (int)tr + (w < 0.f ? -1 : (w >= 1.f ? 1 : 0));
         w = w < 0.f ? w + 1.f : (w >= 1.f ? w - 1.f : w);
-        const float q0 = (unsigned)j0 < (unsigned)nb ? __ldg(Q + j0) : 0.f;
-        const float q1 = (unsigned)(j0 + 1) < (unsigned)nb ? __ldg(Q + j0 + 1) : 0.f;
+        const float q0 = (unsigned)j0 < (unsigned)nb ? ld_data(Q + j0) : 0.f;
+        const float q1 = (unsigned)(j0 + 1) < (unsigned)nb ? ld_data(Q + j0 + 1) : 0.f;
         acc += __fdividef(fmaf(w, q1 - q0, q0), fmaf(cr, cr, dt * dt));
     }
     s.ext_out[(size_t)iy * n + ix] = s.fbp_scale * acc;
@@ -865,11 +865,11 @@ __device__ __forceinline__ double fs_tile(const ShrinkArgs &A, int n, int tile, 
         if (SHRINK) {
             const float *p = A.b_in + (size_t)wrapi(y0 - 1 + ly, n) * n + wrapi(x0 - 1 + lx, n);
 #pragma unroll
-            for (int band = 0; band < 9; ++band) bo[band] = __ldg(p + band * nn);
+            for (int band = 0; band < 9; ++band) bo[band] = ld_data(p + band * nn);
         }
         for (int k = threadIdx.x; k < FS_XW * FS_XH; k += AIR_THREADS) {
             const int iy = k / FS_XW, ix = k - iy * FS_XW;
-            sm[k] = __ldg(A.X + (size_t)wrapi(y0 - 2 + iy, n) * n + wrapi(x0 - 2 + ix, n));
+            sm[k] = ld_data(A.X + (size_t)wrapi(y0 - 2 + iy, n) * n + wrapi(x0 - 2 + ix, n));
         }
         __syncthreads();
         SumSq one{0.f, 0.f, 0.f};

@@ -47,3 +47,16 @@ def test_graphs_serve_other_data_plans_and_streams(prec):
     more = [[air.Plan(w.geom) for w in ws] for _ in range(9)]      # one more than are kept
     for i, plans in enumerate(more + more[:1]):
         check(ws, plans, i, 1e-3)
+
+
+def test_plans_that_take_a_destroyed_plans_place():
+    # a new plan may get the address of a destroyed one, and its buffers those
+    # of freed ones: the destroyed plan's graph must not serve it
+    ws = workloads(1)
+    for seed in range(4):
+        plans = [air.Plan(w.geom) for w in ws]
+        check(ws, plans, seed, 1e-3)
+        pad = torch.empty((seed + 1) << 22, device=DEV)     # shifts what the next plans are given
+        for p in plans:
+            p.close()
+        del pad
