@@ -100,12 +100,12 @@ cudaError_t launch_backprojection(const SliceDesc &s, int mode, cudaStream_t st,
     return e;
 }
 
-// Most splits of the orbit backprojector's segments: about four waves of
-// three blocks per SM, at most 16 (each split adds eight images to the sum).
+// Most splits of the orbit backprojector's segments: about two waves of three
+// blocks per SM, at most 8 (each split adds eight images to the sum).
 static int orb_splits_max(int n, int nf, int sms) {
     const int tiles = ((n + BWD_T - 1) / BWD_T) * ((n + BWD_T - 1) / BWD_T) * (nf == 8 ? 1 : 2);
-    const int S = (4 * 3 * sms + tiles - 1) / tiles;
-    return S < 1 ? 1 : (S > 16 ? 16 : S);
+    const int S = (2 * 3 * sms + tiles - 1) / tiles;
+    return S < 1 ? 1 : (S > 8 ? 8 : S);
 }
 
 // Column parts of the orbit projector: as few as give the device about 24
@@ -377,6 +377,9 @@ struct HostTables {
     OrbitTables orb;
     FbpOrbits fbp;
     std::vector<float2> fbp_c;
+    // the tables as a plan holds them, one behind the other, for one upload
+    mutable std::once_flag packed;
+    mutable std::vector<char> blob;
 };
 
 air_status build_tables(const air_geometry &g, double dg, int ntxy, HostTables &T) {
@@ -577,7 +580,7 @@ air_status plan_build(const air_geometry *geom, air_plan *P) {
     s.orb_ks = choose_orb_ks(s.orb_ntask, sms);
     for (int p = 0; p < 8; ++p) s.orb_frame[p] = O.frame[p];
     // carve one allocation
-    struct Piece { void **dst; size_t bytes; };
+    struct Piece { void **dst; size_t bytes; const void *src = nullptr; size_t off = 0; };
     float *x, *r, *p, *q, *rhs0, *gg, *gg2, *b, *b2, *z, *zc, *ybuf, *xbuf, *xp, *xt, *bpart;
     const size_t npad = (size_t)n * (n + 1) * 2;   // pair copies of the projector's input (floats)
     RayFx *ray;
@@ -601,42 +604,42 @@ air_status plan_build(const air_geometry *geom, air_plan *P) {
     CgState *cg;
     double *partial;
     const size_t npart = (size_t)max_reduce_tiles(s) + 64;
+    auto table = [](auto **dst, const auto &v) { return Piece{(void **)dst, v.size() * sizeof(v[0]), v.data()}; };
     std::vector<Piece> pieces = {
-        {(void **)&ray, rays * sizeof(RayFx)}, {(void **)&walk, rays * sizeof(unsigned)},
-        {(void **)&vt, (size_t)V * ntxy * sizeof(unsigned)},
-        {(void **)&xp, npad * 4}, {(void **)&xt, npad * 4}, {(void **)&bpart, (size_t)parts_max * nn * 4},
-        {(void **)&taps, (size_t)nb * sizeof(float)}, {(void **)&fview, (size_t)V * sizeof(float2)},
-        {(void **)&fbw, (size_t)nb * sizeof(float)}, {(void **)&fbt, (size_t)nb * sizeof(float)},
+        // the tables
+        table(&ray, T->ray), table(&walk, T->walk), table(&vt, T->vt), table(&taps, T->taps), table(&fview, T->fview),
+        table(&fbw, T->fbw), table(&fbt, T->fbt), table(&oseg, O.seg), table(&oray, O.ray), table(&oinfo, O.info),
+        table(&oent, O.ent), table(&otask, O.task), table(&otile0, O.tile0), table(&obray, O.bray),
+        table(&fbpc, T->fbp_c), table(&fbpview, F.view),
+        // zeroed once: the image copies' pads stay zero
+        {(void **)&xp, npad * 4}, {(void **)&xt, npad * 4}, {(void **)&ostack, nstack * sizeof(float4)},
+        {(void **)&cg, sizeof(CgState)},
+        // workspace
+        {(void **)&bpart, (size_t)parts_max * nn * 4}, {(void **)&oz, nz * sizeof(float4)},
         {(void **)&x, nn * 4}, {(void **)&r, nn * 4}, {(void **)&p, nn * 4}, {(void **)&q, nn * 4},
         {(void **)&rhs0, nn * 4}, {(void **)&gg, nn * 4}, {(void **)&gg2, nn * 4}, {(void **)&b, 9 * nn * 4}, {(void **)&b2, 9 * nn * 4},
         {(void **)&z, rays * 4}, {(void **)&zc, rays * 4}, {(void **)&ybuf, rays * 4}, {(void **)&xbuf, nn * 4},
-        {(void **)&oseg, O.seg.size() * sizeof(OrbSeg)}, {(void **)&oray, O.ray.size() * sizeof(RayFx)},
-        {(void **)&oinfo, O.info.size() * sizeof(uint2)}, {(void **)&oent, O.ent.size() * sizeof(uint2)},
-        {(void **)&otask, O.task.size() * sizeof(unsigned)}, {(void **)&otile0, O.tile0.size() * sizeof(int)},
-        {(void **)&ostack, nstack * sizeof(float4)}, {(void **)&obray, O.bray.size() * sizeof(uint4)},
-        {(void **)&oz, nz * sizeof(float4)}, {(void **)&fbpc, T->fbp_c.size() * sizeof(float2)},
-        {(void **)&fbpview, F.view.size() * sizeof(int)},
-        {(void **)&cg, sizeof(CgState)}, {(void **)&partial, npart * sizeof(double)}};
-    size_t total = 0;
-    for (auto &pc : pieces) total = align_up(total, 256) + pc.bytes;
+        {(void **)&partial, npart * sizeof(double)}};
+    size_t total = 0, tables_end = 0, zero_end = 0;
+    for (auto &pc : pieces) {
+        pc.off = align_up(total, 256);
+        total = pc.off + pc.bytes;
+        if (pc.src) tables_end = total;
+        if (pc.dst == (void **)&cg) zero_end = total;
+    }
     total = align_up(total, 256);
     char *mem = nullptr;
     if (cudaMalloc(&mem, total) != cudaSuccess) {
         cudaGetLastError();
         return fail(AIR_ERR_OOM, "cudaMalloc of the plan workspace failed (" + std::to_string(total) + " bytes)");
     }
-    size_t off = 0;
-    for (auto &pc : pieces) {
-        off = align_up(off, 256);
-        *pc.dst = mem + off;
-        off += pc.bytes;
-    }
+    for (auto &pc : pieces) *pc.dst = mem + pc.off;
+    std::call_once(T->packed, [&] {
+        T->blob.assign(tables_end, 0);
+        for (auto &pc : pieces)
+            if (pc.src && pc.bytes) std::memcpy(T->blob.data() + pc.off, pc.src, pc.bytes);
+    });
 
-    const std::vector<RayFx> &hray = T->ray;
-    const std::vector<unsigned> &hwalk = T->walk;
-    const std::vector<unsigned> &hvt = T->vt;
-    const std::vector<float> &htaps = T->taps, &hfbw = T->fbw, &hfbt = T->fbt;
-    const std::vector<float2> &hfview = T->fview;
     s.ramp_diag = T->ramp_diag;
     s.fbp_diag = T->fbp_diag;
     s.dso_px = (float)(g.dso_mm / g.pixel_mm);
@@ -644,29 +647,8 @@ air_status plan_build(const air_geometry *geom, air_plan *P) {
     s.inv_dg_lo = (float)(1.0 / dg - (double)s.inv_dg);
     s.jmid = 0.5f * (nb - 1);
     s.fbp_scale = (float)(g.arc / (double)V / (g.pixel_mm * g.pixel_mm));
-    cudaError_t e = cudaMemcpy(ray, hray.data(), rays * sizeof(RayFx), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(walk, hwalk.data(), rays * sizeof(unsigned), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(vt, hvt.data(), hvt.size() * sizeof(unsigned), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(taps, htaps.data(), nb * sizeof(float), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(fview, hfview.data(), V * sizeof(float2), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(fbw, hfbw.data(), nb * sizeof(float), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(fbt, hfbt.data(), nb * sizeof(float), cudaMemcpyHostToDevice);
-    auto upload = [&](void *dst, const void *src, size_t bytes) {
-        if (e == cudaSuccess && bytes) e = cudaMemcpy(dst, src, bytes, cudaMemcpyHostToDevice);
-    };
-    upload(oseg, O.seg.data(), O.seg.size() * sizeof(OrbSeg));
-    upload(oray, O.ray.data(), O.ray.size() * sizeof(RayFx));
-    upload(oinfo, O.info.data(), O.info.size() * sizeof(uint2));
-    upload(oent, O.ent.data(), O.ent.size() * sizeof(uint2));
-    upload(otask, O.task.data(), O.task.size() * sizeof(unsigned));
-    upload(otile0, O.tile0.data(), O.tile0.size() * sizeof(int));
-    upload(fbpc, T->fbp_c.data(), T->fbp_c.size() * sizeof(float2));
-    upload(fbpview, F.view.data(), F.view.size() * sizeof(int));
-    upload(obray, O.bray.data(), O.bray.size() * sizeof(uint4));
-    if (e == cudaSuccess && nstack) e = cudaMemset(ostack, 0, nstack * sizeof(float4));   // the pad rows stay zero
-    if (e == cudaSuccess) e = cudaMemset(cg, 0, sizeof(CgState));
-    if (e == cudaSuccess) e = cudaMemset(xp, 0, npad * 4);   // the pads stay zero
-    if (e == cudaSuccess) e = cudaMemset(xt, 0, npad * 4);
+    cudaError_t e = cudaMemcpy(mem, T->blob.data(), tables_end, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemset(mem + tables_end, 0, zero_end - tables_end);
     if (e != cudaSuccess) {
         cudaFree(mem);
         return fail(AIR_ERR_CUDA, std::string("plan table upload: ") + cudaGetErrorString(e));

@@ -281,20 +281,27 @@ void build_orbits(const air_geometry &g, double dg, OrbitTables &T) {
     const int tpr = (n + BWD_T - 1) / BWD_T, nt = tpr * tpr;
     std::vector<int> tile0(2 * (size_t)(nt + 1), 0);
     std::vector<std::vector<uint2>> lists(2 * (size_t)nt);
+    std::vector<double> angle((size_t)(tpr + 1) * (tpr + 1)), width(angle.size());   // at the tiles' corners
     for (size_t si = 0; si < sorted.size(); ++si) {
         const Seg &S = sorted[si];
+        for (int iy = 0; iy <= tpr; ++iy)
+            for (int ix = 0; ix <= tpr; ++ix) {
+                const double ex = std::min(n, ix * BWD_T) - S.sx, ey = std::min(n, iy * BWD_T) - S.sy;
+                const size_t i = (size_t)iy * (tpr + 1) + ix;
+                angle[i] = std::atan2(S.cx * ey - S.cy * ex, S.cx * ex + S.cy * ey);
+                width[i] = (2.0 * std::fabs(ex) + std::fabs(ey)) / std::sqrt(ex * ex + ey * ey);
+            }
         for (int ty = 0; ty < tpr; ++ty)
             for (int tx = 0; tx < tpr; ++tx) {
                 const double x0 = tx * BWD_T, x1 = std::min(n, (tx + 1) * BWD_T);
                 const double y0 = ty * BWD_T, y1 = std::min(n, (ty + 1) * BWD_T);
                 double gmin = 1e30, gmax = -1e30, wide = 0.0;
-                for (double y : {y0, y1})
-                    for (double x : {x0, x1}) {
-                        const double ex = x - S.sx, ey = y - S.sy;
-                        const double gc = std::atan2(S.cx * ey - S.cy * ex, S.cx * ex + S.cy * ey);
-                        gmin = std::min(gmin, gc);
-                        gmax = std::max(gmax, gc);
-                        wide = std::max(wide, (2.0 * std::fabs(ex) + std::fabs(ey)) / std::hypot(ex, ey));
+                for (int cy = ty; cy <= ty + 1; ++cy)
+                    for (int cx = tx; cx <= tx + 1; ++cx) {
+                        const size_t i = (size_t)cy * (tpr + 1) + cx;
+                        gmin = std::min(gmin, angle[i]);
+                        gmax = std::max(gmax, angle[i]);
+                        wide = std::max(wide, width[i]);
                     }
                 const double f0 = std::ceil(gmin / dg + S.ioff - 0.02), f1 = std::floor(gmax / dg + S.ioff + 0.02);
                 const int a = (int)std::max(0.0, std::min(f0, (double)S.d.cnt));
