@@ -36,7 +36,6 @@ enum Op : int {
     OP_FRAMELET_T, // out = W^T in          (API call)
     OP_TRANSPOSE,  // xp, xt = padded src, transpose(src)   (before every OP_FWD; arg = FwdSrc)
     OP_BWD_FIN,    // sum the backprojector's view parts, then the BwdMode epilogue
-    OP_AXPY,       // q = x + step r            (forward step of Eq. 6, r = A'^T(Y - A x))
     OP_PROX,       // x = W^T S_tau(W q)        (framelet proximal step)
     OP_FBP,        // ext_out = fan-beam FBP weighted backprojection of zc
     OP_FBP_PACK,   // the filtered views of an orbit side by side      (before OP_FBP_ORB)
@@ -49,13 +48,19 @@ enum Op : int {
     OP_COUNT
 };
 
-enum FwdSrc : int { SRC_X = 0, SRC_P = 1, SRC_EXT = 2 };
+// SRC_P_NEXT (OP_ORB_PACK): p after its CG update p = r + beta p, made on the way
+enum FwdSrc : int { SRC_X = 0, SRC_P = 1, SRC_EXT = 2, SRC_P_NEXT = 3 };
 enum RampSrc : int { RSRC_Y = 0, RSRC_Z = 1, RSRC_EXT = 2 };
+// Flags beside a phase's argument.  ARG_SWAP: p is in the workspace's q and q
+// in its p (the orbit path's copies read p at eight places, so its update
+// goes to the other image, where q is no longer needed).  ARG_PACK: the filter
+// writes the orbits' packed samples instead of zc.
+enum ArgFlag : int { ARG_SWAP = 16, ARG_PACK = 32, ARG_MASK = 15 };
 enum BwdMode : int {
     BWD_PLAIN = 0,   // out = dx * acc                      (air_backproject)
     BWD_RHS0 = 1,    // rhs0 = dx * acc
-    BWD_RESID = 2,   // r = rhs0 + mu g - (dx acc + mu x); p = r; rho = r.r
-    BWD_Q = 3        // q = dx acc + mu p; pq = p.q; stop if pq <= 0
+    BWD_Q = 2,       // q = dx acc + mu p; pq = p.q; stop if pq <= 0
+    BWD_STEP = 3     // q = x + step (rhs0 - dx acc)        (forward step of Eq. 6)
 };
 
 // Device-resident CG / Bregman scalars of one slice.  FP64 where the paper's
@@ -188,6 +193,7 @@ struct SliceDesc {
     const uint2 *orb_ent;              // {segment | rays << 17 | candidates << 24, first ray in the padded arrays}
     const uint4 *orb_bray;             // padded rays {L0, |M|, 0}
     float4 *orb_z;                     // [planes of a ray][padded rays]: c times the samples of a ray's orbit
+    const uint2 *orb_zmap;             // per physical ray: its place in orb_z (floats), and its c
     float4 *orb_stack;                 // [2 planes][n][n + 4]: the projector's input in four frames a plane
     float *b, *b2;                     // 9*n*n each (Bregman variable, double-buffered)
     float *z, *zc;                     // V*nb
@@ -264,7 +270,7 @@ __host__ __device__ inline int tiles_of(const SliceDesc &s, int op) {
     case OP_FWD: return tiles_fwd(s);
     case OP_RAMP: return tiles_ramp(s);
     case OP_BWD: return tiles_bwd(s);
-    case OP_CG_A: case OP_CG_B: case OP_ZERO: case OP_BWD_FIN: case OP_AXPY: case OP_RESTART: return tiles_vec(s);
+    case OP_CG_A: case OP_CG_B: case OP_ZERO: case OP_BWD_FIN: case OP_RESTART: return tiles_vec(s);
     case OP_TRANSPOSE: return tiles_tr(s);
     case OP_FBP_PACK: return (int)(((size_t)s.fbp_nbase * (s.nb + 4) + AIR_THREADS - 1) / AIR_THREADS);
     case OP_FBP_ORB: return tiles_shr(s) * s.fbp_splits;

@@ -129,7 +129,7 @@ air_status prepare(int n, air_plan *const *plans, const float *const *Y, const f
         if (tc && !allow_tc)
             return fail(AIR_ERR_INVALID_ARG, "the persistent batch runs the FP32 filter; use FP32 plans");
         B->slices[i] = solve_desc(plans[i], Y[i], lambda[i], mu[i], X[i], nullptr);
-        B->progs[i] = solve_program(n_outer[i], n_cg[i], tc, plans[i]->desc.orb != 0);
+        B->progs[i] = solve_program(n_outer[i], n_cg[i], tc, plans[i]->desc.orb != 0, true);
         B->nphases = std::max(B->nphases, B->progs[i].size());
     }
     cudaGetDevice(&B->device);
@@ -254,8 +254,9 @@ air_status capture_chains(Capture &G, const Batch &B, air_plan *const *plans, in
                 const Launch &T = ls[q];
                 const SliceDesc &sd = B.slices[T.slice];
                 // the measured sinogram changes from call to call: through the descriptor
-                if (ramp_tc_apply(plans[T.slice], sd.z, T.arg == RSRC_Y ? d_slices + T.slice : nullptr, sd.zc, sd.cg,
-                                  T.arg == RSRC_Z, G.side[s0 + (int)((q - li) % nside)]) != AIR_OK)
+                const bool meas = T.arg == RSRC_Y;
+                if (ramp_tc_apply(plans[T.slice], sd.z, meas ? d_slices + T.slice : nullptr, sd.zc, sd.cg, !meas,
+                                  G.side[s0 + (int)((q - li) % nside)]) != AIR_OK)
                     tc_msg = air_last_error();
                 *kernels += 2;   // the split and the tensor-core product
             }

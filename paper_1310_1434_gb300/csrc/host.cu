@@ -93,8 +93,8 @@ int choose_bwd_parts(const SliceDesc &s) {
     return S < 1 ? 1 : (S > s.V ? s.V : S);
 }
 
-cudaError_t launch_backprojection(const SliceDesc &s, int mode, cudaStream_t st, bool overlap) {
-    cudaError_t e = s.orb ? launch_op(OP_ORB_ZPACK, s, mode, st, overlap) : cudaSuccess;
+cudaError_t launch_backprojection(const SliceDesc &s, int mode, bool packed, cudaStream_t st, bool overlap) {
+    cudaError_t e = s.orb && !packed ? launch_op(OP_ORB_ZPACK, s, mode, st, overlap) : cudaSuccess;
     if (e == cudaSuccess) e = launch_op(s.orb ? OP_ORB_BWD : OP_BWD, s, mode, st, overlap);
     if (e == cudaSuccess && (mode != BWD_PLAIN || bwd_images(s) > 1)) e = launch_op(OP_BWD_FIN, s, mode, st, overlap);
     return e;
@@ -158,7 +158,7 @@ size_t plan_bytes_estimate(const air_geometry &g) {
     if (const int nf = orbit_frames(g); nf) {
         parts = std::max(parts, (size_t)8 * orb_splits_max(g.n, nf, sm_count()));
         const size_t segs = 2 * ((size_t)g.n_views / nf + 2);
-        orbit = nn * 32 + (size_t)g.n * 128 + (rays / nf + segs * ORB_CAND) * (sizeof(RayFx) + 8 + 1 + 16 + 4 * nf) + segs * sizeof(OrbSeg) +
+        orbit = nn * 32 + (size_t)g.n * 128 + (rays / nf + segs * ORB_CAND) * (sizeof(RayFx) + 8 + 1 + 16 + 4 * nf) + rays * 8 + segs * sizeof(OrbSeg) +
                 (size_t)tiles_bwd_xy(s) * (segs * 6 + 8);
     }
     size_t b = orbit + rays * (sizeof(RayFx) + 4) + (size_t)g.n_views * tiles_bwd_xy(s) * 4 + (size_t)g.n_bins * 4;
@@ -327,7 +327,7 @@ air_status autotune(air_plan *P) {
         if (S > most || (S == S0 && best < 1e30f)) continue;
         t.bwd_parts = S;
         const float ms = timed([&] {
-            if (e == cudaSuccess) e = launch_backprojection(t, BWD_RHS0, st, false);
+            if (e == cudaSuccess) e = launch_backprojection(t, BWD_RHS0, true, st, false);
         });
         if (ms < best * 0.98f) {
             best = ms;
@@ -342,7 +342,7 @@ air_status autotune(air_plan *P) {
         if (!s.orb || 8 * S > P->bwd_parts_max) continue;
         t.orb_splits = S;
         const float ms = timed([&] {
-            if (e == cudaSuccess) e = launch_backprojection(t, BWD_RHS0, st, false);
+            if (e == cudaSuccess) e = launch_backprojection(t, BWD_RHS0, true, st, false);
         });
         if (ms < best * 0.98f) {
             best = ms;
@@ -590,7 +590,7 @@ air_status plan_build(const air_geometry *geom, air_plan *P) {
     float *fbw, *fbt;
     OrbSeg *oseg;
     RayFx *oray;
-    uint2 *oinfo, *oent;
+    uint2 *oinfo, *oent, *ozmap;
     uint4 *obray;
     float4 *oz;
     float2 *fbpc;
@@ -609,13 +609,13 @@ air_status plan_build(const air_geometry *geom, air_plan *P) {
         // the tables
         table(&ray, T->ray), table(&walk, T->walk), table(&vt, T->vt), table(&taps, T->taps), table(&fview, T->fview),
         table(&fbw, T->fbw), table(&fbt, T->fbt), table(&oseg, O.seg), table(&oray, O.ray), table(&oinfo, O.info),
-        table(&oent, O.ent), table(&otask, O.task), table(&otile0, O.tile0), table(&obray, O.bray),
+        table(&oent, O.ent), table(&otask, O.task), table(&otile0, O.tile0), table(&obray, O.bray), table(&ozmap, O.zmap),
         table(&fbpc, T->fbp_c), table(&fbpview, F.view),
-        // zeroed once: the image copies' pads stay zero
+        // zeroed once: the image copies' pads and the empty rays' samples stay zero
         {(void **)&xp, npad * 4}, {(void **)&xt, npad * 4}, {(void **)&ostack, nstack * sizeof(float4)},
-        {(void **)&cg, sizeof(CgState)},
+        {(void **)&oz, nz * sizeof(float4)}, {(void **)&cg, sizeof(CgState)},
         // workspace
-        {(void **)&bpart, (size_t)parts_max * nn * 4}, {(void **)&oz, nz * sizeof(float4)},
+        {(void **)&bpart, (size_t)parts_max * nn * 4},
         {(void **)&x, nn * 4}, {(void **)&r, nn * 4}, {(void **)&p, nn * 4}, {(void **)&q, nn * 4},
         {(void **)&rhs0, nn * 4}, {(void **)&gg, nn * 4}, {(void **)&gg2, nn * 4}, {(void **)&b, 9 * nn * 4}, {(void **)&b2, 9 * nn * 4},
         {(void **)&z, rays * 4}, {(void **)&zc, rays * 4}, {(void **)&ybuf, rays * 4}, {(void **)&xbuf, nn * 4},
@@ -665,6 +665,7 @@ air_status plan_build(const air_geometry *geom, air_plan *P) {
     s.orb_info = oinfo;
     s.orb_ent = oent;
     s.orb_bray = obray;
+    s.orb_zmap = ozmap;
     s.fbp_c = fbpc;
     s.fbp_view = fbpview;
     choose_fbp(s, F, bpart, parts_max, sms);
@@ -787,19 +788,27 @@ extern "C" air_status air_plan_status(const air_plan *P) {
         if (e_ != cudaSuccess) return fail(AIR_ERR_CUDA, std::string(#expr) + ": " + cudaGetErrorString(e_)); \
     } while (0)
 
+// The FP32 filter puts its results where the orbit backprojector reads them;
+// behind the tensor-core filter OP_ORB_ZPACK does (its epilogue's scattered
+// stores took longer: 2.52 against 2.41 ms for two outer steps of five CG steps
+// at 512^2 / 800 views).
+static bool filter_packs(const air_plan *P, const SliceDesc &s) {
+    return s.orb && !(P->geom.precision == AIR_PREC_BF16X3 && P->geom.filter == AIR_FILTER_RAMLAK);
+}
 static size_t img_bytes(const air_plan *P) { return (size_t)P->geom.n * P->geom.n * 4; }
 static size_t sino_bytes(const air_plan *P) { return (size_t)P->geom.n_views * P->geom.n_bins * 4; }
 
 namespace air {
-// Z = C Y into dst (plan precision), from src (device).
-air_status apply_filter(const air_plan *P, const SliceDesc &base, const float *src, float *dst,
+// Z = C Y into dst (plan precision), from src (device); pack: into the orbits'
+// packed samples (FP32 filter; dst is not written).
+air_status apply_filter(const air_plan *P, const SliceDesc &base, const float *src, float *dst, bool pack,
                         cudaStream_t st) {
     if (P->geom.precision == AIR_PREC_BF16X3 && P->geom.filter == AIR_FILTER_RAMLAK)
         return ramp_tc_apply(P, src, nullptr, dst, base.cg, 0, st);
     SliceDesc s = base;
     s.ext_in = src;
     s.ext_out = dst;
-    CUDA_TRY(launch_op(OP_RAMP, s, RSRC_EXT, st));
+    CUDA_TRY(launch_op(OP_RAMP, s, RSRC_EXT | (pack ? ARG_PACK : 0), st));
     return AIR_OK;
 }
 }  // namespace air
@@ -822,7 +831,7 @@ extern "C" air_status air_filter(const air_plan *P, const float *Y, float *Z, ai
     TRY(check_dev_ptr(Y, "Y"));
     TRY(check_dev_ptr(Z, "Z"));
     if (overlap(Y, sino_bytes(P), Z, sino_bytes(P))) return fail(AIR_ERR_INVALID_ARG, "Y and Z overlap");
-    return apply_filter(P, P->desc, Y, Z, (cudaStream_t)stream);
+    return apply_filter(P, P->desc, Y, Z, false, (cudaStream_t)stream);
 }
 
 extern "C" air_status air_backproject(const air_plan *P, const float *Y, float *X, air_stream stream) {
@@ -833,7 +842,7 @@ extern "C" air_status air_backproject(const air_plan *P, const float *Y, float *
     SliceDesc s = P->desc;
     s.ext_in = Y;
     s.ext_out = X;
-    CUDA_TRY(launch_backprojection(s, BWD_PLAIN, (cudaStream_t)stream));
+    CUDA_TRY(launch_backprojection(s, BWD_PLAIN, false, (cudaStream_t)stream));
     return AIR_OK;
 }
 
@@ -844,11 +853,12 @@ extern "C" air_status air_filtered_backproject(const air_plan *P, const float *Y
     TRY(check_dev_ptr(X, "X"));
     if (overlap(X, img_bytes(P), Y, sino_bytes(P))) return fail(AIR_ERR_INVALID_ARG, "X and Y overlap");
     const cudaStream_t st = (cudaStream_t)stream;
-    TRY(apply_filter(P, P->desc, Y, P->desc.zc, st));
+    const bool packed = filter_packs(P, P->desc);
+    TRY(apply_filter(P, P->desc, Y, P->desc.zc, packed, st));
     SliceDesc s = P->desc;
     s.ext_in = P->desc.zc;
     s.ext_out = X;
-    CUDA_TRY(launch_backprojection(s, BWD_PLAIN, st));
+    CUDA_TRY(launch_backprojection(s, BWD_PLAIN, packed, st));
     return AIR_OK;
 }
 
@@ -899,28 +909,32 @@ namespace air {
 // Each outer step's CG restarts from the residual the previous CG left,
 // corrected for the change of the right-hand side (OP_RESTART): CG keeps
 // r = b - M X, and b changes between outer steps only by mu (g_new - g_old).
-std::vector<Phase> solve_program(int n_outer, int n_cg, bool tc_ramp, bool orb) {
+// `aligned`: every CG step is seven phases, whatever the path, so that the
+// slices of a batch meet in the operators they share.
+std::vector<Phase> solve_program(int n_outer, int n_cg, bool tc_ramp, bool orb, bool aligned) {
     std::vector<Phase> prog;
-    const int ramp = tc_ramp ? OP_RAMP_TC : OP_RAMP;
+    const int ramp = tc_ramp ? OP_RAMP_TC : OP_RAMP, pack = orb && !tc_ramp ? ARG_PACK : 0;
     const int copies = orb ? OP_ORB_PACK : OP_TRANSPOSE, fwd = orb ? OP_ORB_FWD : OP_FWD;
     auto push_bwd = [&](int mode) {
-        if (orb) prog.push_back({OP_ORB_ZPACK, mode});
+        if (orb && tc_ramp) prog.push_back({OP_ORB_ZPACK, mode});
         prog.push_back({orb ? OP_ORB_BWD : OP_BWD, mode});
     };
-    prog.push_back({ramp, RSRC_Y});        // zc = C y
-    push_bwd(BWD_RHS0);   // rhs0 = A^T zc
+    prog.push_back({ramp, RSRC_Y | pack});   // zc = C y
+    push_bwd(BWD_RHS0);                      // rhs0 = A^T zc
     prog.push_back({OP_BWD_FIN, BWD_RHS0});
-    prog.push_back({OP_ZERO, 0});         // X = 0, b = 0, g = g' = 0
-    prog.push_back({OP_RESTART, -1});     // r = p = rhs0 (X = 0, g = 0)
+    prog.push_back({OP_ZERO, 0});            // X = 0, b = 0, g = g' = 0
+    prog.push_back({OP_RESTART, -1});        // r = p = rhs0 (X = 0, g = 0)
     for (int k = 0; k < n_outer; ++k) {
         for (int i = 0; i < n_cg; ++i) {
-            prog.push_back({copies, SRC_P});    // q = M p
+            const int swap = orb && (i & 1) ? ARG_SWAP : 0;                       // see ARG_SWAP
+            prog.push_back({copies, (orb && i > 0 ? SRC_P_NEXT : SRC_P) | swap});   // q = M p
             prog.push_back({fwd, SRC_P});
-            prog.push_back({ramp, RSRC_Z});
+            prog.push_back({ramp, RSRC_Z | pack});
             push_bwd(BWD_Q);
-            prog.push_back({OP_BWD_FIN, BWD_Q});
-            prog.push_back({OP_CG_A, 0});
-            prog.push_back({OP_CG_B, 0});
+            prog.push_back({OP_BWD_FIN, BWD_Q | swap});
+            prog.push_back({OP_CG_A, swap});
+            if (!orb) prog.push_back({OP_CG_B, 0});
+            else if (aligned && !tc_ramp) prog.push_back({OP_NOP, 0});
         }
         prog.push_back({OP_SHRINK, k & 1});
         if (k + 1 < n_outer) prog.push_back({OP_RESTART, k & 1});   // r += mu (g_k - g_{k-1})
@@ -932,33 +946,32 @@ std::vector<Phase> solve_program(int n_outer, int n_cg, bool tc_ramp, bool orb) 
 // from X = 0 (the first L2 step of the split-Bregman program with g = 0 and
 // mu = lambda, without the shrink).
 std::vector<Phase> l2_program(int n_cg, bool tc_ramp, bool orb) {
-    std::vector<Phase> prog = solve_program(1, n_cg, tc_ramp, orb);
+    std::vector<Phase> prog = solve_program(1, n_cg, tc_ramp, orb, false);
     prog.pop_back();   // the SHRINK of the outer step
     return prog;
 }
 
 // Forward-backward splitting AIR: per iteration the forward step of Eq. (6),
-// X + step A'^T (Y - A X) (the residual epilogue at mu = 0 gives
-// r = A'^T Y - A'^T A X), then the framelet proximal step.
+// q = X + step A'^T (Y - A X) in the backprojection's epilogue, then the
+// framelet proximal step.
 std::vector<Phase> fbs_program(int n_iter, bool tc_ramp, bool orb) {
     std::vector<Phase> prog;
-    const int ramp = tc_ramp ? OP_RAMP_TC : OP_RAMP;
+    const int ramp = tc_ramp ? OP_RAMP_TC : OP_RAMP, pack = orb && !tc_ramp ? ARG_PACK : 0;
     const int copies = orb ? OP_ORB_PACK : OP_TRANSPOSE, fwd = orb ? OP_ORB_FWD : OP_FWD;
     auto push_bwd = [&](int mode) {
-        if (orb) prog.push_back({OP_ORB_ZPACK, mode});
+        if (orb && tc_ramp) prog.push_back({OP_ORB_ZPACK, mode});
         prog.push_back({orb ? OP_ORB_BWD : OP_BWD, mode});
     };
-    prog.push_back({ramp, RSRC_Y});
+    prog.push_back({ramp, RSRC_Y | pack});
     push_bwd(BWD_RHS0);
     prog.push_back({OP_BWD_FIN, BWD_RHS0});
     prog.push_back({OP_ZERO, 0});
     for (int k = 0; k < n_iter; ++k) {
         prog.push_back({copies, SRC_X});
         prog.push_back({fwd, SRC_X});
-        prog.push_back({ramp, RSRC_Z});
-        push_bwd(BWD_RESID);
-        prog.push_back({OP_BWD_FIN, BWD_RESID});
-        prog.push_back({OP_AXPY, 0});
+        prog.push_back({ramp, RSRC_Z | pack});
+        push_bwd(BWD_STEP);
+        prog.push_back({OP_BWD_FIN, BWD_STEP});
         prog.push_back({OP_PROX, 0});
     }
     return prog;
@@ -968,8 +981,8 @@ air_status run_program_single(const air_plan *P, const SliceDesc &s, const std::
                               cudaStream_t st) {
     for (const Phase &ph : prog) {
         if (ph.op == OP_RAMP_TC) {
-            const float *src = ph.arg == RSRC_Y ? s.y : s.z;
-            TRY(ramp_tc_apply(P, src, nullptr, s.zc, s.cg, ph.arg == RSRC_Z, st));
+            const bool meas = ph.arg == RSRC_Y;
+            TRY(ramp_tc_apply(P, meas ? s.y : s.z, nullptr, s.zc, s.cg, !meas, st));
         } else {
             CUDA_TRY(launch_op(ph.op, s, ph.arg, st));
         }
@@ -1013,7 +1026,7 @@ extern "C" air_status air_solve(const air_plan *P, const float *Y, float lambda,
     if (resid) TRY(check_dev_ptr(resid, "resid"));
     const bool tc = P->geom.precision == AIR_PREC_BF16X3 && P->geom.filter == AIR_FILTER_RAMLAK;
     SliceDesc s = solve_desc(P, Y, lambda, mu, X, resid);
-    return run_program_single(P, s, solve_program(n_outer, n_cg, tc, s.orb != 0), (cudaStream_t)stream);
+    return run_program_single(P, s, solve_program(n_outer, n_cg, tc, s.orb != 0, false), (cudaStream_t)stream);
 }
 
 extern "C" air_status air_solve_l2(const air_plan *P, const float *Y, float lambda, int n_cg, float *X,
@@ -1035,7 +1048,6 @@ extern "C" air_status air_solve_fbs(const air_plan *P, const float *Y, float lam
     TRY(check_dev_ptr(X, "X"));
     const bool tc = P->geom.precision == AIR_PREC_BF16X3 && P->geom.filter == AIR_FILTER_RAMLAK;
     SliceDesc s = solve_desc(P, Y, 0.f, 1.f, X, nullptr);
-    s.mu = 0.f;                 // the residual epilogue then gives A'^T (Y - A X)
     s.tau = step * lambda;      // the proximal threshold
     s.step = step;
     return run_program_single(P, s, fbs_program(n_iter, tc, P->desc.orb != 0), (cudaStream_t)stream);
@@ -1080,7 +1092,7 @@ extern "C" air_status air_solve_host(const air_plan *P, const float *Y_host, flo
     CUDA_TRY(cudaMemcpyAsync(P->ybuf, Y_host, sino_bytes(P), cudaMemcpyHostToDevice, st));
     const bool tc = P->geom.precision == AIR_PREC_BF16X3 && P->geom.filter == AIR_FILTER_RAMLAK;
     SliceDesc s = solve_desc(P, P->ybuf, lambda, mu, P->xbuf, nullptr);
-    TRY(run_program_single(P, s, solve_program(n_outer, n_cg, tc, P->desc.orb != 0), st));
+    TRY(run_program_single(P, s, solve_program(n_outer, n_cg, tc, P->desc.orb != 0, false), st));
     CUDA_TRY(cudaMemcpyAsync(X_host, P->xbuf, img_bytes(P), cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
     return tc ? air_plan_status(P) : AIR_OK;

@@ -29,7 +29,7 @@ air_status check_dev_ptr(const void *p, const char *what);
 bool overlap(const void *a, size_t na, const void *b, size_t nb);
 size_t align_up(size_t v, size_t a);
 double fan_pitch(const air_geometry &g);
-std::vector<Phase> solve_program(int n_outer, int n_cg, bool tc_ramp, bool orb);
+std::vector<Phase> solve_program(int n_outer, int n_cg, bool tc_ramp, bool orb, bool aligned);
 std::vector<Phase> l2_program(int n_cg, bool tc_ramp, bool orb);
 std::vector<Phase> fbs_program(int n_iter, bool tc_ramp, bool orb);
 air_status check_solve_args(const air_plan *P, const float *Y, float lambda, float mu, int n_outer,
@@ -40,12 +40,13 @@ air_status run_program_single(const air_plan *P, const SliceDesc &s, const std::
 RayFx make_ray_fx(double px, double py, double ux, double uy, int n, unsigned *walk);
 int choose_bwd_parts(const SliceDesc &s);
 // A^T of ext_in (BWD_PLAIN) or zc on the plan's path: the parts and, where
-// there is more than one, their sum with the mode's epilogue.
-cudaError_t launch_backprojection(const SliceDesc &s, int mode, cudaStream_t st, bool overlap = true);
+// there is more than one, their sum with the mode's epilogue.  packed: the
+// orbits' samples are packed already (ARG_PACK).
+cudaError_t launch_backprojection(const SliceDesc &s, int mode, bool packed, cudaStream_t st, bool overlap = true);
 air_status autotune(air_plan *P);
 void batch_forget(uint64_t plan_id);
 size_t plan_bytes_estimate(const air_geometry &g);
-air_status apply_filter(const air_plan *P, const SliceDesc &base, const float *src, float *dst,
+air_status apply_filter(const air_plan *P, const SliceDesc &base, const float *src, float *dst, bool pack,
                         cudaStream_t st);
 // Loads the allocation-free filtered adjoint's static scratch on the current
 // device (CUDA loads a module, and allocates its device arrays, on first

@@ -45,13 +45,11 @@ __global__ void __launch_bounds__(AIR_THREADS, min_blocks<OP>) k_op(const SliceD
     } else if constexpr (OP == OP_BWD_FIN) {
         tile_bwd_fin(s, arg, tile);
     } else if constexpr (OP == OP_CG_A) {
-        tile_cg_a(s, tile);
+        tile_cg_a(s, arg, tile);
     } else if constexpr (OP == OP_CG_B) {
         tile_cg_b(s, tile);
     } else if constexpr (OP == OP_ZERO) {
         tile_zero(s, tile);
-    } else if constexpr (OP == OP_AXPY) {
-        tile_axpy(s, tile);
     } else if constexpr (OP == OP_PROX) {
         tile_prox(s, tile, sm);
     } else if constexpr (OP == OP_FBP) {
@@ -107,7 +105,6 @@ cudaError_t launch_op(int op, const SliceDesc &s, int arg, cudaStream_t st, bool
     case OP_FRAMELET_T: return launch_one<OP_FRAMELET>(s, 1, st, overlap);
     case OP_TRANSPOSE: return launch_one<OP_TRANSPOSE>(s, arg, st, overlap);
     case OP_BWD_FIN: return launch_one<OP_BWD_FIN>(s, arg, st, overlap);
-    case OP_AXPY: return launch_one<OP_AXPY>(s, arg, st, overlap);
     case OP_PROX: return launch_one<OP_PROX>(s, arg, st, overlap);
     case OP_FBP: return launch_one<OP_FBP>(s, arg, st, overlap);
     case OP_FBP_PACK: return launch_one<OP_FBP_PACK>(s, arg, st, overlap);
@@ -164,10 +161,9 @@ k_group(const SliceDesc *__restrict__ slices, const Task *__restrict__ tasks, in
     else if constexpr (OP == OP_RAMP) tile_ramp(s, t.arg, tile, sm);
     else if constexpr (OP == OP_BWD) tile_bwd(s, t.arg, tile, sm);
     else if constexpr (OP == OP_BWD_FIN) tile_bwd_fin(s, t.arg, tile);
-    else if constexpr (OP == OP_CG_A) tile_cg_a(s, tile);
+    else if constexpr (OP == OP_CG_A) tile_cg_a(s, t.arg, tile);
     else if constexpr (OP == OP_CG_B) tile_cg_b(s, tile);
     else if constexpr (OP == OP_ZERO) tile_zero(s, tile);
-    else if constexpr (OP == OP_AXPY) tile_axpy(s, tile);
     else if constexpr (OP == OP_PROX) tile_prox(s, tile, sm);
     else if constexpr (OP == OP_TRANSPOSE) tile_transpose(s, t.arg, tile, sm);
     else if constexpr (OP == OP_SHRINK) run_shrink(s, t.arg, tile, sm);
@@ -215,7 +211,6 @@ cudaError_t launch_group(int op, const SliceDesc *d_slices, const Task *d_tasks,
     case OP_ZERO: return launch_group_op<OP_ZERO>(d_slices, d_tasks, ntasks, total_tiles, smem, st);
     case OP_TRANSPOSE: return launch_group_op<OP_TRANSPOSE>(d_slices, d_tasks, ntasks, total_tiles, smem, st);
     case OP_SHRINK: return launch_group_op<OP_SHRINK>(d_slices, d_tasks, ntasks, total_tiles, smem, st);
-    case OP_AXPY: return launch_group_op<OP_AXPY>(d_slices, d_tasks, ntasks, total_tiles, smem, st);
     case OP_PROX: return launch_group_op<OP_PROX>(d_slices, d_tasks, ntasks, total_tiles, smem, st);
     case OP_RESTART: return launch_group_op<OP_RESTART>(d_slices, d_tasks, ntasks, total_tiles, smem, st);
     case OP_ORB_PACK: return launch_group_op<OP_ORB_PACK>(d_slices, d_tasks, ntasks, total_tiles, smem, st);

@@ -122,7 +122,7 @@ extern "C" air_status air_filtered_backproject_noalloc(const air_plan *P, const 
         d.ext_out = X;
         d.bwd_parts = std::max(1, (int)std::min<size_t>(P->desc.bwd_parts, room));
         d.bwd_part = bwd_images(d) > 1 ? scratch + off : nullptr;
-        e = launch_backprojection(d, BWD_PLAIN, s);
+        e = launch_backprojection(d, BWD_PLAIN, false, s);
     }
     if (e != cudaSuccess) return fail(AIR_ERR_CUDA, std::string("filtered backprojection: ") + cudaGetErrorString(e));
     return AIR_OK;

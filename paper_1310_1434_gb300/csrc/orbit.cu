@@ -3,6 +3,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 
 #include "host_common.h"
 
@@ -322,6 +323,16 @@ void build_orbits(const air_geometry &g, double dg, OrbitTables &T) {
             if (t < nt) ent.insert(ent.end(), lists[(size_t)c * nt + t].begin(), lists[(size_t)c * nt + t].end());
         }
 
+    std::vector<uint2> zmap((size_t)V * nb);
+    for (const Seg &S : sorted)
+        for (int f = 0; f < nf; ++f)
+            for (int i = 0; i < S.d.cnt && S.d.zoff[f] >= 0; ++i) {
+                unsigned c;
+                std::memcpy(&c, &rays[S.d.ray0 + i].cs, 4);
+                zmap[S.d.zoff[f] + ((S.d.down >> f) & 1 ? -i : i)] =
+                    make_uint2((unsigned)((f / 4) * bray.size() + S.d.pad0 + i) * 4u + (unsigned)(f & 3), c);
+            }
+
     T.eps = (float)eps;
     for (size_t i = 0; i < sorted.size(); ++i) {
         OrbSeg d = sorted[i].d;
@@ -340,6 +351,7 @@ void build_orbits(const air_geometry &g, double dg, OrbitTables &T) {
     T.tile0 = std::move(tile0);
     T.ent = std::move(ent);
     T.bray = std::move(bray);
+    T.zmap = std::move(zmap);
     T.nf = nf;
 }
 

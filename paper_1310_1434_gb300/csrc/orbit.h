@@ -36,6 +36,7 @@ struct OrbitTables {
     std::vector<int> tile0;           // [2 classes][pixel tiles + 1] offsets into ent
     std::vector<uint2> ent;           // backprojector: per class and tile the segments that meet it
     std::vector<uint4> bray;          // padded rays: each segment's, then ORB_CAND empty ones
+    std::vector<uint2> zmap;          // per physical ray: place among the packed samples (floats), c
 };
 
 // The views of a full scan grouped by its symmetries, for the analytic

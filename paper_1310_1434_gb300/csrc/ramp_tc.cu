@@ -480,8 +480,8 @@ void ramp_tc_destroy(air_plan *P) {
     P->tc_bytes = 0;
 }
 
-air_status ramp_tc_apply(const air_plan *P, const float *src, const SliceDesc *measured, float *dst, const CgState *cg, int respect_stop,
-                         cudaStream_t st) {
+air_status ramp_tc_apply(const air_plan *P, const float *src, const SliceDesc *measured, float *dst, const CgState *cg,
+                         int respect_stop, cudaStream_t st) {
     const TcRes *R = static_cast<const TcRes *>(P->tc);
     if (!R) return fail(AIR_ERR_INVALID_ARG, "plan has no tensor-core filter");
     const int V = P->geom.n_views, nb = P->geom.n_bins;

@@ -250,7 +250,7 @@ void admit(air_server *S) {
         r->slot = S->free_slots.back();
         S->free_slots.pop_back();
         const bool tc = r->geom.precision == AIR_PREC_BF16X3 && r->geom.filter == AIR_FILTER_RAMLAK;
-        r->prog = solve_program(r->n_outer, r->n_cg, tc, plan->desc.orb != 0);
+        r->prog = solve_program(r->n_outer, r->n_cg, tc, plan->desc.orb != 0, false);
         r->pc = 0;
         const size_t sino = (size_t)r->geom.n_views * r->geom.n_bins * 4;
         S->h_slices[r->slot] = solve_desc(plan, plan->ybuf, r->lam, r->mu, plan->xbuf, nullptr);
@@ -337,7 +337,8 @@ air_status enqueue_step(air_server *S) {
             Request *r = it->second[0];
             const SliceDesc &sd = S->h_slices[r->slot];
             const int arg = r->prog[r->pc].arg;
-            st1 = ramp_tc_apply(r->plan, arg == RSRC_Y ? sd.y : sd.z, nullptr, sd.zc, sd.cg, arg == RSRC_Z, S->stream);
+            const bool meas = arg == RSRC_Y;
+            st1 = ramp_tc_apply(r->plan, meas ? sd.y : sd.z, nullptr, sd.zc, sd.cg, !meas, S->stream);
         }
         if (st1 != AIR_OK) return st1;
         return finish_step(S, k);
@@ -359,7 +360,8 @@ air_status enqueue_step(air_server *S) {
         Request *r = it->second[i];
         const SliceDesc &sd = S->h_slices[r->slot];
         const int arg = r->prog[r->pc].arg;
-        st = ramp_tc_apply(r->plan, arg == RSRC_Y ? sd.y : sd.z, nullptr, sd.zc, sd.cg, arg == RSRC_Z, S->side[q++ % nside]);
+        const bool meas = arg == RSRC_Y;
+        st = ramp_tc_apply(r->plan, meas ? sd.y : sd.z, nullptr, sd.zc, sd.cg, !meas, S->side[q++ % nside]);
     }
     for (int k2 = 0; k2 < nside; ++k2) {       // join even after a failure: the stream stays ordered
         cudaEventRecord(S->join[k2], S->side[k2]);

@@ -352,7 +352,7 @@ __device__ __forceinline__ void tile_bwd(const SliceDesc &s, int mode, int tile,
 // whose tuned split, and with it the order of its sums, follows this sum's
 // time.
 template <int N>
-__device__ __forceinline__ double bwd_fin(const SliceDesc &s, int mode, int i) {
+__device__ __forceinline__ double bwd_fin(const SliceDesc &s, int mode, bool swap, int i) {
     struct __align__(4 * N) Vec { float v[N]; };
     auto get = [&](const float *a) { return *reinterpret_cast<const Vec *>(a + i); };
     auto put = [&](float *a, const Vec &x) { *reinterpret_cast<Vec *>(a + i) = x; };
@@ -372,57 +372,50 @@ __device__ __forceinline__ double bwd_fin(const SliceDesc &s, int mode, int i) {
         put(s.ext_out, a);
     } else if (mode == BWD_RHS0) {
         put(s.rhs0, a);
-    } else if (mode == BWD_RESID) {
-        const Vec x = get(s.x), g = get(s.g), b = get(s.rhs0);
-        Vec r;
+    } else if (mode == BWD_STEP) {
+        const Vec x = get(s.x), b = get(s.rhs0);
+        Vec o;
 #pragma unroll
-        for (int q = 0; q < N; ++q) {
-            r.v[q] = fmaf(s.mu, g.v[q], b.v[q]) - fmaf(s.mu, x.v[q], a.v[q]);
-            part += (double)r.v[q] * (double)r.v[q];
-        }
-        put(s.r, r);
-        put(s.p, r);
+        for (int q = 0; q < N; ++q) o.v[q] = fmaf(s.step, b.v[q] - a.v[q], x.v[q]);
+        put(s.q, o);
     } else {  // BWD_Q
-        const Vec p = get(s.p);
+        const Vec p = get(swap ? s.q : s.p);
         Vec o;
 #pragma unroll
         for (int q = 0; q < N; ++q) {
             o.v[q] = fmaf(s.mu, p.v[q], a.v[q]);
             part += (double)p.v[q] * (double)o.v[q];
         }
-        put(s.q, o);
+        put(swap ? s.p : s.q, o);
     }
     return part;
 }
 
-__device__ __forceinline__ void tile_bwd_fin(const SliceDesc &s, int mode, int tile) {
+__device__ __forceinline__ void tile_bwd_fin(const SliceDesc &s, int arg, int tile) {
     __shared__ double sh[AIR_THREADS / 32];
+    const int mode = arg & ARG_MASK;
+    const bool swap = (arg & ARG_SWAP) != 0;
     if (mode == BWD_Q && s.cg->stop) return;
     const int nn = s.n * s.n, base = tile * VEC_PER_TILE;
     double part = 0.0;
     if (s.orb && nn % 4 == 0) {
         const int i = base + 4 * (int)threadIdx.x;
-        if (i < nn) part = bwd_fin<4>(s, mode, i);
+        if (i < nn) part = bwd_fin<4>(s, mode, swap, i);
     } else {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int i = base + k * AIR_THREADS + (int)threadIdx.x;
-            if (i < nn) part += bwd_fin<1>(s, mode, i);
+            if (i < nn) part += bwd_fin<1>(s, mode, swap, i);
         }
     }
-    if (mode == BWD_PLAIN || mode == BWD_RHS0) return;
+    if (mode == BWD_PLAIN || mode == BWD_RHS0 || mode == BWD_STEP) return;
     part = block_sum(part, sh);
     double tot;
     if (reduce_tiles(s, tile, tiles_vec(s), part, sh, &tot) && threadIdx.x == 0) {
         CgState *c = s.cg;
-        if (mode == BWD_RESID) {
-            c->rho = tot;
-            c->stop = !(tot != 0.0);
-        } else {
-            c->pq = tot;
-            if (!(tot > 0.0)) c->stop = 1;
-            else c->alpha = c->rho / tot;
-        }
+        c->pq = tot;
+        if (!(tot > 0.0)) c->stop = 1;
+        else c->alpha = c->rho / tot;
     }
 }
 
@@ -463,14 +456,27 @@ __device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigne
     return d;
 }
 
+// Where the filter's result of sample i goes: its row, or (ARG_PACK) its place
+// among the orbits' packed samples, times the ray's c.
+__device__ __forceinline__ void put_filtered(const SliceDesc &s, bool pack, float *dst, size_t i, float v) {
+    if (pack) {
+        const uint2 m = __ldg(s.orb_zmap + i);
+        reinterpret_cast<float *>(s.orb_z)[m.x] = __uint_as_float(m.y) * v;
+    } else {
+        dst[i] = v;
+    }
+}
+
 __device__ __forceinline__ void tile_ramp(const SliceDesc &s, int arg, int tile, float *sm) {
+    const bool pack = (arg & ARG_PACK) != 0;
+    arg &= ARG_MASK;
     const float *src = arg == RSRC_Y ? s.y : (arg == RSRC_Z ? s.z : s.ext_in);
     float *dst = arg == RSRC_EXT ? s.ext_out : s.zc;
     const int nb = s.nb;
     const size_t off = (size_t)tile * nb;
     if (arg == RSRC_Z && s.cg->stop) return;
     if (!s.filter) {
-        for (int j = threadIdx.x; j < nb; j += AIR_THREADS) dst[off + j] = src[off + j];
+        for (int j = threadIdx.x; j < nb; j += AIR_THREADS) put_filtered(s, pack, dst, off + j, src[off + j]);
         return;
     }
     const int lags = ramp_lags(nb), PO = ramp_pad(nb), PQ = ramp_pq(nb);
@@ -532,8 +538,8 @@ __device__ __forceinline__ void tile_ramp(const SliceDesc &s, int arg, int tile,
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const float2 a = unpair2(acc[q]);
-            if (j0 + 2 * q < nb) dst[off + j0 + 2 * q] = fmaf(diag, ctr[2 * q], a.x);
-            if (j0 + 2 * q + 1 < nb) dst[off + j0 + 2 * q + 1] = fmaf(diag, ctr[2 * q + 1], a.y);
+            if (j0 + 2 * q < nb) put_filtered(s, pack, dst, off + j0 + 2 * q, fmaf(diag, ctr[2 * q], a.x));
+            if (j0 + 2 * q + 1 < nb) put_filtered(s, pack, dst, off + j0 + 2 * q + 1, fmaf(diag, ctr[2 * q + 1], a.y));
         }
     }
     __syncthreads();
@@ -587,10 +593,11 @@ __device__ __forceinline__ void tile_fbp(const SliceDesc &s, int tile) {
 // ======================================================================
 // CG vector updates (Eq. 5 system) with FP64 inner products.
 // ======================================================================
-__device__ __forceinline__ void tile_cg_a(const SliceDesc &s, int tile) {
+__device__ __forceinline__ void tile_cg_a(const SliceDesc &s, int arg, int tile) {
     __shared__ double sh[AIR_THREADS / 32];
     if (s.cg->stop) return;
     const float a = (float)s.cg->alpha;
+    const float *pv = arg & ARG_SWAP ? s.q : s.p, *qv = arg & ARG_SWAP ? s.p : s.q;
     const int nn = s.n * s.n;
     const int base = tile * VEC_PER_TILE;
     double part = 0.0;
@@ -598,8 +605,8 @@ __device__ __forceinline__ void tile_cg_a(const SliceDesc &s, int tile) {
     for (int k = 0; k < 4; ++k) {
         const int i = base + k * AIR_THREADS + threadIdx.x;
         if (i < nn) {
-            s.x[i] = fmaf(a, s.p[i], s.x[i]);
-            const float rv = fmaf(-a, s.q[i], s.r[i]);
+            s.x[i] = fmaf(a, pv[i], s.x[i]);
+            const float rv = fmaf(-a, qv[i], s.r[i]);
             s.r[i] = rv;
             part += (double)rv * (double)rv;
         }
@@ -655,18 +662,6 @@ __device__ __forceinline__ void tile_restart(const SliceDesc &s, int arg, int ti
         CgState *c = s.cg;
         c->rho = tot;
         c->stop = !(tot != 0.0);
-    }
-}
-
-// q = x + step r: the forward step of forward-backward splitting (Eq. 6),
-// with r = A'^T (Y - A x) from the OP_BWD_FIN residual epilogue at mu = 0.
-__device__ __forceinline__ void tile_axpy(const SliceDesc &s, int tile) {
-    const int nn = s.n * s.n;
-    const int base = tile * VEC_PER_TILE;
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-        const int i = base + k * AIR_THREADS + threadIdx.x;
-        if (i < nn) s.q[i] = fmaf(s.step, s.r[i], s.x[i]);
     }
 }
 
@@ -1008,10 +1003,9 @@ __device__ __forceinline__ void run_tile(const SliceDesc &s, int op, int arg, in
     case OP_RAMP: tile_ramp(s, arg, tile, sm); break;
     case OP_BWD: tile_bwd(s, arg, tile, sm); break;
     case OP_BWD_FIN: tile_bwd_fin(s, arg, tile); break;
-    case OP_CG_A: tile_cg_a(s, tile); break;
+    case OP_CG_A: tile_cg_a(s, arg, tile); break;
     case OP_CG_B: tile_cg_b(s, tile); break;
     case OP_ZERO: tile_zero(s, tile); break;
-    case OP_AXPY: tile_axpy(s, tile); break;
     case OP_PROX: tile_prox(s, tile, sm); break;
     case OP_FBP: tile_fbp(s, tile); break;
     case OP_SHRINK: run_shrink(s, arg, tile, sm); break;

@@ -38,8 +38,16 @@ __device__ __forceinline__ void orb_pixel(int code, int n, int k, int r, int &ix
 // Frames without ORB_T read along k and are turned in shared memory.
 // ======================================================================
 __device__ __forceinline__ void tile_orb_pack(const SliceDesc &s, int arg, int tile, float *sm) {
-    if (arg == SRC_P && s.cg->stop) return;
-    const float *src = arg == SRC_X ? s.x : (arg == SRC_P ? s.p : s.ext_in);
+    const bool swap = (arg & ARG_SWAP) != 0;
+    arg &= ARG_MASK;
+    const bool cg = arg == SRC_P || arg == SRC_P_NEXT, next = arg == SRC_P_NEXT;
+    if (cg && s.cg->stop) return;
+    // SRC_P_NEXT: p = r + beta p on the way, from the image that held it to the
+    // other one; plane 0 writes what it reads for its first frame, every pixel
+    // once.  (Folded into the general path's copies it gained nothing.)
+    const float *src = arg == SRC_X ? s.x : (!cg ? s.ext_in : (swap != next ? s.q : s.p));
+    float *to = swap ? s.q : s.p;
+    const float bt = next ? (float)s.cg->beta : 0.f;
     const int n = s.n, tpr = (n + 31) / 32, nt = tpr * tpr;
     const int plane = tile / nt, t = tile - plane * nt;
     const int k0 = (t % tpr) * 32, r0 = (t / tpr) * 32;
@@ -56,7 +64,12 @@ __device__ __forceinline__ void tile_orb_pack(const SliceDesc &s, int arg, int t
             if (k0 + kk < n && r0 + rr < n) {
                 int ix, iy;
                 orb_pixel(code, n, k0 + kk, r0 + rr, ix, iy);
-                v = ld_data(src + (size_t)iy * n + ix);
+                const size_t i = (size_t)iy * n + ix;
+                v = src[i];
+                if (next) {
+                    v = fmaf(bt, v, s.r[i]);
+                    if (plane == 0 && q == 0) to[i] = v;
+                }
             }
             f[q][kk][rr] = v;
         }

@@ -11,6 +11,7 @@
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
+#include <cstring>
 #include <map>
 #include <unordered_map>
 #include <vector>
@@ -57,6 +58,10 @@ int main(int argc, char **argv) {
             if (s.zoff[f] < 0) continue;
             const int z = s.zoff[f] + ((s.down >> f) & 1 ? -j : j), v = z / nb, b = z % nb;
             rays.at(z) += 1;
+            // the filter's place for this ray's sample is the backprojector's
+            unsigned c;
+            memcpy(&c, &r.cs, 4);
+            bad += T.zmap.at(z).x != ((f / 4) * T.bray.size() + s.pad0 + j) * 4 + (f & 3) || T.zmap[z].y != c;
             const int code = T.frame[T.nf == 8 ? f : 4 * s.cls + f];
             std::map<int, double> diff;
             double sum = 0.0;
