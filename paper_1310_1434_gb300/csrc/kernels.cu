@@ -29,7 +29,7 @@ static cudaError_t opt_in_smem(Kernel kernel, std::atomic<unsigned long long> &d
 // The orbit backprojector is held to three blocks per SM by its shared memory
 // (60 KB at eight frames); its registers must allow as many.
 template <int OP>
-constexpr int min_blocks = OP == OP_ORB_BWD ? 3 : 0;
+constexpr int min_blocks = OP == OP_ORB_BWD || OP == OP_ORB_FWD ? 3 : 0;
 
 template <int OP>
 __global__ void __launch_bounds__(AIR_THREADS, min_blocks<OP>) k_op(const SliceDesc s, int arg) {

@@ -129,34 +129,44 @@ __device__ __forceinline__ ulonglong2 ld_pixels_if(const ulonglong2 *p, unsigned
     return v;
 }
 
+constexpr int ORB_U = 4;                                          // columns whose loads are in flight together
 template <int NP>
 struct OrbAcc {
     unsigned long long v[2 * NP];   // frames {0, 1}, {2, 3} of each plane
 };
 
-template <int NP>
-__device__ __forceinline__ void orb_step(unsigned long long &np, const ulonglong2 *col, size_t plane,
-                                         unsigned Ma, int n, OrbAcc<NP> &a) {
-    unsigned ov0, ov1;
-    orb_overlap((unsigned)np, Ma, ov0, ov1);
-    const int nr = min(max((int)(np >> 32), -1 - n), ORB_PAD - 1);   // ~row, the row clamped to [-2, n]
-    const ulonglong2 *c = col - nr;                                  // col is one row past the column's row 0
-    ulonglong2 x0[NP], x1[NP];
+// U columns of the walk: every load is issued before the first FMA, so that a
+// warp has 4 U of them (two planes) in flight.
+template <int NP, int U>
+__device__ __forceinline__ void orb_steps(unsigned long long &np, const ulonglong2 *col, int ld, size_t plane, unsigned Ma,
+                                          int n, OrbAcc<NP> &a, OrbAcc<NP> &b) {
+    ulonglong2 x0[U][NP], x1[U][NP];
+    unsigned ov0[U], ov1[U];
 #pragma unroll
-    for (int q = 0; q < NP; ++q) {
-        x0[q] = ld_pixels(c + q * plane - 1);
-        x1[q] = ld_pixels_if(c + q * plane, ov1);
-    }
-    const float f0 = __uint2float_rn(ov0), f1 = __uint2float_rn(ov1);
-    const unsigned long long w0 = pair2(f0, f0), w1 = pair2(f1, f1);
+    for (int u = 0; u < U; ++u) {
+        orb_overlap((unsigned)np, Ma, ov0[u], ov1[u]);
+        const int nr = min(max((int)(np >> 32), -1 - n), ORB_PAD - 1);   // ~row, the row clamped to [-2, n]
+        const ulonglong2 *c = col + u * ld - nr;                         // col is one row past the column's row 0
 #pragma unroll
-    for (int q = 0; q < NP; ++q) {
-        a.v[2 * q] = fma2(w0, x0[q].x, a.v[2 * q]);
-        a.v[2 * q + 1] = fma2(w0, x0[q].y, a.v[2 * q + 1]);
-        a.v[2 * q] = fma2(w1, x1[q].x, a.v[2 * q]);
-        a.v[2 * q + 1] = fma2(w1, x1[q].y, a.v[2 * q + 1]);
+        for (int q = 0; q < NP; ++q) {
+            x0[u][q] = ld_pixels(c + q * plane - 1);
+            x1[u][q] = ld_pixels_if(c + q * plane, ov1[u]);
+        }
+        np -= Ma;
     }
-    np -= Ma;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const float f0 = __uint2float_rn(ov0[u]), f1 = __uint2float_rn(ov1[u]);
+        const unsigned long long w0 = pair2(f0, f0), w1 = pair2(f1, f1);
+        OrbAcc<NP> &s = u & 1 ? b : a;
+#pragma unroll
+        for (int q = 0; q < NP; ++q) {
+            s.v[2 * q] = fma2(w0, x0[u][q].x, s.v[2 * q]);
+            s.v[2 * q + 1] = fma2(w0, x0[u][q].y, s.v[2 * q + 1]);
+            s.v[2 * q] = fma2(w1, x1[u][q].x, s.v[2 * q]);
+            s.v[2 * q + 1] = fma2(w1, x1[u][q].y, s.v[2 * q + 1]);
+        }
+    }
 }
 
 template <int NP>
@@ -192,13 +202,17 @@ __device__ __forceinline__ void tile_orb_fwd_np(const SliceDesc &s, int arg, int
         unsigned long long np = ~((unsigned long long)r.L0 + (unsigned long long)q0 * Ma);
         OrbAcc<NP> a{}, b{};
         int k = q0;
-#pragma unroll 2
-        for (; k + 1 < q1; k += 2) {
-            orb_step<NP>(np, col, plane, Ma, n, a);
-            orb_step<NP>(np, col + ld, plane, Ma, n, b);
+#pragma unroll 1
+        for (; k + ORB_U <= q1; k += ORB_U) {
+            orb_steps<NP, ORB_U>(np, col, ld, plane, Ma, n, a, b);
+            col += ORB_U * ld;
+        }
+#pragma unroll 1
+        for (; k + 2 <= q1; k += 2) {
+            orb_steps<NP, 2>(np, col, ld, plane, Ma, n, a, b);
             col += 2 * ld;
         }
-        if (k < q1) orb_step<NP>(np, col, plane, Ma, n, a);
+        if (k < q1) orb_steps<NP, 1>(np, col, ld, plane, Ma, n, a, b);
 #pragma unroll
         for (int q = 0; q < 2 * NP; ++q) {
             const float2 x = unpair2(a.v[q]), y = unpair2(b.v[q]);
