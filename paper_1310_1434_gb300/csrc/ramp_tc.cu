@@ -33,11 +33,13 @@
 #include <cuda_bf16.h>
 #include <cudaTypedefs.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <string>
 #include <vector>
 
+#include "packed.cuh"
 #include "ramp_tc.h"
 
 namespace air {
@@ -158,47 +160,107 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float *out) {
 
 // ------------------------------------------------------------ kernels
 // One view per block: split the row into three BF16 pieces (GEMM operand A)
-// and write the near-band part of Z.
+// and write the near-band part of Z.  As in the FP32 filter (tile_ramp) a
+// thread owns eight consecutive bins as packed pairs, and the windows of left
+// and right pairs slide by one pair a lag, here from the innermost lag
+// outward, in groups of four; the row is stored by pairs, de-interleaved by
+// pair index mod 4.  The eight bins are four odd and four even ones: two
+// 8-byte stores for each piece.  At 800 x 738 the kernel takes 6 us (10 with a
+// bin per thread: two shared loads for each lag held it to the load/store
+// pipe, 66-88 % busy).
 // measured: a slice descriptor whose sinogram y takes Y's place, or nullptr.
+constexpr int SN_PO = NEAR + 1;                     // sample offset of bin 0: odd, (SN_PO - 3) / 2 = 3 mod 4
+static_assert(NEAR == 64, "the near band is eight groups of four odd lags");
+__host__ __device__ inline int sn_pq(int kp) { return (SN_PO + kp + NEAR + 16) / 8 + 2; }   // pairs per residue
+
+__device__ __forceinline__ uint2 bf16x4(float a, float b, float c, float d) {
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(a, b), hi = __floats2bfloat162_rn(c, d);
+    return make_uint2(*reinterpret_cast<const unsigned *>(&lo), *reinterpret_cast<const unsigned *>(&hi));
+}
+
 __global__ void __launch_bounds__(256) k_split_near(const float *Y, const SliceDesc *measured, float *Z,
                                                     __nv_bfloat16 *__restrict__ A, const float *__restrict__ taps,
                                                     float near_diag, int nb, int kp, const CgState *cg,
                                                     int respect_stop) {
-    extern __shared__ __align__(16) float P[];    // [NEAR + nb + NEAR], zero padded
+    extern __shared__ __align__(16) float sm[];
+    const int PQ = sn_pq(kp), v = blockIdx.x;
+    unsigned long long *P = reinterpret_cast<unsigned long long *>(sm), *tp = P + 4 * PQ;   // pairs; {h, h} of lags 1, 3, ..
+    if (threadIdx.x < NEAR / 2) {
+        const float h = __ldg(taps + 2 * threadIdx.x + 1);
+        tp[threadIdx.x] = pair2(h, h);
+    }
     grid_wait();
     if (respect_stop && cg->stop) return;
-    const int v = blockIdx.x;
     const float *y = (measured ? measured->y : Y) + (size_t)v * nb;
-    for (int k = threadIdx.x; k < nb + 2 * NEAR; k += blockDim.x) {
-        const int i = k - NEAR;
-        P[k] = (i >= 0 && i < nb) ? ld_data(y + i) : 0.f;
+    auto half = [&](int k) { return sm + 2 * (((k >> 1) & 3) * PQ + (k >> 3)) + (k & 1); };
+    for (int k = threadIdx.x; k < 8 * PQ; k += blockDim.x) {
+        const int i = k - SN_PO;
+        *half(k) = (i >= 0 && i < nb) ? ld_data(y + i) : 0.f;
     }
     __syncthreads();
     __nv_bfloat16 *a = A + (size_t)v * 3 * kp;
-    for (int k = threadIdx.x; k < kp; k += blockDim.x) {
-        const float x = k < nb ? P[NEAR + k] : 0.f;
-        const __nv_bfloat16 h = __float2bfloat16_rn(x);
-        const float r1 = x - __bfloat162float(h);           // exact
-        const __nv_bfloat16 m = __float2bfloat16_rn(r1);
-        const float r2 = r1 - __bfloat162float(m);          // exact
-        const int col = a_col(k, kp / 2);
-        a[col] = h;
-        a[kp + col] = m;
-        a[2 * kp + col] = __float2bfloat16_rn(r2);
-    }
     float *z = Z + (size_t)v * nb;
-    float t[NEAR / 2];                                  // the odd-lag taps, in registers
+    const bool vec = (nb & 1) == 0;                 // rows start on 8-byte boundaries
+    for (int t = threadIdx.x; t < kp / 8; t += blockDim.x) {
+        const int j0 = 8 * t;
+        float c[8], r1[8], r2[8];
+        __nv_bfloat16 h[8];
 #pragma unroll
-    for (int q = 0; q < NEAR / 2; ++q) t[q] = __ldg(taps + 2 * q + 1);
-    for (int j = threadIdx.x; j < nb; j += blockDim.x) {
-        const float c = P[NEAR + j];
-        float acc = 0.f;
-#pragma unroll
-        for (int q = 0; q < NEAR / 2; ++q) {
-            const int m = 2 * q + 1;
-            acc = fmaf(t[q], __fadd_rn(__fsub_rn(P[NEAR + j - m], c), __fsub_rn(P[NEAR + j + m], c)), acc);
+        for (int i = 0; i < 8; ++i) {
+            c[i] = *half(SN_PO + j0 + i);
+            h[i] = __float2bfloat16_rn(c[i]);
+            r1[i] = c[i] - __bfloat162float(h[i]);                                // exact
+            r2[i] = r1[i] - __bfloat162float(__float2bfloat16_rn(r1[i]));         // exact
         }
-        z[j] = fmaf(near_diag, c, acc);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {               // odd bins first, then even ones
+            const int o = 1 - e;
+            uint2 *d = reinterpret_cast<uint2 *>(a + (e ? kp / 2 : 0) + j0 / 2);
+            d[0] = bf16x4(c[o], c[o + 2], c[o + 4], c[o + 6]);
+            d[kp / 4] = bf16x4(r1[o], r1[o + 2], r1[o + 4], r1[o + 6]);
+            d[2 * (kp / 4)] = bf16x4(r2[o], r2[o + 2], r2[o + 4], r2[o + 6]);
+        }
+        if (j0 >= nb) continue;
+        unsigned long long nc[4], L[4], R[4], acc[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            nc[q] = pair2(-c[2 * q], -c[2 * q + 1]);
+            acc[q] = 0ull;
+            L[q] = P[q * PQ + t + 8];                                  // samples j0 + 2 q - 1: pair 32 + q
+            R[q] = P[((q + 1) & 3) * PQ + t + 8 + (q + 1) / 4];        // samples j0 + 2 q + 1: pair 33 + q
+        }
+        const unsigned long long *pl = P + t + 7, *pr = P + t + 9;
+#pragma unroll 1
+        for (int i = 0; i < NEAR / 2; i += 4) {
+            const ulonglong2 h01 = *reinterpret_cast<const ulonglong2 *>(tp + i),
+                             h23 = *reinterpret_cast<const ulonglong2 *>(tp + i + 2);
+            const unsigned long long hh[4] = {h01.x, h01.y, h23.x, h23.y};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    acc[q] = fma2(hh[u], add2(add2(L[q], nc[q]), add2(R[q], nc[q])), acc[q]);
+#pragma unroll
+                for (int q = 3; q > 0; --q) L[q] = L[q - 1];
+                L[0] = pl[(3 - u) * PQ];                               // pair 31 - i
+#pragma unroll
+                for (int q = 0; q < 3; ++q) R[q] = R[q + 1];
+                R[3] = u < 3 ? pr[(u + 1) * PQ] : pr[1];               // pair 37 + i
+            }
+            pl -= 1;
+            pr += 1;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float2 s = unpair2(acc[q]);
+            const float2 o = make_float2(fmaf(near_diag, c[2 * q], s.x), fmaf(near_diag, c[2 * q + 1], s.y));
+            if (vec && j0 + 2 * q < nb) {
+                *reinterpret_cast<float2 *>(z + j0 + 2 * q) = o;
+            } else {
+                if (j0 + 2 * q < nb) z[j0 + 2 * q] = o.x;
+                if (j0 + 2 * q + 1 < nb) z[j0 + 2 * q + 1] = o.y;
+            }
+        }
     }
 }
 
@@ -361,6 +423,8 @@ k_ramp_gemm(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
 }
 
 // ------------------------------------------------------------ host side
+size_t split_smem(int kp) { return 8 * (4 * (size_t)sn_pq(kp) + NEAR / 2); }
+
 uint16_t bf16_rn(float x) {   // round-to-nearest-even to BF16 (finite inputs)
     uint32_t u;
     std::memcpy(&u, &x, 4);
@@ -457,7 +521,7 @@ air_status ramp_tc_create(air_plan *P) {
         e = cudaFuncSetAttribute(k_ramp_gemm, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM);
         if (e == cudaSuccess)   // the largest any plan needs: the limit is per kernel, not per plan
             e = cudaFuncSetAttribute(k_split_near, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)((RAMP_MAX_BINS + 2 * NEAR) * sizeof(float)));
+                                     (int)split_smem(RAMP_MAX_BINS));
     }
     if (e != cudaSuccess || !maps) {
         cudaFree(R->mem);
@@ -485,7 +549,7 @@ air_status ramp_tc_apply(const air_plan *P, const float *src, const SliceDesc *m
     const TcRes *R = static_cast<const TcRes *>(P->tc);
     if (!R) return fail(AIR_ERR_INVALID_ARG, "plan has no tensor-core filter");
     const int V = P->geom.n_views, nb = P->geom.n_bins;
-    cudaError_t e = launch_overlapped(k_split_near, dim3(V), dim3(256), (nb + 2 * NEAR) * sizeof(float), true, st, src,
+    cudaError_t e = launch_overlapped(k_split_near, dim3(V), dim3(std::min(256, (R->kp / 8 + 31) / 32 * 32)), split_smem(R->kp), true, st, src,
                                       measured, dst, R->a, R->near_taps, R->near_diag, nb, R->kp, cg, respect_stop);
     const dim3 grid((V + TM - 1) / TM, R->np / TN);   // both parities: 2 x (np / 2) / TN
     if (e == cudaSuccess)

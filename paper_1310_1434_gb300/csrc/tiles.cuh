@@ -450,12 +450,6 @@ __host__ __device__ inline int ramp_lags(int nb) { return nb < 2 ? 4 : (nb / 2 +
 __host__ __device__ inline int ramp_pad(int nb) { return 2 * ramp_lags(nb) - 1; }
 __host__ __device__ inline int ramp_pq(int nb) { return (2 * ramp_pad(nb) + (nb + 7) / 8 * 8) / 8 + 2; }
 
-__device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {
-    unsigned long long d;
-    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
-    return d;
-}
-
 // Where the filter's result of sample i goes: its row, or (ARG_PACK) its place
 // among the orbits' packed samples, times the ray's c.
 __device__ __forceinline__ void put_filtered(const SliceDesc &s, bool pack, float *dst, size_t i, float v) {
@@ -496,6 +490,7 @@ __device__ __forceinline__ void tile_ramp(const SliceDesc &s, int arg, int tile,
     }
     __syncthreads();
     const float diag = s.ramp_diag;
+    const bool vec = !pack && (nb & 1) == 0;       // rows start on 8-byte boundaries
 #pragma unroll 1
     for (int j0 = threadIdx.x * RAMP_R; j0 < nb; j0 += AIR_THREADS * RAMP_R) {
         // lags from the outermost inward: the terms grow as the lag shrinks
@@ -538,8 +533,14 @@ __device__ __forceinline__ void tile_ramp(const SliceDesc &s, int arg, int tile,
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const float2 a = unpair2(acc[q]);
-            if (j0 + 2 * q < nb) put_filtered(s, pack, dst, off + j0 + 2 * q, fmaf(diag, ctr[2 * q], a.x));
-            if (j0 + 2 * q + 1 < nb) put_filtered(s, pack, dst, off + j0 + 2 * q + 1, fmaf(diag, ctr[2 * q + 1], a.y));
+            const float2 o = make_float2(fmaf(diag, ctr[2 * q], a.x), fmaf(diag, ctr[2 * q + 1], a.y));
+            const size_t i = off + j0 + 2 * q;
+            if (vec && j0 + 2 * q < nb) {
+                *reinterpret_cast<float2 *>(dst + i) = o;
+            } else {
+                if (j0 + 2 * q < nb) put_filtered(s, pack, dst, i, o.x);
+                if (j0 + 2 * q + 1 < nb) put_filtered(s, pack, dst, i + 1, o.y);
+            }
         }
     }
     __syncthreads();

@@ -4,25 +4,9 @@
 #pragma once
 
 #include "air_internal.cuh"
+#include "packed.cuh"
 
 namespace air {
-
-// Two FP32 FMAs in one instruction, each rounded as fmaf.
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b, unsigned long long c) {
-    unsigned long long d;
-    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
-    return d;
-}
-__device__ __forceinline__ unsigned long long pair2(float x, float y) {
-    unsigned long long d;
-    asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(x), "f"(y));
-    return d;
-}
-__device__ __forceinline__ float2 unpair2(unsigned long long d) {
-    float2 f;
-    asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(d));
-    return f;
-}
 
 // Physical pixel of the canonical pixel (k, r) in a frame.
 __device__ __forceinline__ void orb_pixel(int code, int n, int k, int r, int &ix, int &iy) {
