@@ -129,13 +129,10 @@ __device__ __forceinline__ bool reduce_tiles(const SliceDesc &s, int tile, int n
     __shared__ int last;
     if (threadIdx.x == 0) {
         s.partial[tile] = val;
-        __threadfence();
-        const unsigned prev = atomicAdd(&s.cg->counter, 1u);
-        last = prev == (unsigned)(ntiles - 1);
+        last = count_in(&s.cg->counter) == (unsigned)(ntiles - 1);
     }
     __syncthreads();
     if (!last) return false;
-    __threadfence();
     double v = 0.0;
     for (int i = threadIdx.x; i < ntiles; i += AIR_THREADS) v += __ldcg(s.partial + i);
     v = block_sum(v, sh);
