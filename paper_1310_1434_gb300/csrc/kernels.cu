@@ -31,11 +31,16 @@ static cudaError_t opt_in_smem(Kernel kernel, std::atomic<unsigned long long> &d
 template <int OP>
 constexpr int min_blocks = OP == OP_ORB_BWD || OP == OP_ORB_FWD ? 3 : 0;
 
+// These tile functions wait for the kernel before themselves (grid_wait),
+// once they have read what they need of the plan's tables.
+template <int OP>
+constexpr bool own_wait = OP == OP_FWD || OP == OP_RAMP || OP == OP_ORB_ZPACK || OP == OP_ORB_BWD;
+
 template <int OP>
 __global__ void __launch_bounds__(AIR_THREADS, min_blocks<OP>) k_op(const SliceDesc s, int arg) {
     extern __shared__ __align__(16) float sm[];
     const int tile = blockIdx.x;
-    grid_wait();
+    if constexpr (!own_wait<OP>) grid_wait();
     if constexpr (OP == OP_FWD) {
         tile_fwd(s, arg, tile);
     } else if constexpr (OP == OP_RAMP) {
@@ -156,7 +161,8 @@ k_group(const SliceDesc *__restrict__ slices, const Task *__restrict__ tasks, in
     int staged = -1;
     const SliceDesc &s = stage_desc(slices, t.slice, &sd, &staged);
     const int tile = b - t.tile0;
-    grid_wait();     // the tables above are written by copies, which no kernel overlaps
+    // (the tables above are written by copies, which no kernel overlaps)
+    if constexpr (!own_wait<OP>) grid_wait();
     if constexpr (OP == OP_FWD) tile_fwd(s, t.arg, tile);
     else if constexpr (OP == OP_RAMP) tile_ramp(s, t.arg, tile, sm);
     else if constexpr (OP == OP_BWD) tile_bwd(s, t.arg, tile, sm);

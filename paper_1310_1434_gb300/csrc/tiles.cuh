@@ -74,7 +74,6 @@ __device__ __forceinline__ float fx_ray(const float2 *XP, const float2 *XTP, int
 }
 
 __device__ __forceinline__ void tile_fwd(const SliceDesc &s, int arg, int tile) {
-    if (arg == SRC_P && s.cg->stop) return;
     float *dst = arg == SRC_EXT ? s.ext_out : s.z;
     // tile = (view group, bin range); a warp holds neighbouring bins of one
     // view, and the warps of a block neighbouring views, whose rays walk
@@ -83,11 +82,14 @@ __device__ __forceinline__ void tile_fwd(const SliceDesc &s, int arg, int tile) 
     const int nbt = (s.nb + bpb - 1) / bpb;
     const int v = (tile / nbt) * s.fwd_vpb + threadIdx.x / bpb;
     const int j = (tile % nbt) * bpb + threadIdx.x % bpb;
-    if (v >= s.V || j >= s.nb) return;
-    const int idx = v * s.nb + j;
+    const bool in = v < s.V && j < s.nb;
+    const int idx = in ? v * s.nb + j : 0;
     const RayFx r = s.ray[idx];
+    const unsigned walk = __ldg(s.walk + idx);
+    grid_wait();
+    if (!in || (arg == SRC_P && s.cg->stop)) return;
     dst[idx] = s.dx * (fabsf(r.cs) * fx_ray(reinterpret_cast<const float2 *>(s.xp),
-                                            reinterpret_cast<const float2 *>(s.xt), s.n, r, __ldg(s.walk + idx)));
+                                            reinterpret_cast<const float2 *>(s.xt), s.n, r, walk));
 }
 
 // xp and xt: the pair copies of src and of its transpose (pair r + 1 of a
@@ -96,15 +98,24 @@ __device__ __forceinline__ void tile_fwd(const SliceDesc &s, int arg, int tile) 
 // shared memory; runs before every projection.  The two ends that hold no
 // pixel (X[-1] and X[n]) are zeroed once with the plan.
 __device__ __forceinline__ void tile_transpose(const SliceDesc &s, int arg, int tile, float *sm) {
-    if (arg == SRC_P && s.cg->stop) return;
+    const int stop = arg == SRC_P ? s.cg->stop : 0;
     const float *src = arg == SRC_X ? s.x : (arg == SRC_P ? s.p : s.ext_in);
     const int n = s.n, tpr = (n + 31) / 32, ld = 2 * pair_ld(n);   // floats per row of pairs
     const int x0 = (tile % tpr) * 32, y0 = (tile / tpr) * 32;
     float(*t)[33] = reinterpret_cast<float(*)[33]>(sm);
     const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    for (int yy = ty; yy < 32; yy += AIR_THREADS / 32)
-        if (y0 + yy < n && x0 + tx < n) {
-            const float v = src[(size_t)(y0 + yy) * n + x0 + tx];
+    constexpr int ROWS = 32 / (AIR_THREADS / 32);
+    float in[ROWS];                                      // on their way together, and with stop
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q) {
+        const int yy = ty + q * (AIR_THREADS / 32);
+        in[q] = y0 + yy < n && x0 + tx < n ? ld_data(src + (size_t)(y0 + yy) * n + x0 + tx) : 0.f;
+    }
+    if (stop) return;
+#pragma unroll
+    for (int q = 0; q < ROWS; ++q)
+        if (const int yy = ty + q * (AIR_THREADS / 32); y0 + yy < n && x0 + tx < n) {
+            const float v = in[q];
             t[yy][tx] = v;
             float *row = s.xp + (size_t)(y0 + yy) * ld;       // X[x] is pair x+1 .x and pair x .y
             row[2 * (x0 + tx + 1)] = v;
@@ -349,7 +360,7 @@ __device__ __forceinline__ void tile_bwd(const SliceDesc &s, int mode, int tile,
 // whose tuned split, and with it the order of its sums, follows this sum's
 // time.
 template <int N>
-__device__ __forceinline__ double bwd_fin(const SliceDesc &s, int mode, bool swap, int i) {
+__device__ __forceinline__ double bwd_fin(const SliceDesc &s, int mode, bool swap, int stop, int i) {
     struct __align__(4 * N) Vec { float v[N]; };
     auto get = [&](const float *a) { return *reinterpret_cast<const Vec *>(a + i); };
     auto put = [&](float *a, const Vec &x) { *reinterpret_cast<Vec *>(a + i) = x; };
@@ -375,7 +386,7 @@ __device__ __forceinline__ double bwd_fin(const SliceDesc &s, int mode, bool swa
 #pragma unroll
         for (int q = 0; q < N; ++q) o.v[q] = fmaf(s.step, b.v[q] - a.v[q], x.v[q]);
         put(s.q, o);
-    } else {  // BWD_Q
+    } else if (!stop) {  // BWD_Q
         const Vec p = get(swap ? s.q : s.p);
         Vec o;
 #pragma unroll
@@ -392,20 +403,20 @@ __device__ __forceinline__ void tile_bwd_fin(const SliceDesc &s, int arg, int ti
     __shared__ double sh[AIR_THREADS / 32];
     const int mode = arg & ARG_MASK;
     const bool swap = (arg & ARG_SWAP) != 0;
-    if (mode == BWD_Q && s.cg->stop) return;
+    const int stop = mode == BWD_Q ? s.cg->stop : 0;     // on its way with the parts
     const int nn = s.n * s.n, base = tile * VEC_PER_TILE;
     double part = 0.0;
     if (s.orb && nn % 4 == 0) {
         const int i = base + 4 * (int)threadIdx.x;
-        if (i < nn) part = bwd_fin<4>(s, mode, swap, i);
+        if (i < nn) part = bwd_fin<4>(s, mode, swap, stop, i);
     } else {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int i = base + k * AIR_THREADS + (int)threadIdx.x;
-            if (i < nn) part += bwd_fin<1>(s, mode, swap, i);
+            if (i < nn) part += bwd_fin<1>(s, mode, swap, stop, i);
         }
     }
-    if (mode == BWD_PLAIN || mode == BWD_RHS0 || mode == BWD_STEP) return;
+    if (stop || mode == BWD_PLAIN || mode == BWD_RHS0 || mode == BWD_STEP) return;
     part = block_sum(part, sh);
     double tot;
     if (reduce_tiles(s, tile, tiles_vec(s), part, sh, &tot) && threadIdx.x == 0) {
@@ -465,8 +476,9 @@ __device__ __forceinline__ void tile_ramp(const SliceDesc &s, int arg, int tile,
     float *dst = arg == RSRC_EXT ? s.ext_out : s.zc;
     const int nb = s.nb;
     const size_t off = (size_t)tile * nb;
-    if (arg == RSRC_Z && s.cg->stop) return;
     if (!s.filter) {
+        grid_wait();
+        if (arg == RSRC_Z && s.cg->stop) return;
         for (int j = threadIdx.x; j < nb; j += AIR_THREADS) put_filtered(s, pack, dst, off + j, src[off + j]);
         return;
     }
@@ -476,16 +488,19 @@ __device__ __forceinline__ void tile_ramp(const SliceDesc &s, int arg, int tile,
     // k & 1 of pair k / 2
     auto half = [&](int k) { return sm + 2 * (((k >> 1) & 3) * PQ + (k >> 3)) + (k & 1); };
     const float *__restrict__ pw = s.prew;
-    for (int k = threadIdx.x; k < 8 * PQ; k += AIR_THREADS) {
-        const int i = k - PO;
-        *half(k) = (i >= 0 && i < nb) ? (pw ? src[off + i] * __ldg(pw + i) : src[off + i]) : 0.f;
-    }
     for (int i = threadIdx.x; i < lags; i += AIR_THREADS) {
         const int m = PO - 2 * i;
         const float h = m < nb ? __ldg(s.taps + m) : 0.f;
         tp[i] = pair2(h, h);
     }
+    grid_wait();
+    const int stop = arg == RSRC_Z ? s.cg->stop : 0;     // on its way with the row
+    for (int k = threadIdx.x; k < 8 * PQ; k += AIR_THREADS) {
+        const int i = k - PO;
+        *half(k) = (i >= 0 && i < nb) ? (pw ? src[off + i] * __ldg(pw + i) : src[off + i]) : 0.f;
+    }
     __syncthreads();
+    if (stop) return;
     const float diag = s.ramp_diag;
     const bool vec = !pack && (nb & 1) == 0;       // rows start on 8-byte boundaries
 #pragma unroll 1
@@ -593,18 +608,29 @@ __device__ __forceinline__ void tile_fbp(const SliceDesc &s, int tile) {
 // ======================================================================
 __device__ __forceinline__ void tile_cg_a(const SliceDesc &s, int arg, int tile) {
     __shared__ double sh[AIR_THREADS / 32];
-    if (s.cg->stop) return;
+    const int stop = s.cg->stop;
     const float a = (float)s.cg->alpha;
     const float *pv = arg & ARG_SWAP ? s.q : s.p, *qv = arg & ARG_SWAP ? s.p : s.q;
     const int nn = s.n * s.n;
     const int base = tile * VEC_PER_TILE;
+    // the state and the vectors are read together: one memory latency
+    float p4[4], q4[4], x4[4], r4[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int i = min(base + k * AIR_THREADS + (int)threadIdx.x, nn - 1);
+        p4[k] = ld_data(pv + i);
+        q4[k] = ld_data(qv + i);
+        x4[k] = ld_data(s.x + i);
+        r4[k] = ld_data(s.r + i);
+    }
+    if (stop) return;
     double part = 0.0;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int i = base + k * AIR_THREADS + threadIdx.x;
         if (i < nn) {
-            s.x[i] = fmaf(a, pv[i], s.x[i]);
-            const float rv = fmaf(-a, qv[i], s.r[i]);
+            s.x[i] = fmaf(a, p4[k], x4[k]);
+            const float rv = fmaf(-a, q4[k], r4[k]);
             s.r[i] = rv;
             part += (double)rv * (double)rv;
         }
@@ -620,14 +646,22 @@ __device__ __forceinline__ void tile_cg_a(const SliceDesc &s, int arg, int tile)
 }
 
 __device__ __forceinline__ void tile_cg_b(const SliceDesc &s, int tile) {
-    if (s.cg->stop) return;
+    const int stop = s.cg->stop;
     const float bt = (float)s.cg->beta;
     const int nn = s.n * s.n;
     const int base = tile * VEC_PER_TILE;
+    float p4[4], r4[4];                                   // as in tile_cg_a
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int i = min(base + k * AIR_THREADS + (int)threadIdx.x, nn - 1);
+        p4[k] = ld_data(s.p + i);
+        r4[k] = ld_data(s.r + i);
+    }
+    if (stop) return;
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
         const int i = base + k * AIR_THREADS + threadIdx.x;
-        if (i < nn) s.p[i] = fmaf(bt, s.p[i], s.r[i]);
+        if (i < nn) s.p[i] = fmaf(bt, p4[k], r4[k]);
     }
 }
 

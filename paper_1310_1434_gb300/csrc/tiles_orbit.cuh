@@ -25,7 +25,7 @@ __device__ __forceinline__ void tile_orb_pack(const SliceDesc &s, int arg, int t
     const bool swap = (arg & ARG_SWAP) != 0;
     arg &= ARG_MASK;
     const bool cg = arg == SRC_P || arg == SRC_P_NEXT, next = arg == SRC_P_NEXT;
-    if (cg && s.cg->stop) return;
+    const int stop = cg ? s.cg->stop : 0;
     // SRC_P_NEXT: p = r + beta p on the way, from the image that held it to the
     // other one; plane 0 writes what it reads for its first frame, every pixel
     // once.  (Folded into the general path's copies it gained nothing.)
@@ -37,23 +37,38 @@ __device__ __forceinline__ void tile_orb_pack(const SliceDesc &s, int arg, int t
     const int k0 = (t % tpr) * 32, r0 = (t / tpr) * 32;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     float(*f)[32][33] = reinterpret_cast<float(*)[32][33]>(sm);   // [frame][k][r]
+    constexpr int STEP = AIR_THREADS / 32, ROWS = 32 / STEP;
+    float in[4][ROWS], res[4][ROWS];                     // on their way together, and with stop
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
         const int code = s.orb_frame[4 * plane + q];
         const bool tr = (code & ORB_T) != 0;
 #pragma unroll
-        for (int m = 0; m < 32; m += AIR_THREADS / 32) {
-            const int kk = tr ? w + m : lane, rr = tr ? lane : w + m;
-            float v = 0.f;
+        for (int m = 0; m < ROWS; ++m) {
+            const int kk = tr ? w + m * STEP : lane, rr = tr ? lane : w + m * STEP;
+            in[q][m] = res[q][m] = 0.f;
             if (k0 + kk < n && r0 + rr < n) {
                 int ix, iy;
                 orb_pixel(code, n, k0 + kk, r0 + rr, ix, iy);
                 const size_t i = (size_t)iy * n + ix;
-                v = src[i];
-                if (next) {
-                    v = fmaf(bt, v, s.r[i]);
-                    if (plane == 0 && q == 0) to[i] = v;
-                }
+                in[q][m] = ld_data(src + i);
+                if (next) res[q][m] = ld_data(s.r + i);
+            }
+        }
+    }
+    if (stop) return;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        const int code = s.orb_frame[4 * plane + q];
+        const bool tr = (code & ORB_T) != 0;
+#pragma unroll
+        for (int m = 0; m < ROWS; ++m) {
+            const int kk = tr ? w + m * STEP : lane, rr = tr ? lane : w + m * STEP;
+            const float v = next ? fmaf(bt, in[q][m], res[q][m]) : in[q][m];
+            if (next && plane == 0 && q == 0 && k0 + kk < n && r0 + rr < n) {
+                int ix, iy;
+                orb_pixel(code, n, k0 + kk, r0 + rr, ix, iy);
+                to[(size_t)iy * n + ix] = v;
             }
             f[q][kk][rr] = v;
         }
@@ -274,6 +289,7 @@ __device__ __forceinline__ void orb_rows(int d, float f0, float f1, float &lo, f
 constexpr int ORB_SEGS = 4;                              // segments staged at a time
 constexpr int ORB_STAGES = 3;
 constexpr int ORB_ROWS = 4;                              // pixels of a thread, along r
+constexpr int ORB_EARLY = 152;                           // blocks of a launch that leaves SMs idle: one per SM
 constexpr int ORB_ENT = ORB_RAYS + ORB_CAND;             // staged rays of a segment
 
 constexpr int ORB_PATCH_K = 8, ORB_PATCH_R = 16;         // pixels of a warp
@@ -291,14 +307,14 @@ __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
 // Samples of the orbits' rays side by side: orb_z[plane][padded ray] = c times
 // the four samples of the plane's frames, zero for the empty rays.
 __device__ __forceinline__ void tile_orb_zpack(const SliceDesc &s, int mode, int tile) {
-    if (mode == BWD_Q && s.cg->stop) return;
     const float *Z = mode == BWD_PLAIN ? s.ext_in : s.zc;
     const int nch = orb_zchunks(s), seg = tile / nch;
     const OrbSeg &g = s.orb_seg[seg];
     const int i = (tile - seg * nch) * ORB_ZPACK + (int)threadIdx.x;
-    if (i >= g.cnt + ORB_CAND) return;
     const float c = i < g.cnt ? __ldg(&s.orb_ray[g.ray0 + i].cs) : 0.f;
     const int down = g.down;
+    grid_wait();
+    if (i >= g.cnt + ORB_CAND || (mode == BWD_Q && s.cg->stop)) return;
     for (int p = 0; p < orb_planes(s); ++p) {
         float v[4];
 #pragma unroll
@@ -326,7 +342,7 @@ __device__ __forceinline__ float atan_series(float u) {
 __device__ __forceinline__ float orb_atan(float u) { return fabsf(u) <= 0.45f ? atan_series(u) : atanf(u); }
 
 template <int NF>
-__device__ __forceinline__ void tile_orb_bwd_nf(const SliceDesc &s, int tile, float *sm) {
+__device__ __forceinline__ void tile_orb_bwd_nf(const SliceDesc &s, int mode, int tile, float *sm) {
     constexpr int NV = NF / 4;                           // float4s of samples per ray
     constexpr int SEG = ORB_ENT * (1 + NV) + ORB_PAR;    // float4s of a staged segment
     const int n = s.n, ntxy = tiles_bwd_xy(s), S = s.orb_splits;
@@ -340,12 +356,15 @@ __device__ __forceinline__ void tile_orb_bwd_nf(const SliceDesc &s, int tile, fl
     const int e0 = __ldg(s.orb_tile0 + cls * (ntxy + 1) + txy), e1 = __ldg(s.orb_tile0 + cls * (ntxy + 1) + txy + 1);
     const int ne = e1 - e0 > split ? (e1 - e0 - split + S - 1) / S : 0;      // this split's entries
     const uint2 *__restrict__ ent = s.orb_ent + e0 + split;                  // every S-th
-    const int rounds = (ne + ORB_SEGS - 1) / ORB_SEGS;
     float4 *buf = reinterpret_cast<float4 *>(sm);
 
     // warps 2 q and 2 q + 1 stage the round's segment q; warp `round` mod 8
-    // writes every warp's parameters of the four segments
-    auto stage = [&](int round) {
+    // writes every warp's parameters of the four segments.  The rays and the
+    // parameters come from the plan's tables: those of the first two rounds
+    // are asked for before the wait for the last kernel where a launch leaves
+    // SMs idle (128^2 / 90 views: 734 -> 703 us for 20 CG steps; a launch of
+    // more than a block per SM lost half a percent by it).
+    auto stage = [&](int round, bool rays, bool samples) {
         const int e = round * ORB_SEGS + (warp >> 1);
         float4 *ring = buf + (round % ORB_STAGES) * ORB_SEGS * SEG;
         if (e < ne) {
@@ -353,12 +372,12 @@ __device__ __forceinline__ void tile_orb_bwd_nf(const SliceDesc &s, int tile, fl
             const int m = (int)((w.x >> 17) & 0x7fu) + ORB_CAND;
             float4 *st = ring + (warp >> 1) * SEG;
             for (int i = (warp & 1) * 32 + lane; i < m; i += 64) {
-                cp_async16(st + i, s.orb_bray + w.y + i);
+                if (rays) cp_async16(st + i, s.orb_bray + w.y + i);
 #pragma unroll
-                for (int v = 0; v < NV; ++v) cp_async16(st + ORB_ENT * (1 + v) + i, s.orb_z + (size_t)v * s.orb_npad + w.y + i);
+                for (int v = 0; v < NV && samples; ++v) cp_async16(st + ORB_ENT * (1 + v) + i, s.orb_z + (size_t)v * s.orb_npad + w.y + i);
             }
         }
-        if ((round & 7) == warp) {
+        if (rays && (round & 7) == warp) {
             const int q = lane >> 3, pw = lane & 7, eq = round * ORB_SEGS + q;   // segment, warp
             if (eq < ne) {
                 // the ray index over warp pw's pixels, to second order about
@@ -378,7 +397,7 @@ __device__ __forceinline__ void tile_orb_bwd_nf(const SliceDesc &s, int tile, fl
                                      __uint_as_float((w.x >> 17) & 0x7fu), 0.f);
             }
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
+        if (samples) asm volatile("cp.async.commit_group;" ::: "memory");
     };
 
     unsigned long long acc[ORB_ROWS][NF / 2];
@@ -387,16 +406,24 @@ __device__ __forceinline__ void tile_orb_bwd_nf(const SliceDesc &s, int tile, fl
 #pragma unroll
         for (int f = 0; f < NF / 2; ++f) acc[q][f] = 0ull;
 
-    stage(0);
-    stage(1);
+    const bool early = gridDim.x <= ORB_EARLY;
+    if (early) {
+        stage(0, true, false);
+        stage(1, true, false);
+    }
+    grid_wait();
+    const int stop = mode == BWD_Q ? s.cg->stop : 0;     // on its way with the first rounds
+    stage(0, !early, true);
+    stage(1, !early, true);
     // the thread's column and first row from the middle of its warp's pixels
     const float u = (float)(lane & 7) - 0.5f * (ORB_PATCH_K - 1);
     const float v0 = (float)((lane >> 3) * ORB_ROWS) - 0.5f * (ORB_PATCH_R - 1);
+    const int rounds = stop ? 0 : (ne + ORB_SEGS - 1) / ORB_SEGS;
 #pragma unroll 1
     for (int round = 0; round < rounds; ++round) {
         asm volatile("cp.async.wait_group 1;" ::: "memory");
         __syncthreads();             // this round's rays are there; the last round's buffer is free
-        stage(round + 2);
+        stage(round + 2, true, true);
         const int m = min(ORB_SEGS, ne - round * ORB_SEGS);
 #pragma unroll 1
         for (int q = 0; q < m; ++q) {
@@ -439,7 +466,7 @@ __device__ __forceinline__ void tile_orb_bwd_nf(const SliceDesc &s, int tile, fl
             }
         }
     }
-    if (k < n) {
+    if (k < n && !stop) {
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
             float *img = s.bwd_part + (size_t)(split * 8 + cls * 4 + f) * n * n;
@@ -459,9 +486,8 @@ __device__ __forceinline__ void tile_orb_bwd_nf(const SliceDesc &s, int tile, fl
 }
 
 __device__ __forceinline__ void tile_orb_bwd(const SliceDesc &s, int mode, int tile, float *sm) {
-    if (mode == BWD_Q && s.cg->stop) return;
-    if (s.orb == 8) tile_orb_bwd_nf<8>(s, tile, sm);
-    else tile_orb_bwd_nf<4>(s, tile, sm);
+    if (s.orb == 8) tile_orb_bwd_nf<8>(s, mode, tile, sm);
+    else tile_orb_bwd_nf<4>(s, mode, tile, sm);
 }
 
 // ======================================================================
