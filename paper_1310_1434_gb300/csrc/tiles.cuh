@@ -354,12 +354,17 @@ __device__ __forceinline__ void tile_bwd(const SliceDesc &s, int mode, int tile,
 
 // Sums the parts of the backprojection (bwd_images of them) in a fixed order
 // and applies the mode's epilogue (the CG and residual updates of the Eq. 5
-// system).  A thread takes N neighbouring pixels: four with 16-byte accesses
-// for the orbit path's eight images and more, where the image's size keeps
-// them aligned (24 images at 512^2: 19 -> 9 us); one for the general path,
-// whose tuned split, and with it the order of its sums, follows this sum's
-// time.
-template <int N>
+// system).  Bound by the latency of the images' loads: a thread takes N = 4
+// neighbouring pixels where the image's size keeps them aligned, and asks for
+// U = 8 images at a time (the compiler's own unrolling kept fewer in flight).
+// 24 images at 512^2 took 19 us pixel by pixel; 20 CG steps at 350^2 / 200
+// views 1391 us with the compiler's unrolling and 1371 so, a solve with
+// history at 128^2 / 90 views (90 parts) 484 us pixel by pixel and 454.  16 or
+// 24 images at a time cost registers and gained nothing.  The general path's
+// rhs0 stays pixel by pixel: its split, and with it the order of its sums, is
+// tuned on this sum's time there.  The persistent kernel's one register budget
+// has no room for U images (U = 1).
+template <int N, int U>
 __device__ __forceinline__ double bwd_fin(const SliceDesc &s, int mode, bool swap, int stop, int i) {
     struct __align__(4 * N) Vec { float v[N]; };
     auto get = [&](const float *a) { return *reinterpret_cast<const Vec *>(a + i); };
@@ -367,11 +372,26 @@ __device__ __forceinline__ double bwd_fin(const SliceDesc &s, int mode, bool swa
     const int S = bwd_images(s);
     const size_t nn = (size_t)s.n * s.n;
     Vec a{};
-#pragma unroll (N == 4 ? 8 : 4)
-    for (int p = 0; p < S; ++p) {
-        const Vec x = get(s.bwd_part + p * nn);
+    if constexpr (U > 1) {
+#pragma unroll 1
+        for (int p = 0; p < S; p += U) {
+            Vec x[U];
 #pragma unroll
-        for (int q = 0; q < N; ++q) a.v[q] += x.v[q];
+            for (int u = 0; u < U; ++u)
+                if (p + u < S) x[u] = get(s.bwd_part + (p + u) * nn);
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (p + u < S)
+#pragma unroll
+                    for (int q = 0; q < N; ++q) a.v[q] += x[u].v[q];
+        }
+    } else {
+#pragma unroll (N == 4 ? 8 : 4)
+        for (int p = 0; p < S; ++p) {
+            const Vec x = get(s.bwd_part + p * nn);
+#pragma unroll
+            for (int q = 0; q < N; ++q) a.v[q] += x.v[q];
+        }
     }
 #pragma unroll
     for (int q = 0; q < N; ++q) a.v[q] *= s.dx;
@@ -399,6 +419,8 @@ __device__ __forceinline__ double bwd_fin(const SliceDesc &s, int mode, bool swa
     return part;
 }
 
+constexpr int FIN_IMAGES = 8;
+template <int U>
 __device__ __forceinline__ void tile_bwd_fin(const SliceDesc &s, int arg, int tile) {
     __shared__ double sh[AIR_THREADS / 32];
     const int mode = arg & ARG_MASK;
@@ -406,14 +428,14 @@ __device__ __forceinline__ void tile_bwd_fin(const SliceDesc &s, int arg, int ti
     const int stop = mode == BWD_Q ? s.cg->stop : 0;     // on its way with the parts
     const int nn = s.n * s.n, base = tile * VEC_PER_TILE;
     double part = 0.0;
-    if (s.orb && nn % 4 == 0) {
+    if ((s.orb || mode != BWD_RHS0) && nn % 4 == 0) {
         const int i = base + 4 * (int)threadIdx.x;
-        if (i < nn) part = bwd_fin<4>(s, mode, swap, stop, i);
+        if (i < nn) part = bwd_fin<4, U>(s, mode, swap, stop, i);
     } else {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int i = base + k * AIR_THREADS + (int)threadIdx.x;
-            if (i < nn) part += bwd_fin<1>(s, mode, swap, stop, i);
+            if (i < nn) part += bwd_fin<1, 1>(s, mode, swap, stop, i);
         }
     }
     if (stop || mode == BWD_PLAIN || mode == BWD_RHS0 || mode == BWD_STEP) return;
@@ -1034,7 +1056,7 @@ __device__ __forceinline__ void run_tile(const SliceDesc &s, int op, int arg, in
     case OP_TRANSPOSE: tile_transpose(s, arg, tile, sm); break;
     case OP_RAMP: tile_ramp(s, arg, tile, sm); break;
     case OP_BWD: tile_bwd(s, arg, tile, sm); break;
-    case OP_BWD_FIN: tile_bwd_fin(s, arg, tile); break;
+    case OP_BWD_FIN: tile_bwd_fin<1>(s, arg, tile); break;
     case OP_CG_A: tile_cg_a(s, arg, tile); break;
     case OP_CG_B: tile_cg_b(s, tile); break;
     case OP_ZERO: tile_zero(s, tile); break;
