@@ -170,7 +170,7 @@ def run_kernel(args):
     ell, _, Y = inputs.make_case(w)
     X = inputs.rasterize(g, ell)
     plan = air.Plan(g)
-    if args.kernel == "bwd":   # the view split bench.py's roofline times
+    if args.kernel == "bwd":   # the split bench.py's roofline times
         vpb, _, s_max = air.air_plan_config(plan)
         air.air_plan_tune(plan, vpb, min(BWD_PARTS, s_max))
     Yd = torch.as_tensor(Y.astype(np.float32).ravel(), device="cuda")
@@ -675,9 +675,8 @@ def main():
     xout = torch.empty(g8.n ** 2, device=dev)
     air.air_backproject(p800, zin, xout)
     t_bwd_tuned = events_time(torch, stream, lambda: air.air_backproject(p800, zin, xout), 20)
-    # the roofline's configuration: BWD_PARTS view parts in one k_op<OP_BWD>
-    # launch plus their sum (k_op<OP_BWD_FIN>), as `--kernel bwd` runs it for
-    # the ncu capture
+    # the roofline's configuration: OP_ORB_ZPACK, OP_ORB_BWD to BWD_PARTS images
+    # and their sum OP_BWD_FIN, as `--kernel bwd` runs it for the ncu capture
     vpb, s_tuned, s_max = air.air_plan_config(p800)
     s_rf = min(BWD_PARTS, s_max)
     air.air_plan_tune(p800, vpb, s_rf)
@@ -766,8 +765,8 @@ def main():
                       "fwd_hbm_gbs": alg_bytes / (t_fwd * 1e-3) / 1e9,
                       "bwd_hbm_gbs": alg_bytes / (t_bwd * 1e-3) / 1e9,
                       "hbm_frac_of_measured": alg_bytes / (t_bwd * 1e-3) / 1e9 / peaks["hbm_gbs"]},
-        "roofline": {"kernel": f"backprojector (strip sweep, k_op<OP_BWD> over {s_rf} view parts "
-                               "+ k_op<OP_BWD_FIN>), 512^2 / 800 views / 738 bins",
+        "roofline": {"kernel": "backprojector over orbits of rays (k_op<OP_ORB_ZPACK>, k_op<OP_ORB_BWD> to "
+                               f"{s_rf} images, k_op<OP_BWD_FIN>), 512^2 / 800 views / 738 bins",
                      "bound": "alu",
                      "achieved": nnz / (t_bwd * 1e-3) / 1e9,
                      "peak": seg_peak, "unit": "Gsegment/s",
@@ -788,7 +787,7 @@ def main():
                          "peak_per_s": 152 * sm_mhz * 1e6,
                          "bwd_frac": BWD_L1_WAVEFRONTS_512_V800 / (t_bwd * 1e-3) / (152 * sm_mhz * 1e6),
                          "fwd_frac": FWD_L1_WAVEFRONTS_512_V800 / (t_fwd * 1e-3) / (152 * sm_mhz * 1e6),
-                         "note": "bwd time includes the part sum k_op<OP_BWD_FIN>; peak at the SM clock "
+                         "note": "times include the copies before and the image sum after; peak at the SM clock "
                                  "sampled under load"}},
         "cpu_baseline": cpu,
         "precision_vs_fp64_oracle": prec,
@@ -798,9 +797,9 @@ def main():
         dist.destroy_process_group()
 
 
-# View parts of the backprojector launch the roofline times (2048 blocks of
-# 32 x 32 pixels at 512^2: 2.7 waves at 5 blocks per SM).
-BWD_PARTS = 8
+# Images of the backprojector launch the roofline times: eight for each of four
+# splits of the ray segments (1024 blocks of 32 x 32 pixels at 512^2).
+BWD_PARTS = 32
 # Thread-instructions of the least a segment evaluation takes (overlap
 # compare, intersection length, gather, FMA, loop step): the divisor of the
 # issue-limited peak.
@@ -808,13 +807,13 @@ SEG_INST = 8
 # DRAM bytes (read + write) of one backprojector launch on the 512^2 / 800-view
 # slice, from the committed ncu capture of the current kernel (None when the
 # kernel has changed since).
-BWD_DRAM_BYTES_512_V800 = 11_852_288
+BWD_DRAM_BYTES_512_V800 = 3_595_520
 # L1 data-pipe wavefronts of one launch of each operator on the 512^2 /
-# 800-view slice (l1tex__data_pipe_lsu_wavefronts: percent of peak x cycles x
-# 152 SMs) from the committed ncu captures of the current kernels: the
-# backprojector's shared-memory strip updates, the projector's gathers.
-BWD_L1_WAVEFRONTS_512_V800 = 58_059_172
-FWD_L1_WAVEFRONTS_512_V800 = 36_488_677
+# 800-view slice (l1tex__data_pipe_lsu_wavefronts.sum) from the committed ncu
+# captures of the current kernels (OP_ORB_BWD at four splits, OP_ORB_FWD): the
+# backprojector's reads of staged rays and samples, the projector's gathers.
+BWD_L1_WAVEFRONTS_512_V800 = 18_299_717
+FWD_L1_WAVEFRONTS_512_V800 = 18_445_397
 
 
 if __name__ == "__main__":

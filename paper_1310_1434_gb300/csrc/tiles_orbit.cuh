@@ -271,7 +271,7 @@ __device__ __forceinline__ void tile_orb_fwd(const SliceDesc &s, int arg, int ti
 // no pixel of the tile meets, are staged as well: the candidates may run
 // onto them.  The sums of each frame go to an image of their own, which
 // OP_BWD_FIN adds in a fixed order.  At 512^2 / 800 views the kernel takes
-// 86 us, with its packing and sum 102 (general path: 239): 64 M instead of 207
+// 86 us, with its packing and sum 89 (general path: 239): 64 M instead of 207
 // M warp instructions and 18 M instead of 55 M shared-memory wavefronts.
 // Bound: instruction issue (67 % active) and the shared-memory data path (68 %).
 // ======================================================================
