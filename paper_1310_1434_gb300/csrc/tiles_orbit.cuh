@@ -97,9 +97,10 @@ constexpr int ORB_PACK_FLOATS = 4 * 32 * 33;
 // one stack column; outside a ray's own walk range its row is clamped into
 // the zero pads.  The columns of a warp's rays are split over orb_ks warps,
 // whose sums are added in a fixed order: at 512^2 / 800 views eight parts a
-// ray take 89 us, four 98, two 99, one 155 (the image copies included).
+// ray took 89 us, four 98, two 99, one 155 (the image copies included, and
+// before the loads of four columns were issued together: 78.5 us now).
 // Bound: bytes into registers (8 for each ray and column; 18 M L1 data-pipe
-// wavefronts, 64 % of their rate) and L2 latency (a third of the sectors hit
+// wavefronts, 72 % of their rate) and L2 latency (a third of the sectors hit
 // L1).  The general pair's projector takes 137 us there, 36 M wavefronts.
 // ======================================================================
 
@@ -270,8 +271,8 @@ __device__ __forceinline__ void tile_orb_fwd(const SliceDesc &s, int arg, int ti
 // side, times the ray's c.  A segment's rays past the tile's last one, which
 // no pixel of the tile meets, are staged as well: the candidates may run
 // onto them.  The sums of each frame go to an image of their own, which
-// OP_BWD_FIN adds in a fixed order.  At 512^2 / 800 views the kernel takes
-// 86 us, with its packing and sum 89 (general path: 239): 64 M instead of 207
+// OP_BWD_FIN adds in a fixed order.  At 512^2 / 800 views the kernel, cold, takes
+// 86 us, a call with packing and sum 89 (general: 239): 64 M instead of 207
 // M warp instructions and 18 M instead of 55 M shared-memory wavefronts.
 // Bound: instruction issue (67 % active) and the shared-memory data path (68 %).
 // ======================================================================
