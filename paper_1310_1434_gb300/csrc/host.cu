@@ -697,7 +697,12 @@ air_status plan_build(const air_geometry *geom, air_plan *P) {
             return st;
         }
     }
-    air_status st = autotune(P);
+    // The clears above are asynchronous to the host, and the first call on the
+    // plan may come on a stream that does not wait for theirs: its results
+    // would be cleared from under it.
+    e = cudaStreamSynchronize(nullptr);
+    air_status st = e == cudaSuccess ? autotune(P)
+                                     : fail(AIR_ERR_CUDA, std::string("plan table upload: ") + cudaGetErrorString(e));
     if (st == AIR_OK) st = noalloc_prepare();
     if (st != AIR_OK) {
         ramp_tc_destroy(P);
