@@ -149,7 +149,7 @@ air_status prepare(int n, air_plan *const *plans, const float *const *Y, const f
                                          bits(g.dso_mm), bits(fan_pitch(g)), bits(g.beta0), bits(g.arc),
                                          (uintptr_t)g.filter, (uintptr_t)g.precision});
         const uintptr_t how[] = {(uintptr_t)n_outer[i], (uintptr_t)n_cg[i], (uintptr_t)d.fwd_vpb, (uintptr_t)d.bwd_parts,
-                                 (uintptr_t)d.orb_splits};
+                                 (uintptr_t)d.orb, (uintptr_t)d.orb_splits};
         B->key.insert(B->key.end(), std::begin(how), std::end(how));
         B->shape.insert(B->shape.end(), std::begin(how), std::end(how));
         B->data.insert(B->data.end(), {(uintptr_t)Y[i], (uintptr_t)X[i], bits(lambda[i]), bits(mu[i])});

@@ -144,34 +144,31 @@ static int sm_count() {
     return sms;
 }
 
-// Device bytes a plan of this geometry will hold (the pieces of plan_build
-// and, for BF16X3, the tensor-core filter buffers), to within alignment and,
-// for scans with orbit tables, the number of their segments.
+// Device bytes of the tensor-core filter's buffers (ramp_tc_create).
+static size_t filter_bytes(const air_geometry &g) {
+    if (g.precision != AIR_PREC_BF16X3) return 0;
+    const size_t kp = ((size_t)g.n_bins + 127) / 128 * 128;   // split Y; both parities' T_far pieces
+    return (size_t)g.n_views * 3 * kp * 2 + 3 * kp * kp + 1024;
+}
+
+// Least device bytes a plan of this geometry can do with (the pieces of
+// carve, without orbits, and the filter's), to within alignment; needs no
+// tables.
 size_t plan_bytes_estimate(const air_geometry &g) {
     SliceDesc s{};
     s.n = g.n;
     s.V = g.n_views;
     s.nb = g.n_bins;
     const size_t nn = (size_t)g.n * g.n, rays = (size_t)g.n_views * g.n_bins;
-    // the part buffer holds the autotuner's largest split, as plan_build sizes it
-    size_t parts = (size_t)std::min(g.n_views, 2 * choose_bwd_parts(s)), orbit = 0;
-    if (const int nf = orbit_frames(g); nf) {
-        parts = std::max(parts, (size_t)8 * orb_splits_max(g.n, nf, sm_count()));
-        const size_t segs = 2 * ((size_t)g.n_views / nf + 2);
-        orbit = nn * 32 + (size_t)g.n * 128 + (rays / nf + segs * ORB_CAND) * (sizeof(RayFx) + 8 + 1 + 16 + 4 * nf) + rays * 8 + segs * sizeof(OrbSeg) +
-                (size_t)tiles_bwd_xy(s) * (segs * 6 + 8);
-    }
-    size_t b = orbit + rays * (sizeof(RayFx) + 4) + (size_t)g.n_views * tiles_bwd_xy(s) * 4 + (size_t)g.n_bins * 4;
+    // the part buffer holds the autotuner's largest split, as carve sizes it
+    const size_t parts = (size_t)std::min(g.n_views, 2 * choose_bwd_parts(s));
+    size_t b = rays * (sizeof(RayFx) + 4) + (size_t)g.n_views * tiles_bwd_xy(s) * 4 + (size_t)g.n_bins * 4;
     b += nn * 4 * (7 + parts + 18 + 1);          // x r p q rhs0 g g', parts, b b2, xbuf
     b += (size_t)g.n * (g.n + 1) * 8 * 2;        // xp xt (pairs)
     b += (size_t)g.n_views * 8 + (size_t)g.n_bins * 8;   // FBP tables
     b += rays * 4 * 3;                           // z zc ybuf
     b += sizeof(CgState) + ((size_t)max_reduce_tiles(s) + 64) * 8 + 24 * 256;
-    if (g.precision == AIR_PREC_BF16X3) {
-        const size_t kp = ((size_t)g.n_bins + 127) / 128 * 128;   // split Y; both parities' T_far pieces
-        b += (size_t)g.n_views * 3 * kp * 2 + 3 * kp * kp + 1024;
-    }
-    return b;
+    return b + filter_bytes(g);
 }
 }  // namespace air
 
@@ -240,7 +237,7 @@ RayFx air::make_ray_fx(double px, double py, double ux, double uy, int n, unsign
 // configuration.  Timed without launch overlap, each kernel by itself.
 namespace {
 struct TuneKey {
-    int n, V, nb;
+    int n, V, nb, orb;
     double dx, dso, dg, beta0, arc;
     bool operator<(const TuneKey &o) const {
         return std::memcmp(this, &o, sizeof(TuneKey)) < 0;
@@ -261,6 +258,7 @@ air_status autotune(air_plan *P) {
     key.n = s.n;
     key.V = s.V;
     key.nb = s.nb;
+    key.orb = s.orb;
     key.dx = P->geom.pixel_mm;
     key.dso = P->geom.dso_mm;
     key.dg = fan_pitch(P->geom);
@@ -546,34 +544,38 @@ air_status geometry_tables(const air_geometry &g, double dg, int ntxy, std::shar
     *out = T;
     return AIR_OK;
 }
-}  // namespace
+// A plan's one allocation: the pieces that its descriptor points to.
+struct Piece { void **dst; size_t bytes; const void *src = nullptr; size_t off = 0; };
+struct Carve {
+    SliceDesc s{};
+    float *ybuf = nullptr, *xbuf = nullptr;
+    std::vector<Piece> pieces;          // dst: pointers in here, which is not copied
+    size_t total = 0, tables_end = 0, zero_end = 0;
+    int parts_max = 1;                  // images the part buffer holds
 
-air_status plan_build(const air_geometry *geom, air_plan *P) {
-    const air_geometry &g = *geom;
+    // orbits: with the tables and buffers of the scan's orbits, where it has them
+    Carve(const air_geometry &g, const HostTables &T, bool orbits);
+    Carve(const Carve &) = delete;
+};
+
+Carve::Carve(const air_geometry &g, const HostTables &T, bool orbits) {
     const int n = g.n, V = g.n_views, nb = g.n_bins;
     const size_t nn = (size_t)n * n, rays = (size_t)V * nb;
-    SliceDesc s{};
     s.n = n;
     s.V = V;
     s.nb = nb;
     s.half_n = 0.5f * n;
     s.dx = (float)g.pixel_mm;
-    const double dg = fan_pitch(g);
     s.filter = g.filter;
-
     s.fwd_vpb = 1;
     s.bwd_parts = choose_bwd_parts(s);
-    const int ntxy = tiles_bwd_xy(s);
-    std::shared_ptr<const HostTables> T;
-    if (air_status st = geometry_tables(g, dg, ntxy, &T); st != AIR_OK) return st;
-    const OrbitTables &O = T->orb;
-    const FbpOrbits &F = T->fbp;
+    static const OrbitTables none;
+    const OrbitTables &O = orbits ? T.orb : none;
     const int sms = sm_count();
     // the autotuner may pick up to twice the heuristic's view split; the
     // orbit backprojector's splits write eight images each
-    int parts_max = std::min(V, 2 * s.bwd_parts);
-    const int splits_max = O.nf ? orb_splits_max(n, O.nf, sms) : 0;
-    parts_max = std::max(parts_max, 8 * splits_max);
+    parts_max = std::min(V, 2 * s.bwd_parts);
+    if (O.nf) parts_max = std::max(parts_max, 8 * orb_splits_max(n, O.nf, sms));
     s.orb = O.nf;
     s.orb_splits = 1;
     s.orb_ntask = (int)O.task.size();
@@ -581,119 +583,87 @@ air_status plan_build(const air_geometry *geom, air_plan *P) {
     s.orb_npad = (int)O.bray.size();
     s.orb_ks = choose_orb_ks(s.orb_ntask, sms);
     for (int p = 0; p < 8; ++p) s.orb_frame[p] = O.frame[p];
-    // carve one allocation
-    struct Piece { void **dst; size_t bytes; const void *src = nullptr; size_t off = 0; };
-    float *x, *r, *p, *q, *rhs0, *gg, *gg2, *b, *b2, *z, *zc, *ybuf, *xbuf, *xp, *xt, *bpart;
     const size_t npad = (size_t)n * (n + 1) * 2;   // pair copies of the projector's input (floats)
-    RayFx *ray;
-    unsigned *walk;
-    unsigned *vt;
-    float2 *fview;
-    float *fbw, *fbt;
-    OrbSeg *oseg;
-    RayFx *oray;
-    uint2 *oinfo, *oent, *ozmap;
-    uint4 *obray;
-    float4 *oz;
-    float2 *fbpc;
-    int *fbpview;
-    unsigned *otask;
-    int *otile0;
-    float4 *ostack;
     const size_t nstack = O.nf ? (size_t)2 * n * orb_ld(n) : 0;
     const size_t nz = O.bray.size() * orb_planes(s);
-    float *taps;
-    CgState *cg;
-    double *partial;
     const size_t npart = (size_t)max_reduce_tiles(s) + 64;
     auto table = [](auto **dst, const auto &v) { return Piece{(void **)dst, v.size() * sizeof(v[0]), v.data()}; };
-    std::vector<Piece> pieces = {
-        // the tables
-        table(&ray, T->ray), table(&walk, T->walk), table(&vt, T->vt), table(&taps, T->taps), table(&fview, T->fview),
-        table(&fbw, T->fbw), table(&fbt, T->fbt), table(&oseg, O.seg), table(&oray, O.ray), table(&oinfo, O.info),
-        table(&oent, O.ent), table(&otask, O.task), table(&otile0, O.tile0), table(&obray, O.bray), table(&ozmap, O.zmap),
-        table(&fbpc, T->fbp_c), table(&fbpview, F.view),
+    pieces = {
+        // the tables; the orbits' last, so that a plan without them takes the same blob's front
+        table(&s.ray, T.ray), table(&s.walk, T.walk), table(&s.vt, T.vt), table(&s.taps, T.taps), table(&s.fview, T.fview),
+        table(&s.fbp_w, T.fbw), table(&s.fbp_taps, T.fbt), table(&s.fbp_c, T.fbp_c), table(&s.fbp_view, T.fbp.view),
+        table(&s.orb_seg, O.seg), table(&s.orb_ray, O.ray), table(&s.orb_info, O.info), table(&s.orb_ent, O.ent),
+        table(&s.orb_task, O.task), table(&s.orb_tile0, O.tile0), table(&s.orb_bray, O.bray), table(&s.orb_zmap, O.zmap),
         // zeroed once: the image copies' pads and the empty rays' samples stay zero
-        {(void **)&xp, npad * 4}, {(void **)&xt, npad * 4}, {(void **)&ostack, nstack * sizeof(float4)},
-        {(void **)&oz, nz * sizeof(float4)}, {(void **)&cg, sizeof(CgState)},
+        {(void **)&s.xp, npad * 4}, {(void **)&s.xt, npad * 4}, {(void **)&s.orb_stack, nstack * sizeof(float4)},
+        {(void **)&s.orb_z, nz * sizeof(float4)}, {(void **)&s.cg, sizeof(CgState)},
         // workspace
-        {(void **)&bpart, (size_t)parts_max * nn * 4},
-        {(void **)&x, nn * 4}, {(void **)&r, nn * 4}, {(void **)&p, nn * 4}, {(void **)&q, nn * 4},
-        {(void **)&rhs0, nn * 4}, {(void **)&gg, nn * 4}, {(void **)&gg2, nn * 4}, {(void **)&b, 9 * nn * 4}, {(void **)&b2, 9 * nn * 4},
-        {(void **)&z, rays * 4}, {(void **)&zc, rays * 4}, {(void **)&ybuf, rays * 4}, {(void **)&xbuf, nn * 4},
-        {(void **)&partial, npart * sizeof(double)}};
-    size_t total = 0, tables_end = 0, zero_end = 0;
+        {(void **)&s.bwd_part, (size_t)parts_max * nn * 4},
+        {(void **)&s.x, nn * 4}, {(void **)&s.r, nn * 4}, {(void **)&s.p, nn * 4}, {(void **)&s.q, nn * 4},
+        {(void **)&s.rhs0, nn * 4}, {(void **)&s.g, nn * 4}, {(void **)&s.g2, nn * 4}, {(void **)&s.b, 9 * nn * 4},
+        {(void **)&s.b2, 9 * nn * 4}, {(void **)&s.z, rays * 4}, {(void **)&s.zc, rays * 4}, {(void **)&ybuf, rays * 4},
+        {(void **)&xbuf, nn * 4}, {(void **)&s.partial, npart * sizeof(double)}};
     for (auto &pc : pieces) {
         pc.off = align_up(total, 256);
         total = pc.off + pc.bytes;
         if (pc.src) tables_end = total;
-        if (pc.dst == (void **)&cg) zero_end = total;
+        if (pc.dst == (void **)&s.cg) zero_end = total;
     }
     total = align_up(total, 256);
-    char *mem = nullptr;
-    if (cudaMalloc(&mem, total) != cudaSuccess) {
-        cudaGetLastError();
-        return fail(AIR_ERR_OOM, "cudaMalloc of the plan workspace failed (" + std::to_string(total) + " bytes)");
-    }
-    for (auto &pc : pieces) *pc.dst = mem + pc.off;
-    std::call_once(T->packed, [&] {
-        T->blob.assign(tables_end, 0);
-        for (auto &pc : pieces)
-            if (pc.src && pc.bytes) std::memcpy(T->blob.data() + pc.off, pc.src, pc.bytes);
-    });
+}
+}  // namespace
 
-    s.ramp_diag = T->ramp_diag;
-    s.fbp_diag = T->fbp_diag;
+// A plan with or without orbits, in at most `limit` device bytes.
+static air_status plan_attempt(const air_geometry &g, const HostTables &T, bool orbits, size_t limit, air_plan *P) {
+    const double dg = fan_pitch(g);
+    Carve C(g, T, orbits);
+    std::call_once(T.packed, [&] {
+        const Carve F(g, T, true);
+        T.blob.assign(F.tables_end, 0);
+        for (auto &pc : F.pieces)
+            if (pc.src && pc.bytes) std::memcpy(T.blob.data() + pc.off, pc.src, pc.bytes);
+    });
+    const size_t need = C.total + filter_bytes(g);
+    if (C.s.orb && need > limit)
+        return fail(AIR_ERR_OOM, "the plan needs " + std::to_string(need) + " bytes of " + std::to_string(limit));
+    char *mem = nullptr;
+    if (cudaMalloc(&mem, C.total) != cudaSuccess) {
+        cudaGetLastError();
+        return fail(AIR_ERR_OOM, "cudaMalloc of the plan workspace failed (" + std::to_string(C.total) + " bytes)");
+    }
+    for (auto &pc : C.pieces) *pc.dst = mem + pc.off;
+    SliceDesc &s = C.s;
+
+    s.ramp_diag = T.ramp_diag;
+    s.fbp_diag = T.fbp_diag;
     s.dso_px = (float)(g.dso_mm / g.pixel_mm);
     s.inv_dg = (float)(1.0 / dg);
     s.inv_dg_lo = (float)(1.0 / dg - (double)s.inv_dg);
-    s.jmid = 0.5f * (nb - 1);
-    s.fbp_scale = (float)(g.arc / (double)V / (g.pixel_mm * g.pixel_mm));
-    cudaError_t e = cudaMemcpy(mem, T->blob.data(), tables_end, cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemset(mem + tables_end, 0, zero_end - tables_end);
+    s.jmid = 0.5f * (g.n_bins - 1);
+    s.fbp_scale = (float)(g.arc / (double)g.n_views / (g.pixel_mm * g.pixel_mm));
+    cudaError_t e = cudaMemcpy(mem, T.blob.data(), C.tables_end, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemset(mem + C.tables_end, 0, C.zero_end - C.tables_end);
     if (e != cudaSuccess) {
         cudaFree(mem);
         return fail(AIR_ERR_CUDA, std::string("plan table upload: ") + cudaGetErrorString(e));
     }
-    s.ray = ray;
-    s.walk = walk;
-    s.vt = vt;
-    s.fview = fview;
-    s.fbp_w = fbw;
-    s.fbp_taps = fbt;
-    s.taps = taps;
-    s.orb_seg = oseg;
-    s.orb_ray = oray;
-    s.orb_info = oinfo;
-    s.orb_ent = oent;
-    s.orb_bray = obray;
-    s.orb_zmap = ozmap;
-    s.fbp_c = fbpc;
-    s.fbp_view = fbpview;
-    choose_fbp(s, F, bpart, parts_max, sms);
-    s.orb_z = oz;
-    s.orb_task = otask;
-    s.orb_tile0 = otile0;
-    s.orb_stack = ostack;
-    s.x = x; s.r = r; s.p = p; s.q = q; s.rhs0 = rhs0; s.g = gg; s.g2 = gg2; s.b = b; s.b2 = b2; s.xp = xp; s.xt = xt;
-    s.bwd_part = bpart;
-    s.z = z; s.zc = zc; s.y = ybuf;
-    s.cg = cg;
-    s.partial = partial;
+    choose_fbp(s, T.fbp, s.bwd_part, C.parts_max, sm_count());
+    s.y = C.ybuf;
     s.mu = 1.f;
     s.tau = 0.f;
     P->geom = g;
     P->desc = s;
     P->mem = mem;
-    P->bytes = total;
-    P->bwd_parts_max = parts_max;
-    P->ybuf = ybuf;
-    P->xbuf = xbuf;
+    P->bytes = C.total;
+    P->bwd_parts_max = C.parts_max;
+    P->ybuf = C.ybuf;
+    P->xbuf = C.xbuf;
     cudaGetDevice(&P->device);
     if (g.precision == AIR_PREC_BF16X3) {
         air_status st = ramp_tc_create(P);
         if (st != AIR_OK) {
             cudaFree(mem);
+            P->mem = nullptr;
             return st;
         }
     }
@@ -707,14 +677,41 @@ air_status plan_build(const air_geometry *geom, air_plan *P) {
     if (st != AIR_OK) {
         ramp_tc_destroy(P);
         cudaFree(mem);
+        P->mem = nullptr;
         return st;
     }
     return AIR_OK;
 }
 
+// Orbits cost a plan memory (68 -> 94 MB at 512^2 / 800 views): one that does
+// not fit the limit, or the device, with them is made without.
+static air_status plan_build(const air_geometry &g, size_t limit, air_plan *P) {
+    SliceDesc s{};
+    s.n = g.n;
+    std::shared_ptr<const HostTables> T;
+    if (air_status st = geometry_tables(g, fan_pitch(g), tiles_bwd_xy(s), &T); st != AIR_OK) return st;
+    const air_status st = plan_attempt(g, *T, true, limit, P);
+    return st == AIR_ERR_OOM && T->orb.nf ? plan_attempt(g, *T, false, limit, P) : st;
+}
+
+// Device bytes of the plan that plan_create makes under this limit; builds the
+// geometry's tables (which plan_create then finds).  0: they cannot be built.
+size_t air::plan_bytes(const air_geometry &g, size_t limit) {
+    SliceDesc s{};
+    s.n = g.n;
+    std::shared_ptr<const HostTables> T;
+    if (geometry_tables(g, fan_pitch(g), tiles_bwd_xy(s), &T) != AIR_OK) return 0;
+    const size_t b = Carve(g, *T, true).total + filter_bytes(g);
+    return T->orb.nf && b > limit ? Carve(g, *T, false).total + filter_bytes(g) : b;
+}
+
 extern "C" const char *air_last_error(void) { return g_err.c_str(); }
 
 extern "C" air_status air_plan_create(const air_geometry *geom, air_plan **out) {
+    return plan_create(geom, SIZE_MAX, out);
+}
+
+air_status air::plan_create(const air_geometry *geom, size_t limit, air_plan **out) {
     if (!out) return fail(AIR_ERR_INVALID_ARG, "out is NULL");
     *out = nullptr;
     air_status st = validate_geometry(geom);
@@ -723,7 +720,7 @@ extern "C" air_status air_plan_create(const air_geometry *geom, air_plan **out) 
     if (!P) return fail(AIR_ERR_OOM, "host allocation failed");
     static std::atomic<uint64_t> ids{0};
     P->id = ++ids;
-    st = plan_build(geom, P);
+    st = plan_build(*geom, limit, P);
     if (st != AIR_OK) {
         delete P;
         return st;

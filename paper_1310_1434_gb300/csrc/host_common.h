@@ -45,6 +45,10 @@ int choose_bwd_parts(const SliceDesc &s);
 cudaError_t launch_backprojection(const SliceDesc &s, int mode, bool packed, cudaStream_t st, bool overlap = true);
 air_status autotune(air_plan *P);
 void batch_forget(uint64_t plan_id);
+// A plan that takes no orbits where it would need more than `limit` device
+// bytes with them; the bytes it will hold; and the least they can be.
+air_status plan_create(const air_geometry *geom, size_t limit, air_plan **out);
+size_t plan_bytes(const air_geometry &g, size_t limit);
 size_t plan_bytes_estimate(const air_geometry &g);
 air_status apply_filter(const air_plan *P, const SliceDesc &base, const float *src, float *dst, bool pack,
                         cudaStream_t st);

@@ -69,7 +69,7 @@ struct air_server {
     std::vector<Request *> active;
     std::map<uint64_t, std::unique_ptr<Request>> all;
     std::vector<std::pair<air_geometry, air_plan *>> pool;   // idle plans, reused by geometry
-    std::vector<std::pair<air_geometry, size_t>> plan_bytes; // device bytes of a plan, by geometry, once built
+    std::vector<std::pair<air_geometry, size_t>> plan_bytes; // device bytes of a plan, by geometry, once asked for
     std::thread worker;
     bool stop = false;
     uint64_t next_id = 1;
@@ -152,7 +152,7 @@ air_status get_plan(air_server *S, const air_geometry &g, air_plan **out) {
             S->pool.erase(S->pool.begin() + i);
             return AIR_OK;
         }
-    return air_plan_create(&g, out);
+    return plan_create(&g, S->budget, out);
 }
 
 void put_plan(air_server *S, air_plan *p) {
@@ -184,23 +184,29 @@ void finish(air_server *S, Request *r, air_status st) {
     S->cv_done.notify_all();
 }
 
-// Device bytes of a plan of this geometry: measured once a plan of it has
-// been built, the estimate before.
-size_t request_bytes(const air_server *S, const air_geometry &g) {
+// Device bytes of the plan a request of this geometry is given.
+size_t request_bytes(air_server *S, const air_geometry &g) {
     for (const auto &kv : S->plan_bytes)
         if (same_geom(kv.first, g)) return kv.second;
-    return plan_bytes_estimate(g);
+    const size_t b = plan_bytes(g, S->budget);
+    if (!b) return plan_bytes_estimate(g);      // the plan's creation will say why
+    S->plan_bytes.push_back({g, b});
+    return b;
 }
 
 // Admission at a step boundary (called with the lock held).  A request is
-// charged the bytes of the plan it is given, which are known exactly once
-// the plan exists: a request whose estimate fitted but whose plan does not
-// waits with the plan pooled, and one whose plan alone exceeds the budget
-// fails with AIR_ERR_BUDGET.
+// charged the bytes of the plan it is given: one whose plan alone exceeds the
+// budget fails with AIR_ERR_BUDGET, and one whose plan does not fit beside the
+// others' waits (with the plan pooled, should it turn out larger than said).
 void admit(air_server *S) {
     while (!S->queue.empty() && !S->free_slots.empty()) {
         Request *r = S->queue.front();
         r->bytes = request_bytes(S, r->geom);
+        if (r->bytes > S->budget) {                      // can never fit
+            S->queue.pop_front();
+            finish(S, r, fail(AIR_ERR_BUDGET, "the request's plan needs more device bytes than the budget"));
+            continue;
+        }
         if (S->used + r->bytes > S->budget) break;       // FIFO: wait for memory
         trim_pool(S, r->bytes);
         air_plan *plan = nullptr;
@@ -211,9 +217,6 @@ void admit(air_server *S) {
             continue;
         }
         const size_t actual = air_plan_bytes(plan);
-        if (!std::any_of(S->plan_bytes.begin(), S->plan_bytes.end(),
-                         [&](const auto &kv) { return same_geom(kv.first, r->geom); }))
-            S->plan_bytes.push_back({r->geom, actual});
         if (S->used + actual > S->budget) {
             r->bytes = actual;
             if (actual > S->budget) {                     // can never fit
