@@ -117,7 +117,7 @@ air_status prepare(int n, air_plan *const *plans, const float *const *Y, const f
     if (!plans || !Y || !lambda || !mu || !n_outer || !n_cg || !X)
         return fail(AIR_ERR_INVALID_ARG, "NULL array argument");
     B->slices.resize(n);
-    B->progs.resize(n);
+    std::vector<SolveForm> forms;
     for (int i = 0; i < n; ++i) {
         air_status s = check_solve_args(plans[i], Y[i], lambda[i], mu[i], n_outer[i], n_cg[i], X[i]);
         if (s != AIR_OK) return s;
@@ -129,9 +129,10 @@ air_status prepare(int n, air_plan *const *plans, const float *const *Y, const f
         if (tc && !allow_tc)
             return fail(AIR_ERR_INVALID_ARG, "the persistent batch runs the FP32 filter; use FP32 plans");
         B->slices[i] = solve_desc(plans[i], Y[i], lambda[i], mu[i], X[i], nullptr);
-        B->progs[i] = solve_program(n_outer[i], n_cg[i], tc, plans[i]->desc.orb != 0, true);
-        B->nphases = std::max(B->nphases, B->progs[i].size());
+        forms.push_back({n_outer[i], n_cg[i], tc, plans[i]->desc.orb != 0});
     }
+    B->progs = batch_programs(forms);
+    for (const auto &prog : B->progs) B->nphases = std::max(B->nphases, prog.size());
     cudaGetDevice(&B->device);
     B->key.push_back((uintptr_t)B->device);
     B->shape.push_back((uintptr_t)B->device);

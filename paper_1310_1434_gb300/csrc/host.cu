@@ -908,19 +908,19 @@ extern "C" air_status air_shrink(const air_plan *P, const float *X, float *b, fl
 // ------------------------------------------------------------------ solve
 namespace air {
 
-// The split-Bregman program of one slice as a list of phases.
 // The split-Bregman program of one slice (Methods, Eq. 5 and ref. [24]).
 // Each outer step's CG restarts from the residual the previous CG left,
 // corrected for the change of the right-hand side (OP_RESTART): CG keeps
 // r = b - M X, and b changes between outer steps only by mu (g_new - g_old).
-// `aligned`: every CG step is seven phases, whatever the path, so that the
-// slices of a batch meet in the operators they share.
-std::vector<Phase> solve_program(int n_outer, int n_cg, bool tc_ramp, bool orb, bool aligned) {
+// zpack_slot, cg_b_slot: a program without OP_ORB_ZPACK or OP_CG_B keeps its
+// place free (batch_programs).
+std::vector<Phase> solve_program(int n_outer, int n_cg, bool tc_ramp, bool orb, bool zpack_slot, bool cg_b_slot) {
     std::vector<Phase> prog;
     const int ramp = tc_ramp ? OP_RAMP_TC : OP_RAMP, pack = orb && !tc_ramp ? ARG_PACK : 0;
     const int copies = orb ? OP_ORB_PACK : OP_TRANSPOSE, fwd = orb ? OP_ORB_FWD : OP_FWD;
     auto push_bwd = [&](int mode) {
         if (orb && tc_ramp) prog.push_back({OP_ORB_ZPACK, mode});
+        else if (zpack_slot) prog.push_back({OP_NOP, 0});
         prog.push_back({orb ? OP_ORB_BWD : OP_BWD, mode});
     };
     prog.push_back({ramp, RSRC_Y | pack});   // zc = C y
@@ -938,7 +938,7 @@ std::vector<Phase> solve_program(int n_outer, int n_cg, bool tc_ramp, bool orb, 
             prog.push_back({OP_BWD_FIN, BWD_Q | swap});
             prog.push_back({OP_CG_A, swap});
             if (!orb) prog.push_back({OP_CG_B, 0});
-            else if (aligned && !tc_ramp) prog.push_back({OP_NOP, 0});
+            else if (cg_b_slot) prog.push_back({OP_NOP, 0});
         }
         prog.push_back({OP_SHRINK, k & 1});
         if (k + 1 < n_outer) prog.push_back({OP_RESTART, k & 1});   // r += mu (g_k - g_{k-1})
@@ -946,11 +946,26 @@ std::vector<Phase> solve_program(int n_outer, int n_cg, bool tc_ramp, bool orb, 
     return prog;
 }
 
+// The programs of a batch, phase for phase: slices on different paths or with
+// different filters keep each other's extra phases free, so that they meet in
+// the operators they share (30 x 8 steps, FP32 and BF16X3 slices with orbits:
+// 1745 grouped launches; phase by phase as they come, 3008).
+std::vector<std::vector<Phase>> batch_programs(const std::vector<SolveForm> &forms) {
+    bool zpack = false, cg_b = false;
+    for (const SolveForm &f : forms) {
+        zpack |= f.orb && f.tc_ramp;
+        cg_b |= !f.orb;
+    }
+    std::vector<std::vector<Phase>> out;
+    for (const SolveForm &f : forms) out.push_back(solve_program(f.n_outer, f.n_cg, f.tc_ramp, f.orb, zpack, cg_b));
+    return out;
+}
+
 // L2-regularised AIR, Eq. (5): (A'^T A + lambda I) X = A'^T Y by n_cg CG steps
 // from X = 0 (the first L2 step of the split-Bregman program with g = 0 and
 // mu = lambda, without the shrink).
 std::vector<Phase> l2_program(int n_cg, bool tc_ramp, bool orb) {
-    std::vector<Phase> prog = solve_program(1, n_cg, tc_ramp, orb, false);
+    std::vector<Phase> prog = solve_program(1, n_cg, tc_ramp, orb);
     prog.pop_back();   // the SHRINK of the outer step
     return prog;
 }
@@ -1030,7 +1045,7 @@ extern "C" air_status air_solve(const air_plan *P, const float *Y, float lambda,
     if (resid) TRY(check_dev_ptr(resid, "resid"));
     const bool tc = P->geom.precision == AIR_PREC_BF16X3 && P->geom.filter == AIR_FILTER_RAMLAK;
     SliceDesc s = solve_desc(P, Y, lambda, mu, X, resid);
-    return run_program_single(P, s, solve_program(n_outer, n_cg, tc, s.orb != 0, false), (cudaStream_t)stream);
+    return run_program_single(P, s, solve_program(n_outer, n_cg, tc, s.orb != 0), (cudaStream_t)stream);
 }
 
 extern "C" air_status air_solve_l2(const air_plan *P, const float *Y, float lambda, int n_cg, float *X,
@@ -1096,7 +1111,7 @@ extern "C" air_status air_solve_host(const air_plan *P, const float *Y_host, flo
     CUDA_TRY(cudaMemcpyAsync(P->ybuf, Y_host, sino_bytes(P), cudaMemcpyHostToDevice, st));
     const bool tc = P->geom.precision == AIR_PREC_BF16X3 && P->geom.filter == AIR_FILTER_RAMLAK;
     SliceDesc s = solve_desc(P, P->ybuf, lambda, mu, P->xbuf, nullptr);
-    TRY(run_program_single(P, s, solve_program(n_outer, n_cg, tc, P->desc.orb != 0, false), st));
+    TRY(run_program_single(P, s, solve_program(n_outer, n_cg, tc, P->desc.orb != 0), st));
     CUDA_TRY(cudaMemcpyAsync(X_host, P->xbuf, img_bytes(P), cudaMemcpyDeviceToHost, st));
     CUDA_TRY(cudaStreamSynchronize(st));
     return tc ? air_plan_status(P) : AIR_OK;

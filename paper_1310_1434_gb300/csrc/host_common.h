@@ -29,7 +29,10 @@ air_status check_dev_ptr(const void *p, const char *what);
 bool overlap(const void *a, size_t na, const void *b, size_t nb);
 size_t align_up(size_t v, size_t a);
 double fan_pitch(const air_geometry &g);
-std::vector<Phase> solve_program(int n_outer, int n_cg, bool tc_ramp, bool orb, bool aligned);
+std::vector<Phase> solve_program(int n_outer, int n_cg, bool tc_ramp, bool orb, bool zpack_slot = false,
+                                 bool cg_b_slot = false);
+struct SolveForm { int n_outer, n_cg; bool tc_ramp, orb; };
+std::vector<std::vector<Phase>> batch_programs(const std::vector<SolveForm> &forms);
 std::vector<Phase> l2_program(int n_cg, bool tc_ramp, bool orb);
 std::vector<Phase> fbs_program(int n_iter, bool tc_ramp, bool orb);
 air_status check_solve_args(const air_plan *P, const float *Y, float lambda, float mu, int n_outer,

@@ -253,7 +253,7 @@ void admit(air_server *S) {
         r->slot = S->free_slots.back();
         S->free_slots.pop_back();
         const bool tc = r->geom.precision == AIR_PREC_BF16X3 && r->geom.filter == AIR_FILTER_RAMLAK;
-        r->prog = solve_program(r->n_outer, r->n_cg, tc, plan->desc.orb != 0, false);
+        r->prog = solve_program(r->n_outer, r->n_cg, tc, plan->desc.orb != 0);
         r->pc = 0;
         const size_t sino = (size_t)r->geom.n_views * r->geom.n_bins * 4;
         S->h_slices[r->slot] = solve_desc(plan, plan->ybuf, r->lam, r->mu, plan->xbuf, nullptr);
