@@ -747,8 +747,10 @@ extern "C" air_status air_plan_tune(air_plan *P, int fwd_views_per_block, int bw
     if (bwd_view_parts < 1 || bwd_view_parts > P->bwd_parts_max)
         return fail(AIR_ERR_INVALID_ARG, "bwd_view_parts must be in 1.." + std::to_string(P->bwd_parts_max));
     P->desc.fwd_vpb = v;
-    P->desc.bwd_parts = bwd_view_parts;
-    P->desc.orb_splits = std::max(1, bwd_view_parts / 8);
+    // what air_plan_config reports of this plan; the general pair, which an
+    // orbit plan's solves with history run, keeps its own split
+    if (P->desc.orb) P->desc.orb_splits = std::max(1, bwd_view_parts / 8);
+    else P->desc.bwd_parts = bwd_view_parts;
     return AIR_OK;
 }
 
