@@ -800,23 +800,33 @@ struct ShrinkArgs {
     float tau;
 };
 
-// A sum of squares kept in two floats (hi + lo, 48 significant bits): the
-// squares of differences x - y enter with their rounding errors (Knuth's
-// two-sum, an FMA for the product's error).
+// a + b = s + the rounding error it returns (Knuth's two-sum).
+__device__ __forceinline__ float two_sum(float a, float b, float &s) {
+    s = __fadd_rn(a, b);
+    const float t = __fsub_rn(s, a);
+    return __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+}
+
+// A sum of squares kept in three floats (hi + mid + lo), more bits than FP64
+// has: the squares of differences x - y enter without a rounding error above
+// 2^-69 of the sum (two-sums, and an FMA for a product's error).
 struct SumSq {
-    float hi, lo, top;             // top: the largest |x - y|
+    float hi, mid, lo, top;        // top: the largest |x - y|
     __device__ __forceinline__ void add_diff(float x, float y) {
-        const float e = __fsub_rn(x, y), yy = __fsub_rn(e, x);
+        float e, m;
+        const float de = two_sum(x, -y, e);                     // x - y = e + de
         top = fmaxf(top, fabsf(e));
-        const float de = __fsub_rn(__fsub_rn(x, __fsub_rn(e, yy)), __fadd_rn(y, yy));   // x - y = e + de
-        const float p = __fmul_rn(e, e), dp = fmaf(2.f * e, de, fmaf(e, e, -p));
-        add(p, dp);
+        const float p = __fmul_rn(e, e), r = fmaf(e, e, -p);    // (e + de)^2 = p + r + q + rest
+        const float e2 = 2.f * e, q = __fmul_rn(e2, de), rest = fmaf(de, de, fmaf(e2, de, -q));
+        const float a = two_sum(hi, p, hi), b = two_sum(a, r, m), c = two_sum(m, q, m), d = two_sum(mid, m, mid);
+        lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(b, c), __fadd_rn(d, rest)));
     }
-    __device__ __forceinline__ void add(float p, float dp) {
-        const float h = __fadd_rn(hi, p), t = __fsub_rn(h, hi);
-        lo = __fadd_rn(lo, __fadd_rn(__fadd_rn(__fsub_rn(hi, __fsub_rn(h, t)), __fsub_rn(p, t)), dp));
-        hi = h;
+    __device__ __forceinline__ void add(float h, float m, float l) {
+        float t;
+        const float a = two_sum(hi, h, hi), b = two_sum(a, m, t), c = two_sum(mid, t, mid);
+        lo = __fadd_rn(lo, __fadd_rn(l, __fadd_rn(b, c)));
     }
+    __device__ __forceinline__ double value() const { return (double)hi + ((double)mid + (double)lo); }
     // the squares neither overflowed nor lost what the sum needs of them
     __device__ __forceinline__ bool fits() const { return top == 0.f || (top > 0x1p-40f && top < 0x1p50f); }
 };
@@ -830,14 +840,17 @@ struct SumSq {
 // tile's sum of ||W X - d||^2.  Otherwise (the proximal step of
 // forward-backward splitting for R = ||W X||_1 with the tight frame W):
 // W^T soft(W X).  The high-pass bands are shrunk, the low-pass band kept.
-// The residual's squares are summed per warp in two floats (SumSq) and from
+// The residual's squares are summed per block in three floats (SumSq) and from
 // there in FP64: GB300 issues one FP64 instruction for 64 FP32 ones, and four
 // for each of the nine coefficients bound the form that did (FP64 pipe 67 %
 // active).  The coefficient tile is 32 x 8, one row for each warp.
-// At 512^2 the kernel takes 20 us, 36 with FP64 squares and 16 x 16 tiles
-// (49 % of the issue slots; the chain of loads, barriers and the reduction of
-// each short block bounds it).  Walking each warp down a strip of 8 rows with
-// all passes in registers took 27 us: too few warps for that chain.
+// At 512^2 a stand-alone call, which copies b back, takes 25 us: 44 with FP64
+// squares and 16 x 16 tiles, 34 with FP64 squares in these tiles, 24 with two
+// floats, which lose up to 2e-14 of nine squares where FP64 loses 3e-16 and
+// three floats 1e-16; 62 us at 1024^2 (130, 99, 54).  The chain of loads,
+// barriers and the reduction of each short block bounds it.  Walking each warp
+// down a strip of 8 rows with all passes in registers took 7 us more: too few
+// warps for that chain.
 constexpr int FS_W = 30, FS_H = 6;                 // output tile, as tiles_fs counts them
 constexpr int FS_CW = FS_W + 2, FS_CH = FS_H + 2;  // coefficient tile
 constexpr int FS_XW = FS_W + 4, FS_XH = FS_H + 4;  // image tile
@@ -905,7 +918,7 @@ __device__ __forceinline__ double fs_tile(const ShrinkArgs &A, int n, int tile, 
     const int ly = threadIdx.x / FS_CW, lx = threadIdx.x % FS_CW;
     const size_t nn = (size_t)n * n;
     float *R = sm + FS_XW * FS_XH;
-    SumSq sq{0.f, 0.f, 0.f};
+    SumSq sq{0.f, 0.f, 0.f, 0.f};
     double total = 0.0;
 #pragma unroll 1
     for (int y0 = ty * rows; y0 < min(n, (ty + 1) * rows); y0 += FS_H) {
@@ -921,7 +934,7 @@ __device__ __forceinline__ double fs_tile(const ShrinkArgs &A, int n, int tile, 
             sm[k] = ld_data(A.X + (size_t)wrapi(y0 - 2 + iy, n) * n + wrapi(x0 - 2 + ix, n));
         }
         __syncthreads();
-        SumSq one{0.f, 0.f, 0.f};
+        SumSq one{0.f, 0.f, 0.f, 0.f};
         double wide = 0.0;
         fs_coefficients<SHRINK, false>(A, n, x0, y0, bo, sm, R, one, wide);
         const int out_of_range = __syncthreads_or(!one.fits());
@@ -929,7 +942,7 @@ __device__ __forceinline__ double fs_tile(const ShrinkArgs &A, int n, int tile, 
             fs_coefficients<SHRINK, SHRINK>(A, n, x0, y0, bo, sm, R, one, wide);
             total += block_sum(wide, sh);
         } else if (SHRINK) {
-            sq.add(one.hi, one.lo);
+            sq.add(one.hi, one.mid, one.lo);
         }
         if (ly < FS_H && lx < FS_W && y0 + ly < n && x0 + lx < n) {
             float acc = 0.f;       // the column pass, in framelet_t1's order
@@ -943,16 +956,16 @@ __device__ __forceinline__ double fs_tile(const ShrinkArgs &A, int n, int tile, 
         }
         __syncthreads();           // the next tile's
     }
-    if (SHRINK) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-            const float hi = __shfl_xor_sync(0xffffffffu, sq.hi, o), lo = __shfl_xor_sync(0xffffffffu, sq.lo, o);
-            sq.add(hi, lo);
-        }
-        if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = (double)sq.hi + (double)sq.lo;
+    if (SHRINK) {                  // eight threads' sums for each lane of a warp, then its lanes'
+        sm[threadIdx.x] = sq.hi;
+        sm[AIR_THREADS + threadIdx.x] = sq.mid;
+        sm[2 * AIR_THREADS + threadIdx.x] = sq.lo;
         __syncthreads();
-        if (threadIdx.x == 0)
-            for (int w = 0; w < AIR_THREADS / 32; ++w) total += sh[w];
+        if (threadIdx.x < 32) {
+#pragma unroll
+            for (int i = 32 + threadIdx.x; i < AIR_THREADS; i += 32) sq.add(sm[i], sm[AIR_THREADS + i], sm[2 * AIR_THREADS + i]);
+            total += warp_sum(sq.value());
+        }
     }
     return total;
 }
