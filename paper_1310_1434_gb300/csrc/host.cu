@@ -1098,8 +1098,8 @@ extern "C" air_status air_fbp(const air_plan *P, const float *Y, float *X, air_s
     }
     CUDA_TRY(launch_op(OP_FBP_PACK, b, 0, st));
     CUDA_TRY(launch_op(OP_FBP_ORB, b, 0, st));
-    b.orb = 8;                    // the sum of the orbits' images, scaled
-    b.orb_splits = b.fbp_splits * b.fbp_nf / 8;
+    b.orb = 0;                    // the sum of the orbits' images in a row, scaled
+    b.bwd_parts = b.fbp_splits * b.fbp_nf;
     b.dx = b.fbp_scale;
     CUDA_TRY(launch_op(OP_BWD_FIN, b, BWD_PLAIN, st));
     return AIR_OK;

@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(AIR_THREADS, min_blocks<OP>) k_op(const SliceD
     } else if constexpr (OP == OP_BWD) {
         tile_bwd(s, arg, tile, sm);
     } else if constexpr (OP == OP_BWD_FIN) {
-        tile_bwd_fin<FIN_IMAGES>(s, arg, tile);
+        tile_bwd_fin<FIN_IMAGES, true>(s, arg, tile);
     } else if constexpr (OP == OP_CG_A) {
         tile_cg_a(s, arg, tile);
     } else if constexpr (OP == OP_CG_B) {
@@ -166,7 +166,7 @@ k_group(const SliceDesc *__restrict__ slices, const Task *__restrict__ tasks, in
     if constexpr (OP == OP_FWD) tile_fwd(s, t.arg, tile);
     else if constexpr (OP == OP_RAMP) tile_ramp(s, t.arg, tile, sm);
     else if constexpr (OP == OP_BWD) tile_bwd(s, t.arg, tile, sm);
-    else if constexpr (OP == OP_BWD_FIN) tile_bwd_fin<FIN_IMAGES>(s, t.arg, tile);
+    else if constexpr (OP == OP_BWD_FIN) tile_bwd_fin<FIN_IMAGES, true>(s, t.arg, tile);
     else if constexpr (OP == OP_CG_A) tile_cg_a(s, t.arg, tile);
     else if constexpr (OP == OP_CG_B) tile_cg_b(s, tile);
     else if constexpr (OP == OP_ZERO) tile_zero(s, tile);

@@ -3,6 +3,8 @@
 // air_internal.cuh for the launch forms that share them.
 #pragma once
 
+#include <cfloat>
+
 #include "air_internal.cuh"
 #include "tiles_orbit.cuh"
 
@@ -352,6 +354,13 @@ __device__ __forceinline__ void tile_bwd(const SliceDesc &s, int mode, int tile,
 }
 
 
+// a + b = s + the rounding error it returns (Knuth's two-sum).
+__device__ __forceinline__ float two_sum(float a, float b, float &s) {
+    s = __fadd_rn(a, b);
+    const float t = __fsub_rn(s, a);
+    return __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
+}
+
 // Sums the parts of the backprojection (bwd_images of them) in a fixed order
 // and applies the mode's epilogue (the CG and residual updates of the Eq. 5
 // system).  Bound by the latency of the images' loads: a thread takes N = 4
@@ -363,38 +372,69 @@ __device__ __forceinline__ void tile_bwd(const SliceDesc &s, int mode, int tile,
 // 24 images at a time cost registers and gained nothing.  The general path's
 // rhs0 stays pixel by pixel: its split, and with it the order of its sums, is
 // tuned on this sum's time there.  The persistent kernel's one register budget
-// has no room for U images (U = 1).
-template <int N, int U>
+// has no room for U images (U = 1).  ORB: the slice may run the orbit pair.
+template <int N, int U, bool ORB>
 __device__ __forceinline__ double bwd_fin(const SliceDesc &s, int mode, bool swap, int stop, int i) {
     struct __align__(4 * N) Vec { float v[N]; };
     auto get = [&](const float *a) { return *reinterpret_cast<const Vec *>(a + i); };
     auto put = [&](float *a, const Vec &x) { *reinterpret_cast<Vec *>(a + i) = x; };
     const int S = bwd_images(s);
     const size_t nn = (size_t)s.n * s.n;
+    const bool orb = ORB && s.orb;
     Vec a{};
+    auto add = [&](const Vec &x) {
+#pragma unroll
+        for (int q = 0; q < N; ++q) a.v[q] += x.v[q];
+    };
+    // the orbits' images, a multiple of eight: fours by pairs, and the fours
+    // with their rounding errors, so that the sum takes 1.75 roundings of its
+    // own size with the scale and not eight or more
+    Vec err{};
+    auto add_orbits = [&](Vec(&x)[8], bool first) {
+#pragma unroll
+        for (int q = 0; q < N; ++q) {
+            float h;
+            const float e = two_sum((x[0].v[q] + x[1].v[q]) + (x[2].v[q] + x[3].v[q]),
+                                    (x[4].v[q] + x[5].v[q]) + (x[6].v[q] + x[7].v[q]), h);
+            if (first) {
+                a.v[q] = h;
+                err.v[q] = e;
+            } else {
+                err.v[q] += e + two_sum(a.v[q], h, a.v[q]);
+            }
+        }
+    };
     if constexpr (U > 1) {
+        static_assert(U == 8, "as many as the orbits have images");
 #pragma unroll 1
         for (int p = 0; p < S; p += U) {
             Vec x[U];
 #pragma unroll
             for (int u = 0; u < U; ++u)
                 if (p + u < S) x[u] = get(s.bwd_part + (p + u) * nn);
+            if (orb) {
+                add_orbits(x, p == 0);
+            } else {
 #pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (p + u < S)
+                for (int u = 0; u < U; ++u)
+                    if (p + u < S) add(x[u]);
+            }
+        }
+    } else if (orb) {
+#pragma unroll 1
+        for (int p = 0; p < S; p += 8) {
+            Vec x[8];
 #pragma unroll
-                    for (int q = 0; q < N; ++q) a.v[q] += x[u].v[q];
+            for (int u = 0; u < 8; ++u) x[u] = get(s.bwd_part + (p + u) * nn);
+            add_orbits(x, p == 0);
         }
     } else {
 #pragma unroll (N == 4 ? 8 : 4)
-        for (int p = 0; p < S; ++p) {
-            const Vec x = get(s.bwd_part + p * nn);
-#pragma unroll
-            for (int q = 0; q < N; ++q) a.v[q] += x.v[q];
-        }
+        for (int p = 0; p < S; ++p) add(get(s.bwd_part + p * nn));
     }
 #pragma unroll
-    for (int q = 0; q < N; ++q) a.v[q] *= s.dx;
+    for (int q = 0; q < N; ++q)        // (an infinite sum has no error to add)
+        a.v[q] = orb && fabsf(a.v[q]) <= FLT_MAX ? fmaf(s.dx, a.v[q], s.dx * err.v[q]) : s.dx * a.v[q];
     double part = 0.0;
     if (mode == BWD_PLAIN) {
         put(s.ext_out, a);
@@ -420,7 +460,7 @@ __device__ __forceinline__ double bwd_fin(const SliceDesc &s, int mode, bool swa
 }
 
 constexpr int FIN_IMAGES = 8;
-template <int U>
+template <int U, bool ORB>
 __device__ __forceinline__ void tile_bwd_fin(const SliceDesc &s, int arg, int tile) {
     __shared__ double sh[AIR_THREADS / 32];
     const int mode = arg & ARG_MASK;
@@ -430,12 +470,12 @@ __device__ __forceinline__ void tile_bwd_fin(const SliceDesc &s, int arg, int ti
     double part = 0.0;
     if ((s.orb || mode != BWD_RHS0) && nn % 4 == 0) {
         const int i = base + 4 * (int)threadIdx.x;
-        if (i < nn) part = bwd_fin<4, U>(s, mode, swap, stop, i);
+        if (i < nn) part = bwd_fin<4, U, ORB>(s, mode, swap, stop, i);
     } else {
 #pragma unroll
         for (int k = 0; k < 4; ++k) {
             const int i = base + k * AIR_THREADS + (int)threadIdx.x;
-            if (i < nn) part += bwd_fin<1, 1>(s, mode, swap, stop, i);
+            if (i < nn) part += bwd_fin<1, 1, ORB>(s, mode, swap, stop, i);
         }
     }
     if (stop || mode == BWD_PLAIN || mode == BWD_RHS0 || mode == BWD_STEP) return;
@@ -800,13 +840,6 @@ struct ShrinkArgs {
     float tau;
 };
 
-// a + b = s + the rounding error it returns (Knuth's two-sum).
-__device__ __forceinline__ float two_sum(float a, float b, float &s) {
-    s = __fadd_rn(a, b);
-    const float t = __fsub_rn(s, a);
-    return __fadd_rn(__fsub_rn(a, __fsub_rn(s, t)), __fsub_rn(b, t));
-}
-
 // A sum of squares kept in three floats (hi + mid + lo), more bits than FP64
 // has: the squares of differences x - y enter without a rounding error above
 // 2^-69 of the sum (two-sums, and an FMA for a product's error).
@@ -1069,7 +1102,7 @@ __device__ __forceinline__ void run_tile(const SliceDesc &s, int op, int arg, in
     case OP_TRANSPOSE: tile_transpose(s, arg, tile, sm); break;
     case OP_RAMP: tile_ramp(s, arg, tile, sm); break;
     case OP_BWD: tile_bwd(s, arg, tile, sm); break;
-    case OP_BWD_FIN: tile_bwd_fin<1>(s, arg, tile); break;
+    case OP_BWD_FIN: tile_bwd_fin<1, ORB>(s, arg, tile); break;
     case OP_CG_A: tile_cg_a(s, arg, tile); break;
     case OP_CG_B: tile_cg_b(s, tile); break;
     case OP_ZERO: tile_zero(s, tile); break;

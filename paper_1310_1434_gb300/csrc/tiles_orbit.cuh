@@ -271,9 +271,19 @@ __device__ __forceinline__ void tile_orb_fwd(const SliceDesc &s, int arg, int ti
 // side, times the ray's c.  A segment's rays past the tile's last one, which
 // no pixel of the tile meets, are staged as well: the candidates may run
 // onto them.  The sums of each frame go to an image of their own, which
-// OP_BWD_FIN adds in a fixed order.  At 512^2 / 800 views the kernel, cold, takes
-// 86 us, a call with packing and sum 89 (general: 239): 64 M instead of 207
-// M warp instructions and 18 M instead of 55 M shared-memory wavefronts.
+// OP_BWD_FIN adds in a fixed order.
+// A sum of FP32 values that grows over all the views loses more by each
+// addition the larger it gets: the accumulators are put aside every few rounds
+// (`fold`) and start again from zero, about ORB_SUMS partial sums to a pixel
+// and frame over all splits.  They lie in shared memory, where they take the
+// place of a third stage of the ring, which brought nothing.  With the images
+// summed as in bwd_fin the error of A^T against FP64, relative to the image, is
+// 3.4e-8 at 512^2 / 800 views (one accumulator and a running sum 9.3e-8, the
+// general pair 6.0e-8), 3.5e-8 at 350^2 / 200 (6.6e-8, 5.1e-8), 4.6e-8 at
+// 1024^2 / 800 (9.0e-8, 5.6e-8).
+// At 512^2 / 800 views a call with packing and sum takes 87 us (89 with one
+// accumulator and three stages; general: 239): 64 M instead of 207 M warp
+// instructions and 18 M instead of 55 M shared-memory wavefronts.
 // Bound: instruction issue (67 % active) and the shared-memory data path (68 %).
 // ======================================================================
 // Weights of the rows 0 and 1 of a span that starts in row d: f0 belongs to row
@@ -288,8 +298,10 @@ __device__ __forceinline__ void orb_rows(int d, float f0, float f1, float &lo, f
 }
 
 constexpr int ORB_SEGS = 4;                              // segments staged at a time
-constexpr int ORB_STAGES = 3;
+constexpr int ORB_STAGES = 2;
 constexpr int ORB_ROWS = 4;                              // pixels of a thread, along r
+constexpr int ORB_SUMS = 8;                              // partial sums a pixel and frame is made of, or a round each,
+constexpr int ORB_FOLD_MAX = 8;                          // of at most eight rounds
 constexpr int ORB_EARLY = 152;                           // blocks of a launch that leaves SMs idle: one per SM
 constexpr int ORB_ENT = ORB_RAYS + ORB_CAND;             // staged rays of a segment
 
@@ -297,7 +309,7 @@ constexpr int ORB_PATCH_K = 8, ORB_PATCH_R = 16;         // pixels of a warp
 constexpr int ORB_PAR = 2 * AIR_THREADS / 32;            // float4s of a staged segment's parameters, two per warp
 
 __host__ __device__ inline size_t orb_bwd_smem(int nf) {
-    return (size_t)ORB_STAGES * ORB_SEGS * (ORB_ENT * (1 + nf / 4) + ORB_PAR) * 16;
+    return ((size_t)ORB_STAGES * ORB_SEGS * (ORB_ENT * (1 + nf / 4) + ORB_PAR) + (size_t)AIR_THREADS * nf) * 16;
 }
 
 __device__ __forceinline__ void cp_async16(void *dst, const void *src) {
@@ -358,10 +370,11 @@ __device__ __forceinline__ void tile_orb_bwd_nf(const SliceDesc &s, int mode, in
     const int ne = e1 - e0 > split ? (e1 - e0 - split + S - 1) / S : 0;      // this split's entries
     const uint2 *__restrict__ ent = s.orb_ent + e0 + split;                  // every S-th
     float4 *buf = reinterpret_cast<float4 *>(sm);
+    ulonglong2 *aside = reinterpret_cast<ulonglong2 *>(buf + ORB_STAGES * ORB_SEGS * SEG) + threadIdx.x;   // [NF][AIR_THREADS]
 
     // warps 2 q and 2 q + 1 stage the round's segment q; warp `round` mod 8
     // writes every warp's parameters of the four segments.  The rays and the
-    // parameters come from the plan's tables: those of the first two rounds
+    // parameters come from the plan's tables: those of the first round
     // are asked for before the wait for the last kernel where a launch leaves
     // SMs idle (128^2 / 90 views: 734 -> 703 us for 20 CG steps; a launch of
     // more than a block per SM lost half a percent by it).
@@ -408,23 +421,36 @@ __device__ __forceinline__ void tile_orb_bwd_nf(const SliceDesc &s, int mode, in
         for (int f = 0; f < NF / 2; ++f) acc[q][f] = 0ull;
 
     const bool early = gridDim.x <= ORB_EARLY;
-    if (early) {
-        stage(0, true, false);
-        stage(1, true, false);
-    }
+    if (early) stage(0, true, false);
     grid_wait();
-    const int stop = mode == BWD_Q ? s.cg->stop : 0;     // on its way with the first rounds
+    const int stop = mode == BWD_Q ? s.cg->stop : 0;     // on its way with the first round
     stage(0, !early, true);
-    stage(1, !early, true);
     // the thread's column and first row from the middle of its warp's pixels
     const float u = (float)(lane & 7) - 0.5f * (ORB_PATCH_K - 1);
     const float v0 = (float)((lane >> 3) * ORB_ROWS) - 0.5f * (ORB_PATCH_R - 1);
     const int rounds = stop ? 0 : (ne + ORB_SEGS - 1) / ORB_SEGS;
+    // rounds that are summed by themselves: see above
+    const int fold = min(ORB_FOLD_MAX, max(1, (rounds * S + ORB_SUMS - 1) / ORB_SUMS));
+    int due = fold;
 #pragma unroll 1
     for (int round = 0; round < rounds; ++round) {
-        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
         __syncthreads();             // this round's rays are there; the last round's buffer is free
-        stage(round + 2, true, true);
+        stage(round + 1, true, true);
+        if (round == due) {
+#pragma unroll
+            for (int i = 0; i < NF; ++i) {
+                unsigned long long *a = &acc[0][0] + 2 * i;
+                ulonglong2 t = make_ulonglong2(a[0], a[1]);
+                if (round > fold) {
+                    const ulonglong2 f = aside[i * AIR_THREADS];
+                    t = make_ulonglong2(add2(f.x, t.x), add2(f.y, t.y));
+                }
+                aside[i * AIR_THREADS] = t;
+                a[0] = a[1] = 0ull;
+            }
+            due += fold;
+        }
         const int m = min(ORB_SEGS, ne - round * ORB_SEGS);
 #pragma unroll 1
         for (int q = 0; q < m; ++q) {
@@ -465,6 +491,15 @@ __device__ __forceinline__ void tile_orb_bwd_nf(const SliceDesc &s, int mode, in
                     }
                 }
             }
+        }
+    }
+    if (rounds > fold) {
+#pragma unroll
+        for (int i = 0; i < NF; ++i) {
+            const ulonglong2 f = aside[i * AIR_THREADS];
+            unsigned long long *a = &acc[0][0] + 2 * i;
+            a[0] = add2(f.x, a[0]);
+            a[1] = add2(f.y, a[1]);
         }
     }
     if (k < n && !stop) {
