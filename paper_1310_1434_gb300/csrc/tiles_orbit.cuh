@@ -489,66 +489,67 @@ __device__ __forceinline__ void tile_orb_bwd_nf(const SliceDesc &s, int mode, in
     const int rounds = stop ? 0 : (ne + ORB_SEGS - 1) / ORB_SEGS;
     // rounds that are summed by themselves: see above
     const int fold = min(ORB_FOLD_MAX, max(2, (rounds * S + ORB_SUMS - 1) / ORB_SUMS));
-    int due = fold;
 #pragma unroll 1
-    for (int round = 0; round < rounds; ++round) {
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        __syncthreads();             // this round's rays are there; the last round's buffer is free
-        stage(round + 1, true, true);
-        if (round == due) {
-#pragma unroll
-            for (int i = 0; i < NF; ++i) {
-                unsigned long long *a = &acc[0][0] + 2 * i;
-                ulonglong2 t = make_ulonglong2(a[0], a[1]);
-                if (round > fold) {
-                    const ulonglong2 f = aside[i * AIR_THREADS];
-                    t = make_ulonglong2(add2(f.x, t.x), add2(f.y, t.y));
-                }
-                aside[i * AIR_THREADS] = t;
-                a[0] = a[1] = 0ull;
-            }
-            due += fold;
-        }
-        const int m = min(ORB_SEGS, ne - round * ORB_SEGS);
+    for (int round = 0; round < rounds;) {
+        const int from = round, to = min(round + fold, rounds);
 #pragma unroll 1
-        for (int q = 0; q < m; ++q) {
-            const float4 *st = buf + ((round % ORB_STAGES) * ORB_SEGS + q) * SEG;
-            const float4 ia = st[SEG - ORB_PAR + 2 * warp], ib = st[SEG - ORB_PAR + 2 * warp + 1];
-            const int nc = __float_as_int(ib.y), cnt = __float_as_int(ib.z);
-            const float4 *at[ORB_ROWS / 2];
-#pragma unroll
-            for (int y = 0; y < ORB_ROWS / 2; ++y) {
-                const float v = v0 + (float)(2 * y);
-                const int i = __float2int_ru(fmaf(ib.x, u * v, fmaf(ia.w, 0.5f * (u * u - v * v),
-                                                                    fmaf(ia.z, v, fmaf(ia.y, u, ia.x)))));
-                at[y] = st + min(max(i, 0), cnt);
-            }
+        for (; round < to; ++round) {
+            asm volatile("cp.async.wait_group 0;" ::: "memory");
+            __syncthreads();             // this round's rays are there; the last round's buffer is free
+            stage(round + 1, true, true);
+            const int m = min(ORB_SEGS, ne - round * ORB_SEGS);
 #pragma unroll 1
-            for (int c = 0; c < nc; ++c) {
+            for (int q = 0; q < m; ++q) {
+                const float4 *st = buf + ((round % ORB_STAGES) * ORB_SEGS + q) * SEG;
+                const float4 ia = st[SEG - ORB_PAR + 2 * warp], ib = st[SEG - ORB_PAR + 2 * warp + 1];
+                const int nc = __float_as_int(ib.y), cnt = __float_as_int(ib.z);
+                const float4 *at[ORB_ROWS / 2];
 #pragma unroll
                 for (int y = 0; y < ORB_ROWS / 2; ++y) {
-                    const float4 ray = at[y][c];
-                    const unsigned Ma = __float_as_uint(ray.z);
-                    const unsigned long long p =
-                        (unsigned long long)(unsigned)k * Ma +
-                        (((unsigned long long)__float_as_uint(ray.y) << 32) | __float_as_uint(ray.x));
-                    unsigned ov0, ov1;
-                    orb_overlap(~(unsigned)p, Ma, ov0, ov1);
-                    const int d = (int)(p >> 32) - (r + 2 * y);
-                    const float f0 = __uint2float_rn(ov0), f1 = __uint2float_rn(ov1);
-                    float lo, hi;
-                    orb_rows(d, f0, f1, lo, hi);
-                    const unsigned long long w0 = pair2(lo, lo), w1 = pair2(hi, hi);
+                    const float v = v0 + (float)(2 * y);
+                    const int i = __float2int_ru(fmaf(ib.x, u * v, fmaf(ia.w, 0.5f * (u * u - v * v),
+                                                                        fmaf(ia.z, v, fmaf(ia.y, u, ia.x)))));
+                    at[y] = st + min(max(i, 0), cnt);
+                }
+#pragma unroll 1
+                for (int c = 0; c < nc; ++c) {
 #pragma unroll
-                    for (int v = 0; v < NV; ++v) {
-                        const ulonglong2 z = *reinterpret_cast<const ulonglong2 *>(at[y] + ORB_ENT * (1 + v) + c);
-                        acc[2 * y][2 * v] = fma2(w0, z.x, acc[2 * y][2 * v]);
-                        acc[2 * y][2 * v + 1] = fma2(w0, z.y, acc[2 * y][2 * v + 1]);
-                        acc[2 * y + 1][2 * v] = fma2(w1, z.x, acc[2 * y + 1][2 * v]);
-                        acc[2 * y + 1][2 * v + 1] = fma2(w1, z.y, acc[2 * y + 1][2 * v + 1]);
+                    for (int y = 0; y < ORB_ROWS / 2; ++y) {
+                        const float4 ray = at[y][c];
+                        const unsigned Ma = __float_as_uint(ray.z);
+                        const unsigned long long p =
+                            (unsigned long long)(unsigned)k * Ma +
+                            (((unsigned long long)__float_as_uint(ray.y) << 32) | __float_as_uint(ray.x));
+                        unsigned ov0, ov1;
+                        orb_overlap(~(unsigned)p, Ma, ov0, ov1);
+                        const int d = (int)(p >> 32) - (r + 2 * y);
+                        const float f0 = __uint2float_rn(ov0), f1 = __uint2float_rn(ov1);
+                        float lo, hi;
+                        orb_rows(d, f0, f1, lo, hi);
+                        const unsigned long long w0 = pair2(lo, lo), w1 = pair2(hi, hi);
+#pragma unroll
+                        for (int v = 0; v < NV; ++v) {
+                            const ulonglong2 z = *reinterpret_cast<const ulonglong2 *>(at[y] + ORB_ENT * (1 + v) + c);
+                            acc[2 * y][2 * v] = fma2(w0, z.x, acc[2 * y][2 * v]);
+                            acc[2 * y][2 * v + 1] = fma2(w0, z.y, acc[2 * y][2 * v + 1]);
+                            acc[2 * y + 1][2 * v] = fma2(w1, z.x, acc[2 * y + 1][2 * v]);
+                            acc[2 * y + 1][2 * v + 1] = fma2(w1, z.y, acc[2 * y + 1][2 * v + 1]);
+                        }
                     }
                 }
             }
+        }
+        if (to == rounds) break;
+#pragma unroll
+        for (int i = 0; i < NF; ++i) {
+            unsigned long long *a = &acc[0][0] + 2 * i;
+            ulonglong2 t = make_ulonglong2(a[0], a[1]);
+            if (from) {
+                const ulonglong2 f = aside[i * AIR_THREADS];
+                t = make_ulonglong2(add2(f.x, t.x), add2(f.y, t.y));
+            }
+            aside[i * AIR_THREADS] = t;
+            a[0] = a[1] = 0ull;
         }
     }
     if (rounds > fold) {
@@ -560,13 +561,7 @@ __device__ __forceinline__ void tile_orb_bwd_nf(const SliceDesc &s, int mode, in
             a[1] = add2(f.y, a[1]);
         }
     }
-    unsigned long long zero = 0ull;                      // or NaN, with any sum that is not finite
-#pragma unroll
-    for (int i = 0; i < 2 * NF; ++i) zero = fma2((&acc[0][0])[i], 0ull, zero);
-    const float2 finite = unpair2(zero);
-    if (!(finite.x + finite.y == 0.f)) {
-        orb_bwd_hits<NF>(s, cls, split, txy, k, r);
-    } else if (k < n && !stop) {
+    if (k < n && !stop) {
 #pragma unroll
         for (int f = 0; f < NF; ++f) {
             float *img = s.bwd_part + (size_t)(split * 8 + cls * 4 + f) * n * n;
@@ -581,6 +576,11 @@ __device__ __forceinline__ void tile_orb_bwd_nf(const SliceDesc &s, int mode, in
             }
         }
     }
+    unsigned long long zero = 0ull;                      // or NaN, with any sum that is not finite (which is stored again)
+#pragma unroll
+    for (int i = 0; i < 2 * NF; ++i) zero = fma2((&acc[0][0])[i], 0ull, zero);
+    const float2 finite = unpair2(zero);
+    if (!(finite.x + finite.y == 0.f)) orb_bwd_hits<NF>(s, cls, split, txy, k, r);
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();   // shared memory is reused by the next tile of a persistent block
 }
