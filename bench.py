@@ -807,12 +807,12 @@ SEG_INST = 8
 # DRAM bytes (read + write) of one backprojector launch on the 512^2 / 800-view
 # slice, from the committed ncu capture of the current kernel (None when the
 # kernel has changed since).
-BWD_DRAM_BYTES_512_V800 = 3_595_520
+BWD_DRAM_BYTES_512_V800 = 3_609_856
 # L1 data-pipe wavefronts of one launch of each operator on the 512^2 /
 # 800-view slice (l1tex__data_pipe_lsu_wavefronts.sum) from the committed ncu
 # captures of the current kernels (OP_ORB_BWD at four splits, OP_ORB_FWD): the
 # backprojector's reads of staged rays and samples, the projector's gathers.
-BWD_L1_WAVEFRONTS_512_V800 = 18_299_717
+BWD_L1_WAVEFRONTS_512_V800 = 18_878_081
 FWD_L1_WAVEFRONTS_512_V800 = 18_445_397
 
 

@@ -101,8 +101,16 @@ AIR_API air_status air_plan_destroy(air_plan *plan);
  * Full scans whose views are taken into one another by at least four of the
  * eight symmetries of the pixel grid (n_views even and beta0 a multiple of
  * half the view pitch, or n_views a multiple of 4; n >= 64) run the projector
- * pair over orbits of symmetric rays: their projector has one tile shape, and
- * bwd_view_parts counts images, eight for each split of the backprojector. */
+ * pair over orbits of symmetric rays, unless
+ *   - one of their rays runs along a line of the pixel grid (with an even n, an
+ *     odd n_bins and beta0 = 0 the middle ray of the first view always does),
+ *   - the fan is wide, the source close or the rays much denser than the pixels
+ *     (more than 96 rays of a view in 32 x 32 pixels), or
+ *   - the device has no memory for the orbits beside the rest of the plan.
+ * The projector of such a plan has one tile shape, and its bwd_view_parts
+ * counts images, eight for each split of the backprojector; air_plan_tune sets
+ * those and leaves the view split of the general pair, which air_solve runs
+ * when it returns a history, as it was tuned. */
 AIR_API air_status air_plan_tune(air_plan *plan, int fwd_views_per_block, int bwd_view_parts);
 AIR_API air_status air_plan_config(const air_plan *plan, int *fwd_views_per_block, int *bwd_view_parts,
                                    int *bwd_view_parts_max);
@@ -186,7 +194,7 @@ AIR_API air_status air_framelet(const air_plan *plan, const float *in, float *ou
  *   t = W X + b;  d = soft(t, thresh) on bands 1..8, d = t on band 0;
  *   b <- t - d (in place);  g = W^T (d - b_new).
  * X: n*n, b: 9*n*n (in/out), g: n*n (out).  resid: device double, may be
- * NULL; receives ||W X - d||_2 accumulated in FP64.  thresh >= 0. */
+ * NULL; receives ||W X - d||_2 accumulated to FP64's precision.  thresh >= 0. */
 AIR_API air_status air_shrink(const air_plan *plan, const float *X, float *b, float *g, float thresh,
                       double *resid, air_stream stream);
 
@@ -196,8 +204,9 @@ AIR_API air_status air_shrink(const air_plan *plan, const float *X, float *b, fl
  *   the d/b update with threshold lambda/mu.
  * Y: n_views*n_bins (input), X: n*n (output only).  resid: device, n_outer
  * doubles, may be NULL: ||W X - d||_2 after each outer step.  lambda >= 0,
- * mu > 0, n_outer >= 0, n_cg >= 0.  CG dot products and the residual norms
- * are accumulated in FP64 on the device; no host synchronisation inside.
+ * mu > 0, n_outer >= 0, n_cg >= 0.  CG dot products are accumulated in FP64 on
+ * the device, the residual norms to its precision; no host synchronisation
+ * inside.
  * With resid the solve runs the general projector pair whatever the scan's
  * symmetries (see air_plan_tune), so that the history keeps one summation
  * order; X then differs from a call without resid by rounding. */
@@ -288,10 +297,12 @@ AIR_API air_status air_solve_batch_persistent(int n, air_plan *const *plans, con
  * device bytes of all resident requests stay within hbm_budget_bytes; a
  * request that arrives while others are running joins the running set at
  * the next step boundary, and all resident requests advance together, one
- * operator phase per device step.  max_slots bounds the resident set. */
+ * operator phase per device step.  max_slots bounds the resident set.  A request
+ * whose plan does not fit the budget with orbits (see air_plan_tune) is served
+ * without them. */
 AIR_API air_status air_server_create(size_t hbm_budget_bytes, int max_slots, air_server **out);
 /* Queues one request; copies Y_host (n_views*n_bins floats) before returning.
- * AIR_ERR_BUDGET if the request alone exceeds the budget. */
+ * AIR_ERR_BUDGET if the request alone exceeds the budget, also without orbits. */
 AIR_API air_status air_server_submit(air_server *srv, const air_geometry *geom, const float *Y_host,
                              float lambda, float mu, int n_outer, int n_cg,
                              uint64_t *request_id);

@@ -40,7 +40,8 @@ constexpr int TC_SIDE = 8;
 // call of a batch times the one-chain and the two-chain graph and keeps the
 // faster; later batches of the same shapes take the same form.  A batch whose
 // backprojector phase takes more than CHAIN_WAVES waves of the device is not
-// tried in two chains.
+// tried in two chains (measured on the general pair; the orbit pair's waves
+// are counted alike).
 constexpr int CHAINS = 2;
 constexpr double CHAIN_WAVES = 64.0;
 // Graphs kept for the compositions used last, and chain choices for the

@@ -877,8 +877,8 @@ struct SumSq {
 // there in FP64: GB300 issues one FP64 instruction for 64 FP32 ones, and four
 // for each of the nine coefficients bound the form that did (FP64 pipe 67 %
 // active).  The coefficient tile is 32 x 8, one row for each warp.
-// At 512^2 a stand-alone call, which copies b back, takes 25 us: 44 with FP64
-// squares and 16 x 16 tiles, 34 with FP64 squares in these tiles, 24 with two
+// At 512^2 a stand-alone call, which copies b back, takes 26 us: 44 with FP64
+// squares and 16 x 16 tiles, 35 with FP64 squares in these tiles, 25 with two
 // floats, which lose up to 2e-14 of nine squares where FP64 loses 3e-16 and
 // three floats 1e-16; 62 us at 1024^2 (130, 99, 54).  The chain of loads,
 // barriers and the reduction of each short block bounds it.  Walking each warp

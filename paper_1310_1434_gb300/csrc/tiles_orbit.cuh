@@ -282,9 +282,9 @@ __device__ __forceinline__ void tile_orb_fwd(const SliceDesc &s, int arg, int ti
 // general pair 6.0e-8), 3.5e-8 at 350^2 / 200 (6.6e-8, 5.1e-8), 4.6e-8 at
 // 1024^2 / 800 (9.0e-8, 5.6e-8).
 // At 512^2 / 800 views a call with packing and sum takes 87 us (89 with one
-// accumulator and three stages; general: 239): 64 M instead of 207 M warp
-// instructions and 18 M instead of 55 M shared-memory wavefronts.
-// Bound: instruction issue (67 % active) and the shared-memory data path (68 %).
+// accumulator and three stages; general: 239): 55 M instead of 207 M warp
+// instructions and 19 M instead of 55 M shared-memory wavefronts.
+// Bound: the shared-memory data path (72 %) and instruction issue (63 % active).
 // ======================================================================
 // Weights of the rows 0 and 1 of a span that starts in row d: f0 belongs to row
 // d and f1 to row d + 1.  In PTX because the compiler made branches of it.
