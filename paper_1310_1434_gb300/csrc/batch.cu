@@ -316,7 +316,8 @@ extern "C" air_status air_solve_batch(int n, air_plan *const *plans, const float
     std::lock_guard<std::mutex> lock(g_batch_mu);
     cudaError_t e = cudaSuccess;
     const size_t b_slices = align_up(n * sizeof(SliceDesc), 256);
-    // this call's descriptors, ahead of the graph on the caller's stream
+    // this call's descriptors (and a new graph's task lists), ahead of the graph on
+    // the caller's stream: a copy from pageable memory may end after its call
     auto describe = [&](BatchGraph &G) {
         return cudaMemcpyAsync(G.dmem, B.slices.data(), n * sizeof(SliceDesc), cudaMemcpyHostToDevice, st);
     };
@@ -363,7 +364,7 @@ extern "C" air_status air_solve_batch(int n, air_plan *const *plans, const float
     e = make_capture(C);
     if (e == cudaSuccess) e = describe(G);
     if (e == cudaSuccess && !tasks.empty())
-        e = cudaMemcpy(d_tasks, tasks.data(), tasks.size() * sizeof(Task), cudaMemcpyHostToDevice);
+        e = cudaMemcpyAsync(d_tasks, tasks.data(), tasks.size() * sizeof(Task), cudaMemcpyHostToDevice, st);
     if (e != cudaSuccess) {
         release(G);
         return fail(AIR_ERR_CUDA, std::string("batch set-up: ") + cudaGetErrorString(e));
@@ -519,13 +520,16 @@ extern "C" air_status air_solve_batch_persistent(int n, air_plan *const *plans, 
         int *d_tb = (int *)(G.dmem + b_slices + b_prog);
         unsigned long long *d_pb = (unsigned long long *)(G.dmem + b_slices + b_prog + b_tb);
         G.ctl = (BatchCtl *)(G.dmem + b_slices + b_prog + b_tb + b_pb);
-        cudaError_t e = cudaMemcpy(d_slices, B.slices.data(), n * sizeof(SliceDesc), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess) e = cudaMemcpy(d_prog, prog.data(), prog.size() * sizeof(Phase), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess)
-            e = cudaMemcpy(d_tb, tile_base.data(), tile_base.size() * sizeof(int), cudaMemcpyHostToDevice);
-        if (e == cudaSuccess)
-            e = cudaMemcpy(d_pb, phase_base.data(), phase_base.size() * sizeof(unsigned long long),
-                           cudaMemcpyHostToDevice);
+        // on the stream the graph runs on: a copy from pageable memory may end
+        // after the call that asks for it
+        cudaError_t e = cudaSuccess;
+        auto put = [&](void *d, const auto &v, size_t count) {
+            if (e == cudaSuccess) e = cudaMemcpyAsync(d, v.data(), count * sizeof(v[0]), cudaMemcpyHostToDevice, st);
+        };
+        put(d_slices, B.slices, n);
+        put(d_prog, prog, prog.size());
+        put(d_tb, tile_base, tile_base.size());
+        put(d_pb, phase_base, phase_base.size());
         if (e == cudaSuccess) e = make_capture(C);
         if (e == cudaSuccess) e = cudaStreamBeginCapture(C.cap, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) {
